@@ -2,6 +2,7 @@
 // polynomial tables read by the forward kernels (widely-linear form, see
 // dpd_internal.h) and by the adjoint input-gradient kernel (see dpd_adj.cuh).
 // Also the FP64 finalisation of the coefficient gradient.
+#include "dpd_device.cuh"
 #include "dpd_internal.h"
 
 namespace dpd {
@@ -33,31 +34,13 @@ __global__ void wl_table_kernel(const H *__restrict__ hin, int Bp, int Bq, int T
         tab[wl_index(B, k, m, 2)] = A.y + C.y;      // P2 = Im(A+C)
         tab[wl_index(B, k, m, 3)] = A.x - C.x;      // P3 = Re(A-C)
         if (adj) {
-            // Per tap: for each power m the quadruple {Q0, Q3, Q1, Q2} of the
-            // bracket conj(E) g + H conj(g) = {Q0 c + Q1 d, Q2 c + Q3 d}
-            // (g = c + j d), then for each m < B-1 the quadruple {S0, S3, S1, S2}
-            // of conj(G) g + F conj(g): the pairs {Q0, Q3}, {Q1, Q2} multiply
-            // {c, d} and {d, c} in packed f32x2 FMAs.
-            const int per_tap = 4 * B + 4 * (B - 1);
-            float *q = adj + per_tap * k;
-            // E_m = (m+1) h_m, H_m = (m+1) hbar_m  (coefficients of r^m)
-            const float s = (float)(m + 1);
-            const float Er = s * A.x, Ei = s * A.y, Hr = s * C.x, Hi = s * C.y;
-            q[4 * m + 0] = Er + Hr;   // Q0
-            q[4 * m + 1] = Er - Hr;   // Q3
-            q[4 * m + 2] = Ei + Hi;   // Q1
-            q[4 * m + 3] = Hi - Ei;   // Q2
-            if (m < B - 1) {
-                // F_m = (m+1) h_{m+1}, G_m = (m+1) hbar_{m+1}
-                const float2 A1 = (m + 1 < Bp) ? h((m + 1) * T + k) : make_float2(0.f, 0.f);
-                const float2 C1 = (m + 1 < Bq) ? h((Bp + m + 1) * T + k) : make_float2(0.f, 0.f);
-                const float Fr = s * A1.x, Fi = s * A1.y, Gr = s * C1.x, Gi = s * C1.y;
-                float *r = q + 4 * B;
-                r[4 * m + 0] = Gr + Fr;   // S0
-                r[4 * m + 1] = Gr - Fr;   // S3
-                r[4 * m + 2] = Gi + Fi;   // S1
-                r[4 * m + 3] = Fi - Gi;   // S2
-            }
+            // {P0, P3} multiplies the gradient sample {c, d}, {P2, P1} its swap
+            // {d, c}: conj(h) g + hbar conj(g) = {P0 c + P2 d, P3 d + P1 c}.
+            float *q = adj + 4 * (k * B + m);
+            q[0] = A.x + C.x;
+            q[1] = A.x - C.x;
+            q[2] = A.y + C.y;
+            q[3] = C.y - A.y;
         }
     }
     if (i == 0) {
@@ -93,52 +76,53 @@ cudaError_t launch_wl_table_f64_many(const double2 *h, int count, int hstride, i
     return cudaGetLastError();
 }
 
-// One block per coefficient: thread t sums rows t, t + 256, ... in order, then a
-// fixed shared-memory tree combines the 256 sums (deterministic, FP64).
-// blockIdx.y selects a problem of a batch (its rows and outputs follow the
-// previous problem's).
-__global__ void adj_finalize_kernel(const float2 *__restrict__ partials, int rows, int K,
-                                    float2 *__restrict__ gh, double2 *__restrict__ gh64)
+// One warp per coefficient: lane t sums rows t, t + 32, ... in order (up to four
+// loads in flight), then a fixed shuffle tree combines the 32 sums
+// (deterministic, FP64).  blockIdx.y selects a problem of a batch (its rows and
+// outputs follow the previous problem's).
+constexpr int kFinalizeWarps = 8;
+
+__global__ void __launch_bounds__(32 * kFinalizeWarps)
+    adj_finalize_kernel(const float2 *__restrict__ partials, int rows, int K, float2 *__restrict__ gh,
+                        double2 *__restrict__ gh64)
 {
-    const int i = blockIdx.x, t = threadIdx.x;
+    grid_dep_wait();
+    const int i = blockIdx.x * kFinalizeWarps + (threadIdx.x >> 5), t = threadIdx.x & 31;
+    if (i >= K) return;
     partials += (size_t)blockIdx.y * rows * K;
-    if (gh) gh += (size_t)blockIdx.y * K;
-    if (gh64) gh64 += (size_t)blockIdx.y * K;
     double re = 0.0, im = 0.0;
-    for (int r = t; r < rows; r += 256) {
+#pragma unroll 4
+    for (int r = t; r < rows; r += 32) {
         const float2 v = partials[(size_t)r * K + i];
         re += v.x;
         im += v.y;
     }
-    __shared__ double sre[256], sim[256];
-    sre[t] = re;
-    sim[t] = im;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (t < w) {
-            sre[t] += sre[t + w];
-            sim[t] += sim[t + w];
-        }
-        __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
     }
     if (t == 0) {
-        if (gh) gh[i] = make_float2((float)sre[0], (float)sim[0]);
-        if (gh64) gh64[i] = make_double2(sre[0], sim[0]);
+        if (gh) gh[(size_t)blockIdx.y * K + i] = make_float2((float)re, (float)im);
+        if (gh64) gh64[(size_t)blockIdx.y * K + i] = make_double2(re, im);
     }
+}
+
+static cudaError_t finalize(const float2 *partials, int rows, int K, int count, float2 *gh, double2 *gh64,
+                            cudaStream_t s)
+{
+    const dim3 grid((unsigned)((K + kFinalizeWarps - 1) / kFinalizeWarps), (unsigned)count);
+    return launch_pdl(adj_finalize_kernel, grid, 32 * kFinalizeWarps, 0, s, partials, rows, K, gh, gh64);
 }
 
 cudaError_t launch_adj_finalize(const float2 *partials, int rows, int K, float2 *gh, cudaStream_t s)
 {
-    adj_finalize_kernel<<<K, 256, 0, s>>>(partials, rows, K, gh, nullptr);
-    count_launch();
-    return cudaGetLastError();
+    return finalize(partials, rows, K, 1, gh, nullptr, s);
 }
 
 cudaError_t launch_adj_finalize64(const float2 *partials, int rows, int K, double2 *out, cudaStream_t s)
 {
-    adj_finalize_kernel<<<K, 256, 0, s>>>(partials, rows, K, nullptr, out);
-    count_launch();
-    return cudaGetLastError();
+    return finalize(partials, rows, K, 1, nullptr, out, s);
 }
 
 // One partial row per problem (the batched refinement): the FP64 sum is the
@@ -162,9 +146,7 @@ cudaError_t launch_adj_finalize64_many(const float2 *partials, int rows, int K, 
         count_launch();
         return cudaGetLastError();
     }
-    adj_finalize_kernel<<<dim3((unsigned)K, (unsigned)count), 256, 0, s>>>(partials, rows, K, nullptr, out);
-    count_launch();
-    return cudaGetLastError();
+    return finalize(partials, rows, K, count, nullptr, out, s);
 }
 
 }  // namespace dpd

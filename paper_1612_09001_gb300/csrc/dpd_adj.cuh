@@ -2,19 +2,19 @@
 // with respect to the input samples and the coefficients, given gy = dL/dy,
 // all under the convention grad = dL/dRe + j dL/dIm.
 //
-// With r = |x|^2, branch polynomials A_k(r) = sum_b h_{2b+1,k} r^b and
-// C_k(r) = sum_b hbar_{2b+1,k} r^b (so that y_n = sum_k A_k(r_{n-k}) x_{n-k}
-// + C_k(r_{n-k}) conj(x_{n-k}) + c, Eq. 1), the Wirtinger derivatives of the
-// term of tap k are
-//   dy/dx       = E_k(r) + G_k(r) conj(x)^2,   E = A + r A',  G = C'
-//   dy/dconj(x) = F_k(r) x^2 + H_k(r),         F = A',        H = C + r C'
-// and
-//   gx_i = sum_k conj(dy_{i+k}/dx_i) gy_{i+k} + (dy_{i+k}/dconj(x_i)) conj(gy_{i+k})
-//        = sum_k [conj(E_k) g + H_k conj(g)] + x_i^2 [conj(G_k) g + F_k conj(g)],  g = gy_{i+k}
-// Each bracket is widely linear in g, so it is evaluated like the forward
-// filter: four real Horner polynomials per bracket, run as two packed f32x2
-// Horner chains whose results multiply the window sample {c, d} and its swap
-// {d, c} (table built by wl_table_kernel, one float4 per power).
+// With r = |x|^2 the filter is y_n = sum_{b,k} h_{b,k} r^b x + hbar_{b,k} r^b conj(x)
+// + c at samples n - k (Eq. 1, order 2b + 1).  Its adjoint first runs the taps
+// backwards over gy, one widely-linear FIR per power of r,
+//   F_b = sum_k conj(h_{b,k}) g_{i+k} + hbar_{b,k} conj(g_{i+k}),
+// and then takes the derivative of the features r^b x, r^b conj(x) at x_i:
+//   gx_i = V + 2 x_i Re(conj(x_i) V'),   V = sum_b r^b F_b,   V' = dV/dr.
+// V and V' come from one Horner pass over b (V' <- r V' + V, V <- r V + F_b), so
+// a sample costs 4 B T + 4 B fused multiply-adds.  The Wirtinger derivatives
+// evaluated tap by tap (four derivative polynomials of B and four of B - 1
+// coefficients per tap, 8 B - 4 per tap) cost 184 against 120 at B = T = 5.
+// Each FIR term is the 2 x 2 real matrix of the forward filter transposed, run
+// as two packed f32x2 FMAs on the window sample {c, d} and its swap {d, c}
+// (table built by wl_table_kernel, one float4 per tap and power).
 //
 // The coefficient gradient is the correlation
 //   gh_{(p,k)} = sum_j r_j^b conj(x_j) gy_{j+k},  gh_{(q,k)} = sum_j r_j^b x_j gy_{j+k},
@@ -26,12 +26,13 @@
 // adj_finalize_kernel.  The basis is recomputed from x: nothing from the
 // forward pass is stored.
 //
-// Data movement.  For 16-byte aligned x and gy both gradients run as persistent
-// kernels fed like the forward filter: one producer thread streams tiles of x
-// and of gy (plus kHalo samples of look-ahead) into a ring of shared-memory
-// slots with bulk copies completed on mbarriers, and the consumer warps read
-// their windows from shared memory.  Other alignments (and callers without an
-// error word) use the plain-load kernels, which read through L1.
+// Data movement.  For 16-byte aligned x and gy both gradients run as kernels
+// whose warps work on their own: every warp owns a contiguous share of the
+// record and a ring of shared-memory slots that its lane 0 fills with bulk
+// copies of x and gy (plus the look-ahead) completed on the warp's own
+// mbarriers, so no warp waits for another one until the final reduction.
+// Other alignments (and callers without an error word) use the plain-load
+// kernels, which read through L1.
 #pragma once
 
 #include "dpd_device.cuh"
@@ -39,18 +40,23 @@
 
 namespace dpd {
 
-constexpr int kAdjV = 4;          // samples per thread (plain-load kernels, staged gx)
-constexpr int kAdjGhV = 4;        // samples per thread of the staged gh kernel
-constexpr int kAdjWarps = 8;      // consumer warps of the staged gx kernel
-constexpr int kAdjGhWarps = 12;   // warps of the staged gh kernel (warp 0 also issues the copies)
-constexpr int kAdjStages = 4;     // ring slots of the staged gx kernel
-// Staged gh tile: 4 sub-blocks of V samples per thread (6144 samples), 2 ring
-// slots (197 KB).  Measured on GB300 (2^24 samples, us): 2 x 4 slots 84.8 /
-// 67.6 / 147.5, 3 x 3 83.9 / 62.7 / 142.8, 4 x 2 83.0 / 63.5 / 138.2 at
-// P = Q = 9, M = 4 / P = Q = 7, M = 3 / P = Q = 11, M = 7: a longer tile spreads
-// warp 0's wait for the slot release over more accumulation.
-constexpr int kAdjGhStages = 2;   // ring slots of the staged gh kernel
-constexpr int kAdjGhSub = 4;      // sub-blocks of V samples per thread and staged gh tile
+constexpr int kAdjV = 4;          // samples per thread and unit
+constexpr int kAdjUnit = 32 * kAdjV;   // samples of a warp's work unit
+constexpr int kAdjWarps = 8;      // warps per CTA of the staged gx kernel
+constexpr int kAdjStages = 2;     // ring slots per warp of the staged gx kernel
+constexpr int kAdjSub = 2;        // units per slot of the staged gx kernel
+constexpr int kAdjGhWarps = 12;   // warps per CTA of the staged gh kernel (about 165 registers per thread)
+constexpr int kAdjGhStages = 2;   // ring slots per warp of the staged gh kernel
+constexpr int kAdjGhSub = 3;      // units per slot of the staged gh kernel
+// Measured on GB300, graph-replayed, P = Q = 9, M = 4, us at 2^23 + 4097 / 2^20
+// samples.  gx (slots x units): 2 x 2 38.8 / 6.4, 2 x 4 39.9 / 6.4, 3 x 2 40.5 / 6.4;
+// two CTAs of 8 warps an SM 39.4, three (80 registers, spills) 49.3, five of 4 warps
+// 40.1.  At 38.8 us it moves 5.2 TB/s; P = Q = 7, M = 3 takes 31.5 us, 6.4 TB/s (96 %
+// of a copy).  The kernel with a producer warp per CTA and derivative polynomials
+// per tap took 51 us.
+// gh with its final sum: 2 x 3 38.9 / 10.7, 2 x 4 39.0 / 10.9, 4 x 2 40.4 / 10.9; 11
+// warps 44.4, 16 (128 registers, spills) 80.7.  24 T FMA/s at 2^23; the ring shared by
+// the CTA's warps, whose slots waited for the slowest warp, took 47.7.
 
 // NS consecutive complex samples p[base .. base+NS-1] (zero past n).  When the
 // buffer is 16-byte aligned, base is even and the rounded-up window lies inside
@@ -93,13 +99,18 @@ __device__ __forceinline__ void adj_slot_window(const float2 *slot, int off, flo
     }
 }
 
-// ---------------------------------------------------------------- staged tiles
-// A slot holds x[s0, s0 + S) and, from element S on, gy[s0, s0 + S + halo);
-// near the end of the signal only the even-length prefix that exists is copied.
-// The look-ahead `halo` (even) covers the furthest gy sample a consumer reads
-// for tile s0: kHalo for gx (T - 1 taps past its last sample, plus one for the
-// float4 rounding of the window), kAdjGhHalo for the tap-grouped gh kernels.
-__host__ __device__ constexpr int adj_slot_elems(int S, int halo = kHalo) { return 2 * S + halo; }
+// ---------------------------------------------------------------- warp rings
+// The record is cut into units of kAdjUnit samples and every warp of a launch
+// takes a contiguous run of them, equal to within one unit: warp w of W takes
+// units [first, first + count).  Consecutive w sit on different CTAs, so a short
+// record spreads over the SMs.  (A run of 2^31 units would be 2 TB of samples.)
+__device__ __forceinline__ int64_t warp_share(int64_t units, int w, int W, int &count)
+{
+    const int64_t q = units / W;
+    const int r = (int)(units - q * W);
+    count = (int)q + (w < r ? 1 : 0);
+    return w * q + (w < r ? w : r);
+}
 
 // The gh kernels read the window of taps k0 .. k0 + TG - 1 with k0 <= T - 1, so
 // their look-ahead reaches T + TG - 2 samples (+1 for the float4 rounding).
@@ -107,84 +118,147 @@ constexpr int kAdjGhMaxTG = 5;
 constexpr int kAdjGhHalo = kMaxT + kAdjGhMaxTG - 1;
 static_assert(kAdjGhHalo % 2 == 0 && kHalo % 2 == 0, "slot parts must stay 16-byte aligned");
 
-__device__ __forceinline__ void adj_slot_counts(int64_t s0, int S, int64_t n, int &xc, int &gc, int halo = kHalo)
-{
-    const int64_t rem = n - s0;
-    xc = (int)((rem < S ? rem : (int64_t)S) & ~int64_t(1));
-    gc = (int)((rem < S + halo ? rem : (int64_t)(S + halo)) & ~int64_t(1));
-}
-
-// NS samples of `src` from global index `g` whose slot copy starts at element
-// `base` of the slot and holds `cnt` samples from global index s0.
+// NS samples from element `off` of a tile whose slot holds the first `cnt` of
+// the `left` samples that the record has from the tile's start (src) on.
 template <int NS>
-__device__ __forceinline__ void adj_slot_window_tail(const float2 *slot_part, int64_t s0, int cnt,
-                                                     const float2 *__restrict__ src, int64_t g, int64_t n,
-                                                     float2 (&out)[NS])
+__device__ __forceinline__ void adj_slot_window_tail(const float2 *slot, int cnt, const float2 *__restrict__ src,
+                                                     int off, int64_t left, float2 (&out)[NS])
 {
 #pragma unroll
     for (int j = 0; j < NS; ++j) {
-        const int64_t gj = g + j;
+        const int g = off + j;
         float2 v = make_float2(0.f, 0.f);
-        if (gj - s0 < cnt)
-            v = slot_part[gj - s0];
-        else if (gj < n)
-            v = __ldg(src + gj);
+        if (g < cnt)
+            v = slot[g];
+        else if (g < left)
+            v = __ldg(src + g);
         out[j] = v;
     }
 }
 
-// The producer thread: stream every tile of this CTA into the ring.  Waits are
-// bounded; after a failed wait the copies already issued are allowed to land
-// before returning.
-__device__ __forceinline__ void adj_produce(const AdjArgs &a, float2 *ring, uint64_t *bars, int stages, int S,
-                                            int64_t ntiles, int halo = kHalo)
-{
-    const int slot_elems = adj_slot_elems(S, halo);
-    int64_t it = 0;
-    bool ok = true;
-    int s = 0;          // slot and parity of tile `it`, kept incrementally (no division per tile)
-    uint32_t ph = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-        if (it > 0 && ++s == stages) {
-            s = 0;
-            ph ^= 1u;
-        }
-        if (it >= stages && !mbar_wait(smem_addr(&bars[stages + s]), ph ^ 1u, a.status)) {
-            ok = false;
-            break;
-        }
-        if (it == 1 && !mbar_wait(smem_addr(&bars[0]), 0u, a.status)) {   // start-up: first tile first
-            ok = false;
-            break;
-        }
-        const int64_t s0 = tile * S;
-        int xc, gc;
-        adj_slot_counts(s0, S, a.n, xc, gc, halo);
-        const uint32_t fb = smem_addr(&bars[s]);
-        mbar_arrive_expect_tx(fb, (uint32_t)(xc + gc) * (uint32_t)sizeof(float2));
-        float2 *slot = ring + (size_t)s * slot_elems;
-        if (xc) bulk_copy_g2s(smem_addr(slot), a.x + s0, (uint32_t)xc * sizeof(float2), fb);
-        if (gc) bulk_copy_g2s(smem_addr(slot + S), a.gy + s0, (uint32_t)gc * sizeof(float2), fb);
-    }
-    if (!ok) {
-        const int64_t first = it > stages ? it - stages : 0;
-        for (int64_t j = first; j < it; ++j)
-            mbar_wait(smem_addr(&bars[j % stages]), (uint32_t)((j / stages) & 1), a.status);
-    }
-}
+// One warp's ring: STAGES slots of SUB units; a slot holds x[s0, s0 + S) and,
+// from element S on, gy[s0, s0 + S + HALO), S = SUB * kAdjUnit (less at the end
+// of the warp's share and of the record, where only the even-length prefix that
+// exists is copied).  Lane 0 issues the copies of tile i + STAGES once the whole
+// warp has read tile i (its windows are in registers): the warp is producer and
+// consumer, so the slot needs a "full" barrier only.
+template <int STAGES, int SUB, int HALO>
+struct AdjRing {
+    static constexpr int S = SUB * kAdjUnit;
+    static constexpr int kSlotElems = 2 * S + HALO;
+    static constexpr size_t kBytes = (size_t)STAGES * kSlotElems * sizeof(float2);   // per warp
 
-// Shared-memory bytes of a staged kernel: barriers, reduction scratch, ring.
-__host__ __device__ constexpr size_t adj_staged_smem(int S, int stages, int scratch_floats, int halo = kHalo)
+    const float2 *x, *gy;   // at the first sample of the warp's share
+    int64_t left;           // samples of the record from there on
+    float2 *slots;          // this warp's slots
+    uint32_t bars;          // shared-memory address of its STAGES barriers
+    int units;              // units in the share
+    int tiles;              // tiles of SUB units (the last may be shorter)
+    int whole;              // the first `whole` tiles lie, with their look-ahead, inside the record
+    int plain;              // the first `plain` of those have SUB units
+
+    // Share of warp w of W; returns its first sample.
+    __device__ __forceinline__ int64_t init(const AdjArgs &a, int64_t total_units, int w, int W, unsigned char *mem,
+                                            uint32_t bar_addr, int lane)
+    {
+        const int64_t s0 = warp_share(total_units, w, W, units) * kAdjUnit;
+        x = a.x + s0;
+        gy = a.gy + s0;
+        left = a.n - s0;
+        slots = reinterpret_cast<float2 *>(mem);
+        bars = bar_addr;
+        tiles = (units + SUB - 1) / SUB;
+        const int64_t f = left >= HALO ? (left - HALO) / S : 0;
+        whole = f < tiles ? (int)f : tiles;
+        plain = whole < units / SUB ? whole : units / SUB;
+        if (lane == 0) {
+            for (int s = 0; s < STAGES; ++s) mbar_init(bars + 8u * s, 1);
+            fence_barrier_init();
+            for (int i = 0; i < STAGES && i < tiles; ++i) issue(i);
+        }
+        __syncwarp();
+        return s0;
+    }
+    __device__ __forceinline__ int units_of(int i) const { return units - i * SUB < SUB ? units - i * SUB : SUB; }
+    // Samples of x and gy that the slot of tile i holds.
+    __device__ __forceinline__ void counts(int i, int &xc, int &gc) const
+    {
+        const int want = units_of(i) * kAdjUnit;
+        xc = want;
+        gc = want + HALO;
+        if (i >= whole) {
+            const int64_t rem = left - (int64_t)i * S;
+            xc = (int)(rem < xc ? rem : (int64_t)xc) & ~1;
+            gc = (int)(rem < gc ? rem : (int64_t)gc) & ~1;
+        }
+    }
+    __device__ __forceinline__ float2 *slot(int i) const { return slots + (i % STAGES) * kSlotElems; }
+    __device__ __forceinline__ void copy(int i, uint32_t xbytes, uint32_t gbytes)
+    {
+        const uint32_t fb = bars + 8u * (i % STAGES), dst = smem_addr(slot(i));
+        mbar_arrive_expect_tx(fb, xbytes + gbytes);
+        if (xbytes) bulk_copy_g2s(dst, x + (int64_t)i * S, xbytes, fb);
+        if (gbytes) bulk_copy_g2s(dst + S * (uint32_t)sizeof(float2), gy + (int64_t)i * S, gbytes, fb);
+    }
+    __device__ __forceinline__ void issue(int i)   // lane 0
+    {
+        if (i < plain) {
+            copy(i, S * (uint32_t)sizeof(float2), (S + HALO) * (uint32_t)sizeof(float2));
+        } else {
+            int xc, gc;
+            counts(i, xc, gc);
+            copy(i, (uint32_t)xc * (uint32_t)sizeof(float2), (uint32_t)gc * (uint32_t)sizeof(float2));
+        }
+    }
+    __device__ __forceinline__ bool wait(int i, int *status) const
+    {
+        return mbar_wait(bars + 8u * (i % STAGES), (uint32_t)((i / STAGES) & 1), status);
+    }
+    // The whole warp has read tile i: refill its slot.
+    __device__ __forceinline__ void refill(int i, int lane)
+    {
+        __syncwarp();
+        if (lane == 0 && i + STAGES < tiles) {
+            fence_proxy_async_smem();   // the reads above precede the copy's writes
+            issue(i + STAGES);
+        }
+    }
+    // After a failed wait on tile i: let the copies in flight land.
+    __device__ __forceinline__ void drain(int i, int *status) const
+    {
+        for (int q = i; q < i + STAGES && q < tiles; ++q) wait(q, status);
+    }
+    // The window of NX samples of x and NG of gy (from k0 on) of element off of tile i.
+    template <int NX, int NG>
+    __device__ __forceinline__ void window(int i, int off, int k0, float2 (&xs)[NX], float2 (&g)[NG]) const
+    {
+        const float2 *sl = slot(i);
+        if (i < whole) {
+            adj_slot_window<NX>(sl, off, xs);
+            adj_slot_window<NG>(sl + S, off + k0, g);
+        } else {
+            int xc, gc;
+            counts(i, xc, gc);
+            const int64_t at = (int64_t)i * S;
+            adj_slot_window_tail<NX>(sl, xc, x + at, off, left - at, xs);
+            adj_slot_window_tail<NG>(sl + S, gc, gy + at, off + k0, left - at, g);
+        }
+    }
+};
+
+// Shared-memory bytes of a staged kernel: barriers, scratch (coefficient table
+// or reduction rows), the rings of its warps.
+template <class Ring>
+__host__ __device__ constexpr size_t adj_staged_smem(int warps, int scratch_floats)
 {
-    return 128 + (((size_t)scratch_floats * 4 + 127) / 128) * 128 +
-           (size_t)stages * (size_t)adj_slot_elems(S, halo) * sizeof(float2);
+    return 512 + (((size_t)scratch_floats * 4 + 127) / 128) * 128 + (size_t)warps * Ring::kBytes;
 }
 
 // ---------------------------------------------------------------- input gradient
 // Adjoint table passed by value (kernel parameter bank), 16-byte aligned so
 // that its packed pairs can be 64-bit constant operands.
 template <int B, int T>
-struct alignas(8) AdjParamTab {
+struct alignas(16) AdjParamTab {
     float v[adj_table_floats(B, T)];
 };
 
@@ -196,99 +270,47 @@ template <int B, int T, int V, bool PARAM = false>
 __device__ __forceinline__ void gx_compute(const float *tab, const AdjParamTab<B, T> &ptab,
                                            const float2 (&xs)[V], const float2 (&g)[V + T - 1], float2 (&acc)[V])
 {
-    constexpr int QB = B, RB = B - 1;       // coefficients per Q / S polynomial
-    constexpr int PER_TAP = 4 * QB + 4 * RB;
     constexpr int W = V + T - 1;
     float2 gs[W];   // window samples swapped: {d, c}
 #pragma unroll
     for (int j = 0; j < W; ++j) gs[j] = make_float2(g[j].y, g[j].x);
-    float ur[V], ui[V], rr[V];
+    float rr[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) rr[v] = fmaf(xs[v].x, xs[v].x, xs[v].y * xs[v].y);
+    float2 val[V], der[V];   // V and V' of the Horner pass
+#pragma unroll
+    for (int b = B - 1; b >= 0; --b) {
+        if (b < B - 1) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const float2 r2 = make_float2(rr[v], rr[v]);
+                der[v] = b < B - 2 ? __ffma2_rn(der[v], r2, val[v]) : val[v];
+                val[v] = __fmul2_rn(val[v], r2);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < T; ++k) {
+            float4 c4;
+            const int o = 4 * (k * B + b);
+            if constexpr (PARAM)
+                c4 = make_float4(ptab.v[o], ptab.v[o + 1], ptab.v[o + 2], ptab.v[o + 3]);
+            else
+                c4 = *reinterpret_cast<const float4 *>(tab + o);
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const float2 p = make_float2(c4.x, c4.y), q = make_float2(c4.z, c4.w);
+                val[v] = (b == B - 1 && k == 0) ? __fmul2_rn(p, g[v + k]) : __ffma2_rn(p, g[v + k], val[v]);
+                val[v] = __ffma2_rn(q, gs[v + k], val[v]);
+            }
+        }
+    }
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        const float2 q = xs[v];
-        rr[v] = fmaf(q.x, q.x, q.y * q.y);
-        ur[v] = fmaf(q.x, q.x, -q.y * q.y);   // x^2
-        ui[v] = 2.f * q.x * q.y;
-    }
-    // {Re, Im} of the gradient of each sample, and of the tap sum of the second
-    // bracket (its factor x^2 does not depend on the tap, so it is applied once
-    // after the tap loop).  Every tap advances all V samples together with
-    // packed f32x2 FMAs (coefficient pairs adjacent in the table).
-    float2 ws[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-        acc[v] = make_float2(0.f, 0.f);
-        ws[v] = make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int k = 0; k < T; ++k) {
-        // quadruple j of tap k's block: the Q quadruples, then the S ones
-        auto coef = [&](int j) -> float4 {
-            if constexpr (PARAM) {
-                const int o = PER_TAP * k + 4 * j;
-                return make_float4(ptab.v[o], ptab.v[o + 1], ptab.v[o + 2], ptab.v[o + 3]);
-            } else {
-                return reinterpret_cast<const float4 *>(tab + PER_TAP * k)[j];
-            }
-        };
-        float2 pa[V], pb[V];
-        {
-            const float4 c4 = coef(QB - 1);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                pa[v] = make_float2(c4.x, c4.y);
-                pb[v] = make_float2(c4.z, c4.w);
-            }
-        }
-#pragma unroll
-        for (int m = QB - 2; m >= 0; --m) {
-            const float4 c4 = coef(m);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const float2 rr2 = make_float2(rr[v], rr[v]);
-                pa[v] = __ffma2_rn(pa[v], rr2, make_float2(c4.x, c4.y));
-                pb[v] = __ffma2_rn(pb[v], rr2, make_float2(c4.z, c4.w));
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            acc[v] = __ffma2_rn(pa[v], g[v + k], acc[v]);    // {Q0 c, Q3 d}
-            acc[v] = __ffma2_rn(pb[v], gs[v + k], acc[v]);   // {Q1 d, Q2 c}
-        }
-        if constexpr (RB > 0) {
-            float2 sa[V], sb[V];
-            {
-                const float4 c4 = coef(QB + RB - 1);
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    sa[v] = make_float2(c4.x, c4.y);
-                    sb[v] = make_float2(c4.z, c4.w);
-                }
-            }
-#pragma unroll
-            for (int m = RB - 2; m >= 0; --m) {
-                const float4 c4 = coef(QB + m);
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const float2 rr2 = make_float2(rr[v], rr[v]);
-                    sa[v] = __ffma2_rn(sa[v], rr2, make_float2(c4.x, c4.y));
-                    sb[v] = __ffma2_rn(sb[v], rr2, make_float2(c4.z, c4.w));
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                // conj(G) g + F conj(g) = {S0 c + S1 d, S2 c + S3 d}
-                ws[v] = __ffma2_rn(sa[v], g[v + k], ws[v]);    // {S0 c, S3 d}
-                ws[v] = __ffma2_rn(sb[v], gs[v + k], ws[v]);   // {S1 d, S2 c}
-            }
-        }
-    }
-    if constexpr (RB > 0) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            // acc += x^2 ws (complex):  {ur wr - ui wi, ur wi + ui wr}
-            acc[v] = __ffma2_rn(make_float2(ur[v], ur[v]), ws[v], acc[v]);
-            acc[v] = __ffma2_rn(make_float2(-ui[v], ui[v]), make_float2(ws[v].y, ws[v].x), acc[v]);
+        if constexpr (B > 1) {
+            const float t = 2.f * fmaf(xs[v].x, der[v].x, xs[v].y * der[v].y);
+            acc[v] = __ffma2_rn(xs[v], make_float2(t, t), val[v]);
+        } else {
+            acc[v] = val[v];
         }
     }
 }
@@ -340,64 +362,48 @@ __global__ void __launch_bounds__(256) adj_gx_kernel(AdjArgs a)
     }
 }
 
-// Staged variant: persistent CTAs of kAdjWarps consumer warps + 1 producer warp
-// walk tiles of S = kAdjWarps * 32 * V samples.  x and gy 16-byte aligned.
+using GxRing = AdjRing<kAdjStages, kAdjSub, kHalo>;
+
+// Staged variant: CTAs of kAdjWarps independent warps (see AdjRing).  x and gy
+// 16-byte aligned.
 template <int B, int T, int V, bool PARAM>
-__global__ void __launch_bounds__(32 * (kAdjWarps + 1))
-    adj_gx_tma_kernel(AdjArgs a, int stages, int64_t ntiles, const __grid_constant__ AdjParamTab<B, T> ptab)
+__global__ void __launch_bounds__(32 * kAdjWarps, 2)
+    adj_gx_tma_kernel(AdjArgs a, int64_t units, const __grid_constant__ AdjParamTab<B, T> ptab)
 {
     constexpr int W = V + T - 1;
     constexpr int TABF = adj_table_floats(B, T);
-    constexpr int S = kAdjWarps * 32 * V;
-    static_assert(T - 1 <= kHalo, "look-ahead must fit the slot");
+    constexpr int S = GxRing::S;
+    static_assert(T - 1 <= kHalo && V == kAdjV, "look-ahead must fit the slot");
+    static_assert(kAdjWarps * kAdjStages * 8 <= 512, "barrier area");
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem);   // full[s], empty[s]
-    float *tab = reinterpret_cast<float *>(smem + 128);
-    float2 *ring = reinterpret_cast<float2 *>(smem + adj_staged_smem(S, 0, adj_tab_padded<B, T>()));
+    float *tab = reinterpret_cast<float *>(smem + 512);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(smem_addr(&bars[s]), 1);
-            mbar_init(smem_addr(&bars[stages + s]), kAdjWarps);
-        }
-        fence_barrier_init();
-    }
-    if constexpr (!PARAM)
-        for (int i = tid; i < TABF; i += blockDim.x) tab[i] = a.adj_tab[i];
-    __syncthreads();
-    if (warp == kAdjWarps) {
-        if (lane == 0) adj_produce(a, ring, bars, stages, S, ntiles);
-        return;
+    grid_dep_wait();
+    GxRing ring;
+    const int64_t f0 = ring.init(a, units, warp * gridDim.x + blockIdx.x, kAdjWarps * gridDim.x,
+                                 smem + adj_staged_smem<GxRing>(warp, adj_tab_padded<B, T>()),
+                                 smem_addr(smem) + 8u * kAdjStages * warp, lane);
+    if constexpr (!PARAM) {
+        for (int i = tid; i < TABF; i += 32 * kAdjWarps) tab[i] = a.adj_tab[i];
+        __syncthreads();
     }
     const bool vec_out = (reinterpret_cast<uintptr_t>(a.gx) & 15) == 0;
-    const int slot_elems = adj_slot_elems(S);
-    int s = 0;          // slot and parity of the current tile, kept incrementally
-    uint32_t ph = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        if (!mbar_wait(smem_addr(&bars[s]), ph, a.status)) return;
-        const float2 *slot = ring + (size_t)s * slot_elems;
-        const int64_t s0 = tile * S;
-        const int off = tid * V;
-        const bool full = s0 + S + kHalo <= a.n;
-        float2 xs[V], g[W];
-        if (full) {
-            adj_slot_window<V>(slot, off, xs);
-            adj_slot_window<W>(slot + S, off, g);
-        } else {
-            int xc, gc;
-            adj_slot_counts(s0, S, a.n, xc, gc);
-            adj_slot_window_tail<V>(slot, s0, xc, a.x, s0 + off, a.n, xs);
-            adj_slot_window_tail<W>(slot + S, s0, gc, a.gy, s0 + off, a.n, g);
+    for (int i = 0; i < ring.tiles; ++i) {
+        if (!ring.wait(i, a.status)) {
+            ring.drain(i, a.status);
+            return;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_addr(&bars[stages + s]));
-        if (++s == stages) {
-            s = 0;
-            ph ^= 1u;
+        const int nu = ring.units_of(i);
+#pragma unroll 1
+        for (int j = 0; j < nu; ++j) {
+            const int off = j * kAdjUnit + lane * V;
+            float2 xs[V], g[W];
+            ring.window(i, off, 0, xs, g);
+            if (j == nu - 1) ring.refill(i, lane);
+            float2 acc[V];
+            gx_compute<B, T, V, PARAM>(tab, ptab, xs, g, acc);
+            gx_store<V>(a.gx, f0 + (int64_t)i * S + off, a.n, vec_out, acc, true);
         }
-        float2 acc[V];
-        gx_compute<B, T, V, PARAM>(tab, ptab, xs, g, acc);
-        gx_store<V>(a.gx, s0 + off, a.n, vec_out, acc, true);
     }
 }
 
@@ -445,38 +451,48 @@ __device__ __forceinline__ void gh_accumulate(const float2 (&xs)[V], const float
     }
 }
 
-// Fixed-order reduction of the accumulators of `nw` warps (threads tid < 32*nw
-// take part; `red` holds nw * NA floats), then one row of partials.  NAMED:
-// synchronise on named barrier 1 (the staged kernels, whose producer warp has
-// left) instead of __syncthreads.
-template <int B, int TG, bool NAMED>
-__device__ __forceinline__ void gh_reduce_row(float2 (&acc2)[2 * B * TG + 1], float *red, int nw, int tid, int k0,
+// Sum of every element of v over the 32 lanes of the warp, scattered: at each
+// step a lane sends half of its elements to its partner and keeps the sums of
+// the other half, so N elements take about N exchanges (a butterfly per element
+// takes 5 N: 510 against 101 shuffles per warp at B = TG = 5).  Element i's sum
+// ends in dst[i].
+template <int N, int O>
+__device__ __forceinline__ void lane_sums(const float (&v)[N], int lane, int base, int valid, float *dst)
+{
+    if constexpr (O == 0) {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (i < valid) dst[base + i] = v[i];
+    } else {
+        constexpr int H = (N + 1) / 2;
+        const bool up = (lane & O) != 0;
+        float w[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const float lo = v[i], hi = i + H < N ? v[i + H < N ? i + H : 0] : 0.f;
+            w[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
+        }
+        lane_sums<H, O / 2>(w, lane, base + (up ? H : 0), up ? valid - H : (valid < H ? valid : H), dst);
+    }
+}
+
+// Fixed-order reduction of the accumulators of the CTA's `nw` warps (`red`
+// holds nw * NA floats), then one row of partials.
+template <int B, int TG>
+__device__ __forceinline__ void gh_reduce_row(const float2 (&acc2)[2 * B * TG + 1], float *red, int nw, int tid, int k0,
                                               bool group0, int T, int Bp, int Bq, float2 *row)
 {
     constexpr int NP = 2 * B * TG + 1;
     constexpr int NA = 2 * NP;
     const int lane = tid & 31, warp = tid >> 5;
+    float v[NA];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-        float2 v = acc2[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-        }
-        acc2[i] = v;
+        v[2 * i] = acc2[i].x;
+        v[2 * i + 1] = acc2[i].y;
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            red[warp * NA + 2 * i] = acc2[i].x;
-            red[warp * NA + 2 * i + 1] = acc2[i].y;
-        }
-    }
-    if constexpr (NAMED)
-        asm volatile("bar.sync 1, %0;" ::"r"(nw * 32) : "memory");
-    else
-        __syncthreads();
+    lane_sums<NA, 16>(v, lane, 0, NA, red + warp * NA);
+    __syncthreads();
     // One (b, kk) pair per thread: X and Y summed over the warps in index
     // order, then both branches.
     for (int e = tid; e <= B * TG; e += nw * 32) {
@@ -522,134 +538,61 @@ __global__ void __launch_bounds__(256) adj_gh_kernel(AdjArgs a, int T, int Bp, i
         gh_accumulate<B, TG, V>(xs, g, blockIdx.y == 0, acc2);
     }
     __shared__ float red[8 * NA];
-    gh_reduce_row<B, TG, false>(acc2, red, blockDim.x >> 5, threadIdx.x, k0, blockIdx.y == 0, T, Bp, Bq,
+    gh_reduce_row<B, TG>(acc2, red, blockDim.x >> 5, threadIdx.x, k0, blockIdx.y == 0, T, Bp, Bq,
                                 a.partials + (size_t)blockIdx.x * K);
 }
 
-// Staged variant: grid (blocks, tap groups) of persistent CTAs of kAdjGhWarps
-// warps, every CTA streaming the tiles of its blockIdx.x share.  x and gy
-// 16-byte aligned.  With 2 B TG + 1 packed accumulators a thread takes about
-// 170 registers, so one CTA fits an SM; the bulk copies are issued by lane 0
-// of warp 0 between its own tiles instead of by a separate producer warp, so
-// that all twelve warps (three per SM sub-partition) accumulate.  At the start
-// of its tile i warp 0 refills the slot of tile i - 1 (once every warp has
-// released it) with tile i - 1 + stages; the whole warp waits, so that its
-// lanes stay converged.
+using GhRing = AdjRing<kAdjGhStages, kAdjGhSub, kAdjGhHalo>;
+
+// Staged variant: grid (blocks, tap groups) of CTAs of kAdjGhWarps independent
+// warps (see AdjRing), block x of a tap group sharing the record with the
+// others of the group.  x and gy 16-byte aligned.  With 2 B TG + 1 packed
+// accumulators a thread takes about 165 registers, so one CTA fits an SM.
 template <int B, int TG, int V>
-__device__ __forceinline__ void adj_gh_tma_body(const AdjArgs &a, int stages, int64_t ntiles, int T, int Bp, int Bq,
-                                                int K)
+__device__ __forceinline__ void adj_gh_tma_body(const AdjArgs &a, int T, int Bp, int Bq, int K)
 {
     constexpr int NA = 4 * B * TG + 2;
     constexpr int NP = NA / 2;
-    constexpr int S = kAdjGhWarps * 32 * V * kAdjGhSub;
     constexpr int NG = V + TG - 1;
+    static_assert(TG <= kAdjGhMaxTG && V == kAdjV, "tap group exceeds the staged look-ahead");
+    static_assert(kAdjGhWarps * kAdjGhStages * 8 <= 512, "barrier area");
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem);   // full[s], empty[s]
-    float *red = reinterpret_cast<float *>(smem + 128);
-    static_assert(TG <= kAdjGhMaxTG, "tap group exceeds the staged look-ahead");
-    float2 *ring = reinterpret_cast<float2 *>(smem + adj_staged_smem(S, 0, kAdjGhWarps * NA, kAdjGhHalo));
+    float *red = reinterpret_cast<float *>(smem + 512);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int k0 = blockIdx.y * TG;
     const bool group0 = blockIdx.y == 0;
-    const bool producer = tid == 0;
-    const int slot_elems = adj_slot_elems(S, kAdjGhHalo);
-    // Local tile i of this CTA is global tile blockIdx.x + i * gridDim.x.
-    const int64_t nlocal = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    auto issue = [&](int64_t i) {   // producer: tile i into slot i % stages (its empty phase passed)
-        const int sl = (int)(i % stages);
-        const int64_t s0 = ((int64_t)blockIdx.x + i * gridDim.x) * S;
-        int xc, gc;
-        adj_slot_counts(s0, S, a.n, xc, gc, kAdjGhHalo);
-        const uint32_t fb = smem_addr(&bars[sl]);
-        float2 *slot = ring + (size_t)sl * slot_elems;
-        mbar_arrive_expect_tx(fb, (uint32_t)(xc + gc) * (uint32_t)sizeof(float2));
-        if (xc) bulk_copy_g2s(smem_addr(slot), a.x + s0, (uint32_t)xc * sizeof(float2), fb);
-        if (gc) bulk_copy_g2s(smem_addr(slot + S), a.gy + s0, (uint32_t)gc * sizeof(float2), fb);
-    };
-    if (producer) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(smem_addr(&bars[s]), 1);
-            mbar_init(smem_addr(&bars[stages + s]), kAdjGhWarps);
-        }
-        fence_barrier_init();
-    }
-    __syncthreads();
-    int64_t issued = 0;   // tiles issued so far (kept by every lane of warp 0)
-    if (warp == 0)
-        for (; issued < stages && issued < nlocal; ++issued)
-            if (producer) issue(issued);
+    grid_dep_wait();
+    GhRing ring;
+    ring.init(a, (a.n + kAdjUnit - 1) / kAdjUnit, warp * gridDim.x + blockIdx.x, kAdjGhWarps * gridDim.x,
+              smem + adj_staged_smem<GhRing>(warp, kAdjGhWarps * NA), smem_addr(smem) + 8u * kAdjGhStages * warp, lane);
     float2 acc2[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) acc2[i] = make_float2(0.f, 0.f);
-    int s = 0;          // slot and parity of the current tile, kept incrementally
-    uint32_t ph = 0;
-    bool ok = true;
-    for (int64_t i = 0; i < nlocal; ++i) {
+    for (int i = 0; i < ring.tiles; ++i) {
         // A failed wait (error word set) ends this warp's tiles; it still joins
         // the reduction so that no warp waits for it.
-        if (!mbar_wait(smem_addr(&bars[s]), ph, a.status)) {
-            ok = false;
+        if (!ring.wait(i, a.status)) {
+            ring.drain(i, a.status);
             break;
         }
-        // Refill: tile i - 1 + stages into the slot of tile i - 1, once all
-        // warps have released that tile (empty phase (i - 1) / stages).
-        if (warp == 0 && i >= 1 && issued < nlocal) {
-            const int64_t done = i - 1;
-            bool w = mbar_wait(smem_addr(&bars[stages + (int)(done % stages)]), (uint32_t)((done / stages) & 1),
-                               a.status);
-            w = __shfl_sync(0xffffffffu, w, 0);   // lane 0's outcome for the whole warp
-            if (!w) {
-                ok = false;
-                break;
-            }
-            if (producer) issue(issued);
-            ++issued;
-            __syncwarp();
-        }
-        const float2 *slot = ring + (size_t)s * slot_elems;
-        const int64_t s0 = ((int64_t)blockIdx.x + i * gridDim.x) * S;
-        const bool fast = s0 + S + kAdjGhHalo <= a.n;
-        int xc = S, gc = S + kAdjGhHalo;
-        if (!fast) adj_slot_counts(s0, S, a.n, xc, gc, kAdjGhHalo);
-        // Sub-block j of the tile: samples (j * threads + tid) * V ..; the slot
-        // is released once the last sub-block's windows are in registers.
+        const int nu = ring.units_of(i);
 #pragma unroll 1
-        for (int j = 0; j < kAdjGhSub; ++j) {
-            const int off = (j * kAdjGhWarps * 32 + tid) * V;
+        for (int j = 0; j < nu; ++j) {
+            const int off = j * kAdjUnit + lane * V;
             float2 xs[V], g[NG];
-            if (fast) {
-                adj_slot_window<V>(slot, off, xs);
-                adj_slot_window<NG>(slot + S, off + k0, g);
-            } else {
-                adj_slot_window_tail<V>(slot, s0, xc, a.x, s0 + off, a.n, xs);
-                adj_slot_window_tail<NG>(slot + S, s0, gc, a.gy, s0 + off + k0, a.n, g);
-            }
-            if (j == kAdjGhSub - 1) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_addr(&bars[stages + s]));
-            }
+            ring.window(i, off, k0, xs, g);
+            if (j == nu - 1) ring.refill(i, lane);
             gh_accumulate<B, TG, V>(xs, g, group0, acc2);
         }
-        if (++s == stages) {
-            s = 0;
-            ph ^= 1u;
-        }
     }
-    if (producer && !ok) {
-        // Let the copies already issued land before the CTA exits.
-        const int64_t first = issued > stages ? issued - stages : 0;
-        for (int64_t q = first; q < issued; ++q)
-            mbar_wait(smem_addr(&bars[q % stages]), (uint32_t)((q / stages) & 1), a.status);
-    }
-    gh_reduce_row<B, TG, false>(acc2, red, kAdjGhWarps, tid, k0, group0, T, Bp, Bq,
-                                a.partials + (size_t)blockIdx.x * K);
+    gh_reduce_row<B, TG>(acc2, red, kAdjGhWarps, tid, k0, group0, T, Bp, Bq, a.partials + (size_t)blockIdx.x * K);
 }
 
 template <int B, int TG, int V>
 __global__ void __launch_bounds__(32 * kAdjGhWarps, 1)
-    adj_gh_tma_kernel(AdjArgs a, int stages, int64_t ntiles, int T, int Bp, int Bq, int K)
+    adj_gh_tma_kernel(AdjArgs a, int T, int Bp, int Bq, int K)
 {
-    adj_gh_tma_body<B, TG, V>(a, stages, ntiles, T, Bp, Bq, K);
+    adj_gh_tma_body<B, TG, V>(a, T, Bp, Bq, K);
 }
 
 // Many independent problems in one launch (the least-squares refinement of a
@@ -658,11 +601,11 @@ __global__ void __launch_bounds__(32 * kAdjGhWarps, 1)
 // from args[z].
 template <int B, int TG, int V>
 __global__ void __launch_bounds__(32 * kAdjGhWarps, 1)
-    adj_gh_tma_batched_kernel(const AdjArgs *__restrict__ args, int stages, int T, int Bp, int Bq, int K)
+    adj_gh_tma_batched_kernel(const AdjArgs *__restrict__ args, int T, int Bp, int Bq, int K)
 {
-    constexpr int S = kAdjGhWarps * 32 * V * kAdjGhSub;
+    grid_dep_wait();   // before args is read: the work list may have just been uploaded
     const AdjArgs a = args[blockIdx.z];
-    adj_gh_tma_body<B, TG, V>(a, stages, (a.n + S - 1) / S, T, Bp, Bq, K);
+    adj_gh_tma_body<B, TG, V>(a, T, Bp, Bq, K);
 }
 
 // ---------------------------------------------------------------- launches
@@ -675,24 +618,21 @@ inline bool adj_staged_ok(const AdjArgs &a)
 template <int B, int T, int V, bool PARAM>
 cudaError_t launch_adj_gx_tma(const AdjArgs &a, const AdjParamTab<B, T> &ptab, int sm_count, cudaStream_t s)
 {
-    constexpr int S = kAdjWarps * 32 * V;
     // The shared-memory table area is kept in both forms (it is small).
-    const size_t smem = adj_staged_smem(S, kAdjStages, adj_tab_padded<B, T>());
+    const size_t smem = adj_staged_smem<GxRing>(kAdjWarps, adj_tab_padded<B, T>());
     auto kern = adj_gx_tma_kernel<B, T, V, PARAM>;
     static SmemAttr smem_rec;
     cudaError_t attr = ensure_smem(smem_rec, (const void *)kern, smem);
     if (attr != cudaSuccess) return attr;
     static OccCache occ_rec;
     int occ = 0;
-    attr = occupancy(occ_rec, (const void *)kern, 32 * (kAdjWarps + 1), smem, &occ);
+    attr = occupancy(occ_rec, (const void *)kern, 32 * kAdjWarps, smem, &occ);
     if (attr != cudaSuccess) return attr;
     if (occ < 1) occ = 1;
-    const int64_t ntiles = (a.n + S - 1) / S;
+    const int64_t units = (a.n + kAdjUnit - 1) / kAdjUnit;
     int64_t grid = (int64_t)sm_count * occ;
-    if (grid > ntiles) grid = ntiles;
-    kern<<<(unsigned)grid, 32 * (kAdjWarps + 1), smem, s>>>(a, kAdjStages, ntiles, ptab);
-    count_launch();
-    return cudaGetLastError();
+    if (grid > units) grid = units;
+    return launch_pdl(kern, dim3((unsigned)grid), 32 * kAdjWarps, smem, s, a, units, ptab);
 }
 
 template <int B, int T>
@@ -726,17 +666,13 @@ cudaError_t launch_adj_gh_tg(const AdjArgs &a, int blocks, int T, int Bp, int Bq
     const int groups = (T + TG - 1) / TG;
     dim3 grid((unsigned)blocks, (unsigned)groups);
     if (adj_staged_ok(a)) {
-        constexpr int V = kAdjGhV;
-        constexpr int S = kAdjGhWarps * 32 * V * kAdjGhSub;
+        constexpr int V = kAdjV;
         constexpr int NA = 4 * B * TG + 2;
-        const size_t smem = adj_staged_smem(S, kAdjGhStages, kAdjGhWarps * NA, kAdjGhHalo);
+        const size_t smem = adj_staged_smem<GhRing>(kAdjGhWarps, kAdjGhWarps * NA);
         static SmemAttr smem_rec;
         const cudaError_t attr = ensure_smem(smem_rec, (const void *)adj_gh_tma_kernel<B, TG, V>, smem);
         if (attr != cudaSuccess) return attr;
-        const int64_t ntiles = (a.n + S - 1) / S;
-        adj_gh_tma_kernel<B, TG, V><<<grid, 32 * kAdjGhWarps, smem, s>>>(a, kAdjGhStages, ntiles, T, Bp, Bq, K);
-        count_launch();
-        return cudaGetLastError();
+        return launch_pdl(adj_gh_tma_kernel<B, TG, V>, grid, 32 * kAdjGhWarps, smem, s, a, T, Bp, Bq, K);
     }
     adj_gh_kernel<B, TG, kAdjV><<<grid, 256, 0, s>>>(a, T, Bp, Bq, K);
     count_launch();
@@ -762,17 +698,14 @@ template <int B, int TG>
 cudaError_t launch_adj_gh_batched_tg(const AdjArgs *args, int count, int blocks, int T, int Bp, int Bq, int K,
                                      cudaStream_t s)
 {
-    constexpr int V = kAdjGhV;
-    constexpr int S = kAdjGhWarps * 32 * V * kAdjGhSub;
+    constexpr int V = kAdjV;
     constexpr int NA = 4 * B * TG + 2;
-    const size_t smem = adj_staged_smem(S, kAdjGhStages, kAdjGhWarps * NA, kAdjGhHalo);
+    const size_t smem = adj_staged_smem<GhRing>(kAdjGhWarps, kAdjGhWarps * NA);
     static SmemAttr smem_rec;
     const cudaError_t attr = ensure_smem(smem_rec, (const void *)adj_gh_tma_batched_kernel<B, TG, V>, smem);
     if (attr != cudaSuccess) return attr;
     dim3 grid((unsigned)blocks, (unsigned)((T + TG - 1) / TG), (unsigned)count);
-    adj_gh_tma_batched_kernel<B, TG, V><<<grid, 32 * kAdjGhWarps, smem, s>>>(args, kAdjGhStages, T, Bp, Bq, K);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(adj_gh_tma_batched_kernel<B, TG, V>, grid, 32 * kAdjGhWarps, smem, s, args, T, Bp, Bq, K);
 }
 
 template <int B>

@@ -81,12 +81,10 @@ struct FwdArgs {
     double *norms = nullptr;
 };
 
-// Floats of the adjoint table: per tap, four polynomials of B coefficients
-// (Q0..Q3 for conj(E) g + H conj(g)) and four of B-1 (S0..S3 for
-// conj(G) g + F conj(g)), stored power-major as quadruples {Q0, Q3, Q1, Q2}
-// then {S0, S3, S1, S2}; see dpd_adj.cuh.
-__host__ __device__ constexpr int adj_table_floats(int B, int T) { return (4 * B + 4 * (B - 1)) * T; }
-constexpr int kMaxAdjTabFloats = adj_table_floats(6, 8);   // 352
+// Floats of the adjoint table: per tap k and power b the transposed 2 x 2 real
+// matrix of the forward table as the quadruple {P0, P3, P2, P1}; see dpd_adj.cuh.
+__host__ __device__ constexpr int adj_table_floats(int B, int T) { return 4 * B * T; }
+constexpr int kMaxAdjTabFloats = adj_table_floats(6, 8);   // 192
 
 struct AdjArgs {
     const float2 *x;
@@ -201,6 +199,27 @@ inline cudaError_t occupancy(OccCache &c, const void *kern, int threads, size_t 
     }
     *occ = en.occ;
     return cudaSuccess;
+}
+
+// Launch `kern` with programmatic stream serialisation: it may begin while the
+// kernel before it in the stream drains, and must call grid_dep_wait() before it
+// touches memory that earlier work wrote or may still read.
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace dpd

@@ -76,6 +76,29 @@ def test_grad_sizes_and_tap_schedules(n, launch):
     check_gh(gh, x, h, gy, P, Q, M)
 
 
+@pytest.mark.parametrize("n", [127, 128, 129, 136, 137, 255, 256, 264, 265, 383, 384, 395, 396, 397, 4 * 384 + 11,
+                               128 * 1824 * 2 + 1])
+@pytest.mark.parametrize("P,Q,M", [(9, 9, 4), (11, 3, 7)])
+def test_grad_warp_ring_edges(n, P, Q, M):
+    """Sizes around a warp's 128-sample unit, the 256- and 384-sample ring tiles
+    of the two staged kernels and their 8- and 12-sample look-ahead, and a
+    record that splits unevenly over every warp of the GPU; from host and
+    from device coefficients."""
+    x, h, gy = make(P, Q, M, n, 3 * n + M)
+    _, gx_ref = oracle.grad(x, h, gy, P, Q, M, want_h=False)
+    xd, gyd = torch.from_numpy(x).cuda(), torch.from_numpy(gy).cuda()
+    for src in (h, torch.from_numpy(h).cuda()):
+        f = dpd.DPD(P, Q, M)
+        f.set_coeffs(src)
+        gx = torch.full_like(xd, complex(5, 5))
+        gh = torch.full((f.K,), complex(5, 5), dtype=torch.complex64, device="cuda")
+        f.grad(xd, gyd, gh=gh, gx=gx)
+        f.sync_status()
+        f.close()
+        assert_parity(gx.cpu().numpy(), gx_ref, what=f"gx n={n}")
+        check_gh(gh.cpu().numpy(), x, h, gy, P, Q, M)
+
+
 @pytest.mark.parametrize("n", [1, 9, 1031, 2 * 1024 + 9, 20011])
 @pytest.mark.parametrize("shift", [(0, 0, 1), (1, 0, 0), (0, 1, 0), (1, 1, 1)])
 def test_grad_alignment_paths(n, shift):
