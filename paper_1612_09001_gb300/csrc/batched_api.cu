@@ -22,8 +22,8 @@ struct dpd_plan_s {
     int nitems = 0;
     int64_t tab_floats = 0;
     int small = 1;            // every stream has B <= 5 and T <= 7
-    int V = 8, warps = 8, stages = 4, ctas_per_sm = 0, group = 0;
-    int nsub = dpd::batch_nsub(8, 8, 4, 8);   // sub-blocks per thread and item (follows the launch shape)
+    int V = 0, warps = 0, stages = 0, ctas_per_sm = 0, group = 0;   // launch shape (default_shape, or set explicitly)
+    int nsub = 0;             // sub-blocks per thread and item (follows the launch shape)
 };
 
 namespace {
@@ -34,6 +34,28 @@ bool overlap(const void *a, size_t na, const void *b, size_t nb)
 {
     const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
     return na && nb && x < y + nb && y < x + na;
+}
+
+// Launch shape of a new plan.  Long batches: 6 samples per thread (the 16-byte
+// window loads of a quarter warp on distinct banks), 16 warps in groups of 4,
+// items of 12,288 samples.  That needs enough items that the last round of
+// them is a small part of a CTA's work, so batches with fewer than four such
+// items per SM take 4 samples per thread, 4 warps and items of 2,048 samples
+// on as many CTAs as fit an SM.  GB300, us per launch, first shape / second
+// shape / 8 samples per thread on 8 warps (items of 8,192): 64 streams, 36.7 M
+// samples 140.8 / 150 / 217.7; 24 streams, 12.2 M 56.2 / 57.7 / 89.3; 33
+// streams, 3.8 M 40.1 / 29.1 / 49.5; 16 streams, 1.3 M 19.3 / 17.5 / 23.1; 8
+// streams, 0.17 M 17.3 / 10.9 / 15.1.
+void default_shape(dpd_plan p)
+{
+    int64_t units = 0;   // of 1024 samples; an item of the first shape has 12
+    for (const dpd::BatchStream &st : p->streams) units += st.n / 1024;
+    const bool large = units >= 4 * 12 * (int64_t)p->sm_count;
+    p->V = large ? 6 : 4;
+    p->warps = large ? 16 : 4;
+    p->stages = large ? 2 : 3;
+    p->group = large ? 4 : 0;
+    p->nsub = dpd::batch_nsub(p->warps, 4, p->stages, p->V);
 }
 
 void free_plan(dpd_plan p)
@@ -166,6 +188,7 @@ dpd_status dpd_plan_batched(const dpd_stream_desc *descs, int count, int where, 
         free_plan(p);
         return DPD_ERR_CUDA;
     }
+    default_shape(p);
     dpd_status st = build_items(p, p->V, p->warps, p->nsub);
     if (st == DPD_OK && cudaDeviceSynchronize() != cudaSuccess) st = DPD_ERR_CUDA;
     if (st != DPD_OK) {
