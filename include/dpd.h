@@ -203,11 +203,12 @@ dpd_status dpd_set_adj_launch(dpd_handle h, int gh_blocks, int tap_group);
  * stream of transmit samples, Sec. 2 and Sec. 4).  The history before x[0] is the last M input
  * samples of the previous dpd_apply_stream call on this handle (zero after
  * dpd_create or dpd_reset_stream), so the outputs equal one dpd_apply over the
- * concatenated input.  Two launches on `stream`: the forward filter (zero
- * history), then one warp that recomputes y[0 .. min(M, n)) with the saved
- * history and saves the last 8 input samples into the handle.  Calls on one
- * handle must therefore be ordered on one stream (or synchronised), and x must
- * stay valid until the second launch has run.  Same buffer rules and errors as
+ * concatenated input.  One launch on `stream`, the forward filter, which reads
+ * the saved history and replaces it by the last 8 input samples; for an x that
+ * is only 8-byte aligned, or with plain loads selected, the forward filter with
+ * zero history and a second launch of one warp that recomputes y[0 .. min(M, n))
+ * and saves the history.  Calls on one handle must therefore be ordered on one
+ * stream (or synchronised), and x must stay valid until the last launch has run.  Same buffer rules and errors as
  * dpd_apply; n == 0 changes nothing.  Allocation-free and capturable.
  */
 dpd_status dpd_apply_stream(dpd_handle h, const void *x, void *y, int64_t n, void *stream);

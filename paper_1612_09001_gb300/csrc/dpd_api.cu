@@ -315,7 +315,10 @@ static dpd::FwdLaunch launch_for(dpd_handle h, int64_t n, bool param_tab)
     return L;
 }
 
-dpd_status dpd_apply(dpd_handle h, const void *x, void *y, int64_t n, void *stream)
+// y = DPD(x) with the samples in `hist` in front of x[0], which is updated, or
+// with zero history (null).  Where the plain-load kernel runs, a history is left
+// to a second launch.
+static dpd_status apply_block(dpd_handle h, const void *x, void *y, int64_t n, void *stream, float2 *hist)
 {
     if (!h || n < 0) return DPD_ERR_INVALID_ARGUMENT;
     if (!h->has_coeffs) return DPD_ERR_NO_COEFFS;
@@ -339,7 +342,16 @@ dpd_status dpd_apply(dpd_handle h, const void *x, void *y, int64_t n, void *stre
         L.use_tma = 0;
         L.V = 4;
     }
-    return cuda_status(dpd::launch_fwd_any(h->B, h->T, a, L, h->sm_count, static_cast<cudaStream_t>(stream)));
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (L.use_tma) a.hist = hist;
+    const cudaError_t e = dpd::launch_fwd_any(h->B, h->T, a, L, h->sm_count, s);
+    if (e != cudaSuccess || !hist || L.use_tma) return cuda_status(e);
+    return cuda_status(dpd::launch_stream_head(h->d_tab, h->B, h->T, a.x, n, hist, a.y, s));
+}
+
+dpd_status dpd_apply(dpd_handle h, const void *x, void *y, int64_t n, void *stream)
+{
+    return apply_block(h, x, y, n, stream, nullptr);
 }
 
 dpd_status dpd_grad(dpd_handle h, const void *x, const void *gy, int64_t n, void *gh, void *gx,
@@ -570,13 +582,7 @@ dpd_status dpd_set_adj_launch(dpd_handle h, int gh_blocks, int tap_group)
 
 dpd_status dpd_apply_stream(dpd_handle h, const void *x, void *y, int64_t n, void *stream)
 {
-    if (!h || n < 0) return DPD_ERR_INVALID_ARGUMENT;
-    if (!h->has_coeffs) return DPD_ERR_NO_COEFFS;
-    if (n == 0) return DPD_OK;
-    const dpd_status st = dpd_apply(h, x, y, n, stream);   // zero history; checks the buffers
-    if (st != DPD_OK) return st;
-    return cuda_status(dpd::launch_stream_head(h->d_tab, h->B, h->T, static_cast<const float2 *>(x), n, h->d_hist,
-                                               static_cast<float2 *>(y), static_cast<cudaStream_t>(stream)));
+    return apply_block(h, x, y, n, stream, h ? h->d_hist : nullptr);
 }
 
 dpd_status dpd_sq_error(dpd_handle h, const void *y, const void *x, int64_t n, float gain_re, float gain_im,

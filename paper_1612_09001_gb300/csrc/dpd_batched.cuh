@@ -185,6 +185,12 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
                 int off = 0;
                 if (s0 < st.n) tile_copy_range(s0, SG, st.n, lo, cnt, off);
                 if (cnt < 0) cnt = 0;
+                if (s0 == 0) {   // zero history; the fence orders it before later copies into the slot
+                    float4 *z = reinterpret_cast<float4 *>(slot + kBatchHdrBytes + kBatchTabBytes);
+#pragma unroll
+                    for (int q = 0; q < kHalo / 2; ++q) z[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    fence_proxy_async_smem();
+                }
                 const uint32_t xbytes = (uint32_t)(cnt * (int64_t)sizeof(float2));
                 // The arrive releases the header stores; the consumers' wait acquires them.
                 mbar_arrive_expect_tx(fb, xbytes + (uint32_t)st.tab_bytes);

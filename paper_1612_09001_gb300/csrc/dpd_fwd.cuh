@@ -130,10 +130,11 @@ __host__ __device__ constexpr int tab_bytes()
 }
 
 // Read the window of thread t_in_tile of a tile that starts at sample s0 from a
-// shared-memory slot holding global samples [s0 - kHalo, ...).  Samples in
-// [lo, vhi) are in the slot; the sample just past vhi (odd tail) comes from
-// global memory; samples outside [0, n) are zero.  Returns true when the whole
-// tile and its history are in the slot (the vectorised fast path).
+// shared-memory slot holding samples [s0 - kHalo, ...); those in front of the
+// input (the first tile) are its history, which put_history has placed there.
+// Samples below vhi are in the slot; the sample just past vhi (odd tail) comes
+// from global memory, and those past n are zero.  Returns true when the whole
+// tile is in the slot (the vectorised fast path).
 template <int T, int V>
 __device__ __forceinline__ bool load_window(const float2 *slot, int64_t s0, int S, int64_t n,
                                             const float2 *__restrict__ x, int t_in_tile,
@@ -141,10 +142,9 @@ __device__ __forceinline__ bool load_window(const float2 *slot, int64_t s0, int 
 {
     constexpr int W = V + T - 1;
     const int64_t g0 = s0 + (int64_t)t_in_tile * V;
-    const int64_t lo = (s0 - kHalo > 0) ? s0 - kHalo : 0;
     const int64_t hi = (s0 + S < n) ? s0 + S : n;
-    const int64_t vhi = lo + ((hi - lo) & ~int64_t(1));
-    const bool full = (s0 >= kHalo) && (s0 + S <= vhi);
+    const int64_t vhi = hi & ~int64_t(1);   // s0 and S are even
+    const bool full = s0 + S <= vhi;
     if (full) {
         constexpr int MP = ((T - 1) + 1) & ~1;   // history rounded up to a 16-byte unit
         constexpr int E = V + MP;
@@ -169,9 +169,9 @@ __device__ __forceinline__ bool load_window(const float2 *slot, int64_t s0, int 
         for (int j = 0; j < W; ++j) {
             const int64_t g = g0 - (T - 1) + j;
             float2 v = make_float2(0.f, 0.f);
-            if (g >= lo && g < vhi)
+            if (g < vhi)
                 v = slot[g - (s0 - kHalo)];
-            else if (g >= 0 && g < n)
+            else if (g < n)
                 v = x[g];
             wr[j] = v.x;
             wi[j] = v.y;
@@ -193,6 +193,34 @@ __device__ __forceinline__ void tile_copy_range(int64_t s0, int S, int64_t n, in
     }
     const int64_t hi = (s0 + S < n) ? s0 + S : n;
     cnt = (hi - lo) & ~int64_t(1);
+}
+
+// The kHalo samples in front of the input, in the slot of the tile at sample 0:
+// `hist` (dpd_apply_stream), or zeros.  By one warp, which also leaves the last
+// kHalo samples of (hist ++ x) in hist for the next block: only this warp of the
+// grid touches hist, and every read of the old one precedes the writes.  The
+// fence orders the stores before a later bulk copy into the same slot.  The
+// consumers need no case for the first tile and no history pointer (one in their
+// code cost the headline kernel two registers and a CTA per SM).  GB300, 16 blocks
+// of 30,720 samples, P = Q = 7, M = 3: 142.9 us; with a second launch per block
+// that recomputed the first M outputs 197.5 (5.6 us of 10 us per block).
+__device__ __forceinline__ void put_history(float2 *slot, const float2 *__restrict__ x, int64_t n, float2 *hist,
+                                            int lane)
+{
+    static_assert(kHalo <= 32, "one lane per history sample");
+    if (lane < kHalo) {
+        float2 v = make_float2(0.f, 0.f), next = v;
+        if (hist) {
+            v = hist[lane];
+            const int64_t src = (int64_t)lane + n;   // of (hist ++ x)
+            next = src < kHalo ? hist[src] : x[src - kHalo];
+        }
+        slot[lane] = v;
+        fence_proxy_async_smem();
+        __syncwarp((1u << kHalo) - 1u);
+        if (hist) hist[lane] = next;
+    }
+    __syncwarp();
 }
 
 template <int V>
@@ -301,6 +329,7 @@ __global__ void __launch_bounds__(fwd_lb_threads<SH>(), fwd_lb_blocks<SH>())
 
     if (warp == nwarps) {
         // ---------------------------------------------------------------- producer
+        if (blockIdx.x == 0) put_history(ring, a.x, a.n, a.hist, lane);   // tile 0: group 0, slot 0
         if (lane != 0) return;
         const uint64_t pol = policy_evict_first();
         int64_t it = 0;

@@ -79,6 +79,9 @@ struct FwdArgs {
     // finish adds the partials in a fixed order, writes the results and clears
     // the counter.
     double *norms = nullptr;
+    // kHalo samples in front of x[0], replaced by those in front of the next
+    // block, or null: zero history (bulk-copy kernel only).
+    float2 *hist = nullptr;
 };
 
 // Floats of the adjoint table: per tap k and power b the transposed 2 x 2 real

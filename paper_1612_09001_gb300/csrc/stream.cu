@@ -1,8 +1,9 @@
-// Stream continuation for dpd_apply_stream.  A block of a continuous stream
-// differs from an isolated block only in its first M outputs: the taps of
-// Eq. 1 reach back into the previous block.  The forward kernels run on the
-// block with zero history; this kernel then recomputes those outputs with the
-// saved history and saves the new one.
+// Stream continuation for dpd_apply_stream where the plain-load forward kernel
+// runs (the bulk-copy kernel takes the history itself).  A block of a continuous
+// stream differs from an isolated block only in its first M outputs: the taps of
+// Eq. 1 reach back into the previous block.  The forward kernel runs on the block
+// with zero history; this kernel then recomputes those outputs with the saved
+// history and saves the new one.
 #include "dpd_handle.h"
 
 namespace dpd {
