@@ -100,12 +100,18 @@ cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *pro
 // G (K x K, row-major), g (K) and t^H t per problem from S.
 cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int B, int T, double2 *G, double2 *g,
                                  double *tt, cudaStream_t s);
-// Power sums of r = |u|^2 per problem: mom[p][k - 1] = sum_n r_n^k, k = 1 .. 2 kMaxB - 1,
-// in a fixed order: per thread as exact FP32 two-sum pairs, then FP64 (part: nprob *
-// kMomBlocks * kMomK doubles of scratch).
+// Power sums of r = |u|^2 per problem: mom[p][k - 1] = sum_n r_n^k, k = 1 .. 2 B - 1
+// (zero up to kMomK), in a fixed order: exact FP32 two-sum pairs within a block,
+// then FP64 (part: nprob * moments_blocks(nprob) * kMomK doubles of scratch).
+// nmax: the longest problem.
 constexpr int kMomK = 2 * kMaxB - 1;
-constexpr int kMomBlocks = 64;
-cudaError_t launch_moments(const GramProblem *probs, int nprob, double *part, double *mom, cudaStream_t s);
+constexpr int kMomBlocks = 456;   // over all problems: three per SM at 152 SMs
+__host__ __device__ constexpr int moments_blocks(int nprob)   // blocks a problem gets at most
+{
+    return nprob < kMomBlocks ? kMomBlocks / nprob : 1;
+}
+cudaError_t launch_moments(const GramProblem *probs, int nprob, int64_t nmax, int B, double *part, double *mom,
+                           cudaStream_t s);
 // Coefficient vectors between the monomial basis and the basis U (both
 // branches, every tap; the constant unchanged), per problem:
 //   to_monomial: out = W in       (h = W h_U)

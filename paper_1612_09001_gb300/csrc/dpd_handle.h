@@ -28,7 +28,7 @@ struct EstimateWorkspace {
     float *ubasis = nullptr;      // [nprob][kUSize] basis coefficients used by the Gram kernels
     double *ubasis64 = nullptr;   // the same values in FP64, for the coefficient transforms
     double *mom = nullptr;        // [nprob][kMomK] power sums of |u|^2
-    double *mom_part = nullptr;   // [nprob][kMomBlocks][kMomK]
+    double *mom_part = nullptr;   // [nprob][blocks][kMomK], max(nprob, kMomBlocks) rows in all
     double2 *hm64 = nullptr;      // [nprob][K] monomial-basis coefficients / transformed right-hand sides
     // single problem: explicit inverse of the Cholesky factor for the solves
     double2 *Linv = nullptr;      // K x K

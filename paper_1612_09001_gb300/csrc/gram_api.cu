@@ -48,7 +48,7 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
         ok = ok && grow(w.norm_part, 0, (size_t)2 * dpd::kFwdNormSlots + 3) &&
              cudaMemset(w.norm_part, 0, ((size_t)2 * dpd::kFwdNormSlots + 3) * sizeof(double)) == cudaSuccess;
         ok = ok && grow(w.ubasis, 0, np * dpd::kUSize) && grow(w.ubasis64, 0, np * dpd::kUSize);
-        ok = ok && grow(w.mom, 0, np * dpd::kMomK) && grow(w.mom_part, 0, np * dpd::kMomBlocks * dpd::kMomK);
+        ok = ok && grow(w.mom, 0, np * dpd::kMomK) && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         ok = ok && grow(w.hm64, 0, np * K);
         ok = ok && grow(w.Linv, 0, (size_t)K * K) && grow(w.tmpv, 0, (size_t)K);
         if (!ok) return DPD_ERR_ALLOC;
@@ -99,8 +99,8 @@ dpd_status compute_basis(dpd_handle h, const std::vector<int64_t> &n, cudaStream
 {
     EstimateWorkspace &w = h->est;
     const int nprob = (int)n.size(), B = h->B;
-    if (dpd::launch_moments(static_cast<const dpd::GramProblem *>(w.probs), nprob, w.mom_part, w.mom, s) !=
-        cudaSuccess)
+    if (dpd::launch_moments(static_cast<const dpd::GramProblem *>(w.probs), nprob, *std::max_element(n.begin(), n.end()), B,
+                            w.mom_part, w.mom, s) != cudaSuccess)
         return DPD_ERR_CUDA;
     std::vector<double> mom((size_t)nprob * dpd::kMomK);
     if (cudaMemcpyAsync(mom.data(), w.mom, sizeof(double) * mom.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -4,6 +4,7 @@
 // kernels of the iterative refinement.
 #include <cooperative_groups.h>
 
+#include "dpd_device.cuh"
 #include "dpd_gram.cuh"
 
 namespace dpd {
@@ -52,59 +53,101 @@ cudaError_t launch_gram_reduce(const float *partials, int nprob, int cpp, int D,
     return cudaGetLastError();
 }
 
-// Each thread sums its powers as FP32 pairs (sum, rounding error) with an
-// exact two-sum per addition: FP32 arithmetic, about 2^-48 relative accuracy,
-// where FP64 additions (about two per clock per SM on GB300) bound the kernel.
-// The pairs become FP64 for the block's fixed-order tree.
-__global__ void moments_kernel(const GramProblem *__restrict__ probs, double *__restrict__ part)
+// Power sums of r = |u|^2, NK = 2 B - 1 of them.  Each thread sums its powers as
+// FP32 pairs (sum, rounding error) with an exact two-sum per addition: FP32
+// arithmetic, about 2^-48 relative accuracy, where FP64 additions (about two per
+// clock per SM on GB300) bound the kernel.  The pairs stay FP32 up to the warp's
+// sum and become FP64 there (before it, if that sum leaves FP32's range).  Eight FP32 operations per sample and power bound
+// it, and the block's sum costs a thread as much as 16 samples: three blocks per
+// SM, four samples' loads in flight per thread.
+// GB300, 2^22 samples, NK = 11: 23.5 us (64 blocks, one load at a time and an
+// FP64 tree per block: 138.4).
+constexpr int kMomThreads = 256;
+
+template <int NK>
+__global__ void __launch_bounds__(kMomThreads) moments_kernel(const GramProblem *__restrict__ probs,
+                                                              double *__restrict__ part)
 {
     const GramProblem pr = probs[blockIdx.y];
-    float hi[kMomK], lo[kMomK];
+    float2 sum[NK];   // (sum, error)
 #pragma unroll
-    for (int k = 0; k < kMomK; ++k) {
-        hi[k] = 0.f;
-        lo[k] = 0.f;
-    }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pr.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 x = pr.u[i];
-        const float r = fmaf(x.x, x.x, x.y * x.y);
-        float p = r;
+    for (int k = 0; k < NK; ++k) sum[k] = make_float2(0.f, 0.f);
+    const int64_t stride = (int64_t)gridDim.x * kMomThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * kMomThreads + threadIdx.x; i0 < pr.n; i0 += 4 * stride) {
+        float2 x[4];
 #pragma unroll
-        for (int k = 0; k < kMomK; ++k) {
-            const float t = hi[k] + p, z = t - hi[k];
-            lo[k] += (hi[k] - (t - z)) + (p - z);
-            hi[k] = t;
-            p *= r;
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            x[q] = i < pr.n ? pr.u[i] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float r = fmaf(x[q].x, x[q].x, x[q].y * x[q].y);
+            float p = r;
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+                two_sum_acc(sum[k].x, sum[k].y, p);
+                p *= r;
+            }
         }
     }
-    __shared__ double red[kMomK][256];
+    __shared__ double red[kMomThreads / 32][NK];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < kMomK; ++k) red[k][threadIdx.x] = (double)hi[k] + (double)lo[k];
-    __syncthreads();
-    for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-        if ((int)threadIdx.x < stride)
+    for (int k = 0; k < NK; ++k) {
+        float2 v = sum[k];
 #pragma unroll
-            for (int k = 0; k < kMomK; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + stride];
-        __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) v = pair_add(v, shfl_xor_pair(v, o));
+        double d = (double)v.x + (double)v.y;
+        if (__any_sync(0xffffffffu, !isfinite(v.x))) {
+            d = (double)sum[k].x + (double)sum[k].y;
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        }
+        if (lane == 0) red[warp][k] = d;
     }
-    if (threadIdx.x < kMomK)
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kMomK + threadIdx.x] = red[threadIdx.x][0];
+    __syncthreads();
+    if (threadIdx.x < NK) {
+        double d = red[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < kMomThreads / 32; ++w) d += red[w][threadIdx.x];
+        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kMomK + threadIdx.x] = d;
+    }
 }
 
-__global__ void moments_sum_kernel(const double *__restrict__ part, int blocks, double *__restrict__ mom)
+// One warp per power: lane l adds blocks l, l + 32, ... in order, then a fixed
+// shuffle tree.  Powers past nk are zero.
+__global__ void __launch_bounds__(32 * kMomK) moments_sum_kernel(const double *__restrict__ part, int blocks, int nk,
+                                                                 double *__restrict__ mom)
 {
-    const int p = blockIdx.x, k = threadIdx.x;
-    if (k >= kMomK) return;
+    const int p = blockIdx.x, k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += part[((size_t)p * blocks + b) * kMomK + k];
-    mom[(size_t)p * kMomK + k] = s;
+    if (k < nk) {
+#pragma unroll 4
+        for (int b = lane; b < blocks; b += 32) s += part[((size_t)p * blocks + b) * kMomK + k];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) mom[(size_t)p * kMomK + k] = s;
 }
 
-cudaError_t launch_moments(const GramProblem *probs, int nprob, double *part, double *mom, cudaStream_t s)
+cudaError_t launch_moments(const GramProblem *probs, int nprob, int64_t nmax, int B, double *part, double *mom,
+                           cudaStream_t s)
 {
-    moments_kernel<<<dim3(kMomBlocks, nprob), 256, 0, s>>>(probs, part);
+    // At least a thousand samples (four per thread) a block.
+    const int64_t need = (nmax + 4 * kMomThreads - 1) / (4 * kMomThreads);
+    const int blocks = (int)(need < moments_blocks(nprob) ? need : moments_blocks(nprob));
+    const dim3 grid((unsigned)blocks, (unsigned)nprob);
+    switch (B) {
+    case 1: moments_kernel<1><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 2: moments_kernel<3><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 3: moments_kernel<5><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 4: moments_kernel<7><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 5: moments_kernel<9><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 6: moments_kernel<11><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    default: return cudaErrorInvalidValue;
+    }
     count_launch();
-    moments_sum_kernel<<<nprob, 32, 0, s>>>(part, kMomBlocks, mom);
+    moments_sum_kernel<<<nprob, 32 * kMomK, 0, s>>>(part, blocks, 2 * B - 1, mom);
     count_launch();
     return cudaGetLastError();
 }
