@@ -230,6 +230,18 @@ dpd_status dpd_sq_error(dpd_handle h, const void *y, const void *x, int64_t n, f
                         double scale, float *loss, void *gy, void *stream);
 
 /*
+ * One Adam step (Kingma and Ba, Algorithm 1; no weight decay) of n float
+ * parameters on the device, for coefficient vectors trained by direct learning:
+ *   t = ++step, m = beta1 m + (1 - beta1) grad, v = beta2 v + (1 - beta2) grad^2,
+ *   param -= lr / (1 - beta1^t) * m / (sqrt(v / (1 - beta2^t)) + eps),
+ * FP64 arithmetic between FP32 loads and stores.  step and lr: one device float
+ * each (a captured step reads the current values).  One block: meant for up to a
+ * few thousand parameters.  Allocation-free and capturable.
+ */
+dpd_status dpd_adam_step(float *param, const float *grad, float *m, float *v, float *step, int64_t n, const float *lr,
+                         double beta1, double beta2, double eps, void *stream);
+
+/*
  * Launch shape of dpd_apply for this handle (used by the autotuner):
  *   mode        bit 0: coefficients passed by value as kernel parameters (used
  *               only after dpd_set_coeffs from host memory; otherwise ignored);

@@ -19,8 +19,9 @@ __device__ __forceinline__ float2 coef_f32(const double2 *h, int i)
 // table tab + x * tstride (0 for a single table).
 template <typename H>
 __global__ void wl_table_kernel(const H *__restrict__ hin, int Bp, int Bq, int T, int B, float *__restrict__ tab,
-                                float *__restrict__ adj, int hstride = 0, int tstride = 0)
+                                float *__restrict__ adj, int hstride, int tstride)
 {
+    grid_dep_wait();
     hin += (size_t)blockIdx.x * hstride;
     tab += (size_t)blockIdx.x * tstride;
     auto h = [hin](int i) { return coef_f32(hin, i); };
@@ -54,26 +55,21 @@ cudaError_t launch_wl_table(const float2 *h, int Bp, int Bq, int T, float *tab, 
                             cudaStream_t s)
 {
     const int B = Bp > Bq ? Bp : Bq;
-    wl_table_kernel<float2><<<1, 64, 0, s>>>(h, Bp, Bq, T, B, tab, adj_tab);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(wl_table_kernel<float2>, dim3(1), 64, 0, s, h, Bp, Bq, T, B, tab, adj_tab, 0, 0);
 }
 
 cudaError_t launch_wl_table_f64(const double2 *h, int Bp, int Bq, int T, float *tab, cudaStream_t s)
 {
     const int B = Bp > Bq ? Bp : Bq;
-    wl_table_kernel<double2><<<1, 64, 0, s>>>(h, Bp, Bq, T, B, tab, nullptr);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(wl_table_kernel<double2>, dim3(1), 64, 0, s, h, Bp, Bq, T, B, tab, nullptr, 0, 0);
 }
 
 cudaError_t launch_wl_table_f64_many(const double2 *h, int count, int hstride, int Bp, int Bq, int T, float *tab,
                                      int tstride, cudaStream_t s)
 {
     const int B = Bp > Bq ? Bp : Bq;
-    wl_table_kernel<double2><<<count, 64, 0, s>>>(h, Bp, Bq, T, B, tab, nullptr, hstride, tstride);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(wl_table_kernel<double2>, dim3((unsigned)count), 64, 0, s, h, Bp, Bq, T, B, tab, nullptr, hstride,
+                      tstride);
 }
 
 // One warp per coefficient: lane t sums rows t, t + 32, ... in order (up to four

@@ -162,7 +162,7 @@ dpd_status dpd_create(int P, int Q, int M, dpd_handle *out)
         cudaMalloc(&f->d_partials, sizeof(float2) * (size_t)f->rows_max * f->K) != cudaSuccess ||
         cudaMalloc(&f->d_status, sizeof(int)) != cudaSuccess ||
         cudaMalloc(&f->d_hist, sizeof(float2) * dpd::kHalo) != cudaSuccess ||
-        cudaMalloc(&f->d_loss_part, sizeof(double) * dpd::kLossBlocks) != cudaSuccess) {
+        cudaMalloc(&f->d_loss_part, sizeof(double) * (dpd::kLossBlocks + 1)) != cudaSuccess) {
         dpd_destroy(f);
         return DPD_ERR_ALLOC;
     }
@@ -173,7 +173,8 @@ dpd_status dpd_create(int P, int Q, int M, dpd_handle *out)
         return DPD_ERR_ALLOC;
     }
     if (cudaMemset(f->d_status, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(f->d_hist, 0, sizeof(float2) * dpd::kHalo) != cudaSuccess) {
+        cudaMemset(f->d_hist, 0, sizeof(float2) * dpd::kHalo) != cudaSuccess ||
+        cudaMemset(f->d_loss_part, 0, sizeof(double) * (dpd::kLossBlocks + 1)) != cudaSuccess) {
         dpd_destroy(f);
         return DPD_ERR_CUDA;
     }
@@ -234,6 +235,17 @@ bool param_tables(dpd_handle h, cudaStream_t s)
 
 }  // namespace
 
+// Whether p is device memory of `device`.
+static bool on_device(const void *p, int device)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+
 dpd_status dpd_num_coeffs(dpd_handle h, int *K)
 {
     if (!h || !K) return DPD_ERR_INVALID_ARGUMENT;
@@ -254,7 +266,7 @@ dpd_status dpd_set_coeffs(dpd_handle h, const void *coeffs, int K, int where, vo
         src = h->d_h;
     } else if (!aligned(coeffs, 8)) {
         return DPD_ERR_INVALID_ARGUMENT;
-    } else if (src != h->d_h) {
+    } else if (!on_device(src, h->device)) {   // the table kernel reads this device's memory in place
         cudaError_t e = cudaMemcpyAsync(h->d_h, coeffs, sizeof(float2) * K, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return DPD_ERR_CUDA;
         src = h->d_h;
@@ -597,6 +609,16 @@ dpd_status dpd_sq_error(dpd_handle h, const void *y, const void *x, int64_t n, f
     return cuda_status(dpd::launch_sq_error(static_cast<const float2 *>(y), static_cast<const float2 *>(x), n,
                                             make_float2(gain_re, gain_im), scale, h->d_loss_part, loss,
                                             static_cast<float2 *>(gy), static_cast<cudaStream_t>(stream)));
+}
+
+dpd_status dpd_adam_step(float *param, const float *grad, float *m, float *v, float *step, int64_t n, const float *lr,
+                         double beta1, double beta2, double eps, void *stream)
+{
+    if (n < 0 || !step || !lr || !aligned(step, 4) || !aligned(lr, 4)) return DPD_ERR_INVALID_ARGUMENT;
+    for (const void *q : {(const void *)param, (const void *)grad, (const void *)m, (const void *)v})
+        if ((n > 0 && !q) || !aligned(q, 4)) return DPD_ERR_INVALID_ARGUMENT;
+    return cuda_status(dpd::launch_adam(param, grad, m, v, step, n, lr, beta1, beta2, eps,
+                                        static_cast<cudaStream_t>(stream)));
 }
 
 dpd_status dpd_reset_stream(dpd_handle h, void *stream)

@@ -22,8 +22,9 @@ import math
 import time
 
 import torch
+from torch.optim.optimizer import _global_optimizer_post_hooks, _global_optimizer_pre_hooks
 
-from . import DPD
+from . import DPD, _lib, _stream_ptr, lib
 from .autograd import DPDFunction
 
 
@@ -41,7 +42,8 @@ class SqErrorLoss(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gl):
         (gy,) = ctx.saved_tensors
-        return gy * gl, None, None, None, None
+        # real by real: the complex product's kernel takes twice as long
+        return torch.view_as_complex(torch.view_as_real(gy) * gl), None, None, None, None
 
 
 class Transmitter:
@@ -109,11 +111,38 @@ class DirectLearner:
         y = self.tx(DPDFunction.apply(self.x, self.h, self.filt))
         return SqErrorLoss.apply(y, self.x, self.filt, self.gain, self.scale)
 
+    def _adam_step(self):
+        """self.opt.step(), as one launch of the library's kernel on the optimiser's own
+        state where nothing but the plain update is asked for: no hooks, schedulers or
+        options of torch's optimiser that the kernel does not have, and the state laid
+        down by an earlier step."""
+        opt, p = self.opt, self.param
+        g = opt.param_groups[0]
+        st = opt.state.get(p)
+        tensors = [p, p.grad, g["lr"]] + ([st["step"], st["exp_avg"], st["exp_avg_sq"]] if st else [])
+        plain = (st and type(opt) is torch.optim.Adam and "step" not in vars(opt) and len(opt.param_groups) == 1
+                 and len(g["params"]) == 1 and g["params"][0] is p
+                 and not (g["weight_decay"] or g["amsgrad"] or g["maximize"] or g["differentiable"])
+                 and not (opt._optimizer_step_pre_hooks or opt._optimizer_step_post_hooks
+                          or _global_optimizer_pre_hooks or _global_optimizer_post_hooks)
+                 and all(isinstance(b, float) for b in (*g["betas"], g["eps"]))
+                 and all(isinstance(t, torch.Tensor) and t.device == p.device and t.dtype == torch.float32
+                         and t.is_contiguous() for t in tensors))
+        if not plain:
+            opt.step()
+            return
+        with torch.no_grad():
+            _lib.check("dpd_adam_step", lib().dpd_adam_step(
+                p.data_ptr(), p.grad.data_ptr(), st["exp_avg"].data_ptr(), st["exp_avg_sq"].data_ptr(),
+                st["step"].data_ptr(), p.numel(), g["lr"].data_ptr(), *g["betas"], g["eps"], _stream_ptr(None)))
+            for t in (p, st["exp_avg"], st["exp_avg_sq"], st["step"]):
+                torch.autograd.graph.increment_version(t)
+
     def _step(self):
-        self.opt.zero_grad(set_to_none=False)
+        self.opt.zero_grad(set_to_none=True)   # the backward pass hands its gradient over: no clear, no addition
         loss = self.loss()
         loss.backward()
-        self.opt.step()
+        self._adam_step()
         return loss
 
     def capture(self, warmup=3):

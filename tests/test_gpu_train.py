@@ -1,0 +1,90 @@
+"""The kernels of a captured training step: the Adam update against FP64 numpy,
+the loss's block sums at the edges of its blocks, and DirectLearner's route to
+the Adam kernel."""
+import numpy as np
+import pytest
+
+import dpd_synth as synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1612_09001_gb300 as dpd  # noqa: E402
+from paper_1612_09001_gb300 import _lib  # noqa: E402
+from paper_1612_09001_gb300.direct import DirectLearner, Transmitter  # noqa: E402
+
+
+@pytest.mark.parametrize("n", [0, 1, 66, 255, 256, 257, 1000])
+@pytest.mark.parametrize("t0", [0, 1, 6, 4095, 2.5])
+def test_adam_step_against_fp64(n, t0):
+    """One step from count t0 (2.5: not a whole number).  The FP64 result is rounded
+    to FP32 once: half an ulp, doubled for the reference's own rounding."""
+    rng = np.random.default_rng([n, int(10 * t0)])
+    p, g, m = (rng.standard_normal(n).astype(np.float32) for _ in range(3))
+    v = (rng.standard_normal(n) ** 2).astype(np.float32)
+    if n:
+        g[0] = v[0] = m[0] = 0.0   # 0 / (sqrt(0) + eps)
+    lr, b1, b2, eps = np.float32(5e-3), 0.9, 0.999, 1e-8
+    d = [torch.from_numpy(a.copy()).cuda() for a in (p, g, m, v)]
+    step, dlr = torch.tensor(float(t0), device="cuda"), torch.tensor(float(lr), device="cuda")
+    _lib.check("dpd_adam_step", dpd.lib().dpd_adam_step(*[a.data_ptr() for a in d], step.data_ptr(), n, dlr.data_ptr(),
+                                                        b1, b2, eps, torch.cuda.current_stream().cuda_stream))
+    t = t0 + 1.0
+    g64 = g.astype(np.float64)
+    m64 = b1 * m.astype(np.float64) + (1 - b1) * g64
+    v64 = b2 * v.astype(np.float64) + (1 - b2) * g64 * g64
+    p64 = p - float(lr) / (1 - b1 ** t) * m64 / (np.sqrt(v64 / (1 - b2 ** t)) + eps)
+    assert float(step) == np.float32(t)
+    for got, ref in zip((d[0], d[2], d[3]), (p64, m64, v64)):
+        assert np.all(np.abs(got.cpu().numpy() - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-44)
+
+
+@pytest.mark.parametrize("n", [1, 31, 256, 257, 4 * 296 * 256, 4 * 296 * 256 + 1, 300007])
+def test_sq_error_block_edges(n):
+    y, x = synth.ofdm2(n, key=(131, n)), synth.ofdm2(n, key=(132, n))
+    f = dpd.DPD(1, 0, 0)
+    yd, xd = torch.from_numpy(y).cuda(), torch.from_numpy(x).cuda()
+    gy = torch.empty_like(yd)
+    e = y.astype(np.complex128) - (0.95 - 0.02j) * x.astype(np.complex128)
+    for _ in range(2):   # the second call finds the completion counter cleared
+        loss = f.sq_error(yd, xd, gain=0.95 - 0.02j, scale=0.5, gy=gy)
+        ref = 0.5 * np.sum(np.abs(e) ** 2)
+        assert abs(float(loss[0]) - ref) <= 1e-6 * ref
+        assert np.abs(gy.cpu().numpy() - e).max() <= 1e-6 * np.abs(e).max()
+    f.close()
+
+
+@pytest.mark.parametrize("big", [3e19, float("inf")])
+def test_sq_error_outside_fp32_sums(big):
+    """Squares whose FP32 sum overflows are summed in FP64; an infinity stays one."""
+    x = torch.zeros(400000, dtype=torch.complex64, device="cuda")   # four or more samples per thread
+    y = torch.full_like(x, 1e19 if big != float("inf") else 1.0)
+    y[::7777] = big if big == float("inf") else 1e19
+    f = dpd.DPD(1, 0, 0)
+    loss = float(f.sq_error(y, x, scale=1e-6 if big != float("inf") else 1.0)[0])
+    if big == float("inf"):
+        assert loss == float("inf")
+    else:
+        assert abs(loss - 4e37) <= 1e-5 * 4e37   # 4e5 samples of 1e38, scale 1e-6
+    f.close()
+
+
+def test_learner_steps_match_the_optimisers_own():
+    """Steps through the Adam kernel against the same learner held to torch's Adam
+    (a step hook keeps it there): the update is FP32-rounded in both, and eps = 1e-8
+    turns a gradient's rounding into at most lr of a step for a coefficient whose
+    gradient is itself rounding, so the trained coefficients agree to a fraction of lr."""
+    t = synth.synthetic_pa(seed=1)
+    x = torch.from_numpy(synth.ofdm2(1 << 14, key=(133, 0))).cuda()
+    out = []
+    for hooked in (False, True):
+        lr = DirectLearner(x, Transmitter([t["iq"], t["pa"]]), 5, 5, 2, lr=5e-3)
+        if hooked:
+            lr.opt.register_step_post_hook(lambda *a: None)
+        lr.capture()
+        for _ in range(20):
+            lr.step()
+        torch.cuda.synchronize()
+        out.append((lr.h.detach().clone(), float(lr.opt.state[lr.param]["step"])))
+    assert out[0][1] == out[1][1] == 23.0
+    assert float((out[0][0] - out[1][0]).abs().max()) <= 1e-4
