@@ -26,7 +26,7 @@
 // lo, with hi hi + hi lo + lo hi summed in FP32 in tensor memory.  Per-CTA
 // partial sums are added in FP64 in a fixed order and S is filled from them
 // and the last samples of the record.  The K x K system is then equilibrated
-// and factored in FP64 (Cholesky), and refined against the FP32 residual
+// and factored (chol_pair.cu), and refined against the FP32 residual
 // t - Psi h computed by the filter and adjoint kernels.
 #pragma once
 
@@ -120,18 +120,15 @@ cudaError_t launch_basis_transform(const double2 *in, double2 *out, const double
                                    int Bq, int T, int to_monomial, cudaStream_t s);
 // CTAs per row chunk the launch wants for nprob problems of up to n rows.
 int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
-// Equilibrated Cholesky factorisation of every G: D G D = L L^H, D = diag(G)^{-1/2}.
-// L (lower, row-major K x K) and d (K) per problem; info[p] = 0 or the failing pivot + 1.
-cudaError_t launch_chol(const double2 *G, int nprob, int K, double2 *L, double *d, int *info, cudaStream_t s);
+// Equilibrated factorisation of every G: D G D = U Delta U^H, D = diag(G)^{-1/2}, U
+// unit lower triangular, Delta diagonal.  U per problem: K (K + 1) / 2 values packed
+// by rows, each an FP32 pair {re.hi, im.hi, re.lo, im.lo}, with 1 / Delta on the
+// diagonal; d: K per problem; info[p] = 0 or the failing pivot + 1.
+cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, int *status, cudaStream_t s);
 // x = G^{-1} rhs using the factorisation; if accumulate, h += x instead of h = x.
-cudaError_t launch_chol_solve(const double2 *L, const double *d, const int *info, const double2 *rhs, int nprob,
-                              int K, double2 *h, int accumulate, cudaStream_t s);
-// Single problem: Linv = L^{-1} (lower, row-major K x K) of the factorisation,
-// then x = G^{-1} rhs = D Linv^H Linv D rhs as two parallel matrix-vector
-// products (tmp: K values of scratch); both skip a failed factorisation.
-cudaError_t launch_chol_invert(const double2 *L, const int *info, int K, double2 *Linv, cudaStream_t s);
-cudaError_t launch_solve_inverse(const double2 *Linv, const double *d, const int *info, const double2 *rhs, int K,
-                                 double2 *tmp, double2 *h, int accumulate, cudaStream_t s);
+// Skips problems that did not factor.
+cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, const double2 *rhs, int nprob,
+                              int K, double2 *h, int accumulate, int *status, cudaStream_t s);
 // Complex64 copy of the FP64 coefficients.
 cudaError_t launch_h_to_f32(const double2 *h, int n, float2 *out, cudaStream_t s);
 // e = t - y (n samples).

@@ -17,7 +17,8 @@ struct EstimateWorkspace {
     float *partials = nullptr;    // [nprob * cpp][kGramRows][kGramPartCols]
     double *S = nullptr;          // [nprob][kGramS][kGramPartCols]: summed P and Q blocks
     double *Clag = nullptr;       // [nprob][kLagEntries]: summed lag sums (tensor-core Gram)
-    double2 *G = nullptr, *g = nullptr, *L = nullptr, *h64 = nullptr, *delta = nullptr;
+    double2 *G = nullptr, *g = nullptr, *h64 = nullptr, *delta = nullptr;
+    float4 *U = nullptr;          // [nprob][K (K + 1) / 2] factors (launch_chol)
     double *d = nullptr, *tt = nullptr;
     int *info = nullptr;
     float2 *hf = nullptr;         // coefficients of the refinement pass (complex64)
@@ -30,14 +31,10 @@ struct EstimateWorkspace {
     double *mom = nullptr;        // [nprob][kMomK] power sums of |u|^2
     double *mom_part = nullptr;   // [nprob][blocks][kMomK], max(nprob, kMomBlocks) rows in all
     double2 *hm64 = nullptr;      // [nprob][K] monomial-basis coefficients / transformed right-hand sides
-    // single problem: explicit inverse of the Cholesky factor for the solves
-    double2 *Linv = nullptr;      // K x K
-    double2 *tmpv = nullptr;      // K
-    bool use_inverse = false;     // refinement solves through Linv (problem 0 only)
     // pinned host copies read back by dpd_estimate (single problem)
     int hK = 0;                   // K the host buffers were sized for
     double2 *h_G = nullptr;       // Gram matrix G, K x K (condition estimate on the host)
-    double2 *h_Linv = nullptr;    // inverse Cholesky factor of D G D, K x K
+    float4 *h_U = nullptr;        // factor of D G D (launch_chol)
     int *h_info = nullptr;        // pivot status of the factorisation
     double *h_norm = nullptr;     // ||t - Psi h||^2, ||t||^2
     cudaEvent_t ev_G = nullptr;   // h_G has landed
@@ -50,7 +47,7 @@ struct EstimateWorkspace {
     void *badj = nullptr;         // dpd::AdjArgs [problems]
     float2 *bpart = nullptr;      // coefficient-gradient partials, [problems][K]
     size_t bprob_cap = 0, bitems_cap = 0;
-    cudaEvent_t ev_L = nullptr;   // h_info (and h_Linv) have landed
+    cudaEvent_t ev_U = nullptr;   // h_info (and h_U) have landed
 };
 
 // Device staging of dpd_apply_host's copy / compute pipeline, created on first use.

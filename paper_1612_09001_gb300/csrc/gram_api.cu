@@ -18,6 +18,8 @@ namespace {
 
 bool aligned8(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
 
+size_t factor_size(int K) { return (size_t)K * (K + 1) / 2; }   // values of a packed factor
+
 template <class T>
 bool grow(T *&p, size_t have, size_t need)
 {
@@ -40,7 +42,7 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
         ok = ok && grow(reinterpret_cast<dpd::GramProblem *&>(w.probs), 0, np);
         ok = ok && grow(w.partials, 0, parts * dpd::kGramRows * dpd::kGramPartCols);
         ok = ok && grow(w.S, 0, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, 0, np * dpd::kLagEntries);
-        ok = ok && grow(w.G, 0, np * K * K) && grow(w.L, 0, np * K * K);
+        ok = ok && grow(w.G, 0, np * K * K) && grow(w.U, 0, np * factor_size(K));
         ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K) && grow(w.delta, 0, np * K);
         ok = ok && grow(w.d, 0, np * K) && grow(w.tt, 0, np) && grow(w.info, 0, np);
         ok = ok && grow(w.hf, 0, (size_t)K) && grow(w.tab, 0, (size_t)dpd::wl_table_floats(h->B, h->T));
@@ -50,29 +52,28 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
         ok = ok && grow(w.ubasis, 0, np * dpd::kUSize) && grow(w.ubasis64, 0, np * dpd::kUSize);
         ok = ok && grow(w.mom, 0, np * dpd::kMomK) && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         ok = ok && grow(w.hm64, 0, np * K);
-        ok = ok && grow(w.Linv, 0, (size_t)K * K) && grow(w.tmpv, 0, (size_t)K);
         if (!ok) return DPD_ERR_ALLOC;
         w.nprob = nprob;
         w.cpp = cpp;
     }
     if (w.hK != K || !w.h_G) {
         cudaFreeHost(w.h_G);
-        cudaFreeHost(w.h_Linv);
+        cudaFreeHost(w.h_U);
         cudaFreeHost(w.h_info);
         cudaFreeHost(w.h_norm);
         w.h_G = nullptr;
-        w.h_Linv = nullptr;
+        w.h_U = nullptr;
         w.h_info = nullptr;
         w.h_norm = nullptr;
         w.hK = 0;
         if (cudaMallocHost(&w.h_G, sizeof(double2) * K * K) != cudaSuccess ||
-            cudaMallocHost(&w.h_Linv, sizeof(double2) * K * K) != cudaSuccess ||
+            cudaMallocHost(&w.h_U, sizeof(float4) * factor_size(K)) != cudaSuccess ||
             cudaMallocHost(&w.h_info, sizeof(int)) != cudaSuccess ||
             cudaMallocHost(&w.h_norm, 2 * sizeof(double)) != cudaSuccess)
             return DPD_ERR_ALLOC;
         w.hK = K;
     }
-    if (!w.ev_L && cudaEventCreateWithFlags(&w.ev_L, cudaEventDisableTiming) != cudaSuccess) return DPD_ERR_CUDA;
+    if (!w.ev_U && cudaEventCreateWithFlags(&w.ev_U, cudaEventDisableTiming) != cudaSuccess) return DPD_ERR_CUDA;
     if (!w.ev_G && cudaEventCreateWithFlags(&w.ev_G, cudaEventDisableTiming) != cudaSuccess) return DPD_ERR_CUDA;
     if (nsamp > w.nsamp) {
         cudaDeviceSynchronize();
@@ -285,13 +286,9 @@ dpd_status refine_once(dpd_handle h, int p, const float2 *u, const float2 *t, in
             return DPD_ERR_CUDA;
         rhs = w.hm64 + (size_t)p * K;
     }
-    if (w.use_inverse && p == 0) {
-        if (dpd::launch_solve_inverse(w.Linv, w.d, w.info, rhs, K, w.tmpv, w.h64, 1, s) != cudaSuccess)
-            return DPD_ERR_CUDA;
-    } else if (dpd::launch_chol_solve(w.L + (size_t)p * K * K, w.d + (size_t)p * K, w.info + p, rhs, 1, K,
-                                      w.h64 + (size_t)p * K, 1, s) != cudaSuccess) {
+    if (dpd::launch_chol_solve(w.U + p * factor_size(K), w.d + (size_t)p * K, w.info + p, rhs, 1, K,
+                               w.h64 + (size_t)p * K, 1, h->d_status, s) != cudaSuccess)
         return DPD_ERR_CUDA;
-    }
     return DPD_OK;
 }
 
@@ -392,15 +389,15 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
                 return DPD_ERR_CUDA;
             rhs = w.hm64;
         }
-        if (dpd::launch_chol_solve(w.L, w.d, w.info, rhs, count, K, w.h64, 1, s) != cudaSuccess) return DPD_ERR_CUDA;
+        if (dpd::launch_chol_solve(w.U, w.d, w.info, rhs, count, K, w.h64, 1, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
     }
     return DPD_OK;
 }
 
-// Condition number of A = D G D = L L^H (the equilibrated Gram matrix, D =
+// Condition number of A = D G D = U Delta U^H (the equilibrated Gram matrix, D =
 // diag(G)^{-1/2}) in the 2-norm: the largest eigenvalue of A (products with A
-// itself, formed from G) times the largest eigenvalue of A^{-1} = L^{-H} L^{-1}
-// (products with the explicit inverse of L that the solves use), FP64 on the
+// itself, formed from G) times the largest eigenvalue of A^{-1} =
+// U^{-H} Delta^{-1} U^{-1} (two triangular solves with the factor), FP64 on the
 // host.  Complex vectors and matrices are kept as separate real and imaginary
 // arrays, padded to an even length N with zeros, and processed two elements
 // at a time with GCC vector types (portable across x86-64 and AArch64): every
@@ -427,18 +424,15 @@ struct Split {
     const double *i(int row) const { return im.data() + (size_t)row * N; }
 };
 
-// y = M x for the first `rows` rows of M (row-major, padded width N); with
-// `lower`, row i reads columns < i + 1 rounded up to the block (M is zero above
-// its diagonal).  Four rows at a time, so every x element is loaded once per
-// four rows.
-void matvec(const Split &M, int rows, bool lower, const double *xr, const double *xi, double *yr, double *yi)
+// y = M x for the first `rows` rows of M (row-major, padded width N).  Four rows at
+// a time, so every x element is loaded once per four rows.
+void matvec(const Split &M, int rows, const double *xr, const double *xi, double *yr, double *yi)
 {
     const int N = M.N;
     int i = 0;
     for (; i + 4 <= rows; i += 4) {
-        const int kend = lower ? std::min(N, (i + 4 + 1) & ~1) : N;
         v2d sr[4] = {}, si[4] = {};
-        for (int k = 0; k < kend; k += 2) {
+        for (int k = 0; k < N; k += 2) {
             const v2d a = ld2(xr + k), b = ld2(xi + k);
             for (int q = 0; q < 4; ++q) {
                 const v2d mr = ld2(M.r(i + q) + k), mi = ld2(M.i(i + q) + k);
@@ -452,9 +446,8 @@ void matvec(const Split &M, int rows, bool lower, const double *xr, const double
         }
     }
     for (; i < rows; ++i) {
-        const int kend = lower ? std::min(N, (i + 1 + 1) & ~1) : N;
         v2d sr = {0, 0}, si = {0, 0};
-        for (int k = 0; k < kend; k += 2) {
+        for (int k = 0; k < N; k += 2) {
             const v2d a = ld2(xr + k), b = ld2(xi + k), mr = ld2(M.r(i) + k), mi = ld2(M.i(i) + k);
             sr += mr * a - mi * b;
             si += mr * b + mi * a;
@@ -464,23 +457,17 @@ void matvec(const Split &M, int rows, bool lower, const double *xr, const double
     }
 }
 
-// y = M^H z for a lower-triangular M (row-major, padded width N): row by row,
-// y[0 .. i] += conj(M_i,0..i) z_i (independent over the columns).
-void matvec_h_lower(const Split &M, int rows, const double *zr, const double *zi, double *yr, double *yi)
+// One step of a column-oriented triangular solve: y[from .. to) -= m[from .. to) z
+// (m conjugated with `conj`), z an element that is final; independent over the
+// elements of the row m.
+void axpy_row(const double *mr, const double *mi, bool conj, double zr, double zi, int from, int to, double *yr,
+              double *yi)
 {
-    const int N = M.N;
-    for (int k = 0; k < N; k += 2) {
-        st2(yr + k, v2d{0, 0});
-        st2(yi + k, v2d{0, 0});
-    }
-    for (int i = 0; i < rows; ++i) {
-        const v2d a = v2d{zr[i], zr[i]}, b = v2d{zi[i], zi[i]};
-        const int kend = std::min(N, (i + 1 + 1) & ~1);
-        for (int k = 0; k < kend; k += 2) {
-            const v2d mr = ld2(M.r(i) + k), mi = ld2(M.i(i) + k);
-            st2(yr + k, ld2(yr + k) + mr * a + mi * b);
-            st2(yi + k, ld2(yi + k) + mr * b - mi * a);
-        }
+    const v2d a = v2d{zr, zr}, b = v2d{zi, zi}, sg = conj ? v2d{-1.0, -1.0} : v2d{1.0, 1.0};
+    for (int k = from & ~1; k < to; k += 2) {   // M is zero outside [from, to)
+        const v2d r = ld2(mr + k), i = sg * ld2(mi + k);
+        st2(yr + k, ld2(yr + k) - (r * a - i * b));
+        st2(yi + k, ld2(yi + k) - (r * b + i * a));
     }
 }
 
@@ -624,23 +611,34 @@ double largest_dgd(const double2 *G, int K)
             A.i(i)[k] = G[(size_t)i * K + k].y * d[i] * d[k];
         }
     return largest(K, N, [&](const double *vr, const double *vi, double *wr, double *wi) {
-        matvec(A, K, false, vr, vi, wr, wi);
+        matvec(A, K, vr, vi, wr, wi);
     });
 }
 
-// Largest eigenvalue of (L L^H)^{-1} = L^{-H} L^{-1}, from L^{-1} (lower triangle).
-double largest_inverse(const double2 *Linv, int K)
+// Largest eigenvalue of (U Delta U^H)^{-1} from the packed factor (launch_chol):
+// two triangular solves per product, by rows of U^T and of U.
+double largest_inverse(const float4 *Up, int K)
 {
     const int N = (K + 1) & ~1;
-    Split Li(K, N), T(1, N);
-    for (int i = 0; i < K; ++i)
-        for (int k = 0; k <= i; ++k) {
-            Li.r(i)[k] = Linv[(size_t)i * K + k].x;
-            Li.i(i)[k] = Linv[(size_t)i * K + k].y;
+    Split U(K, N), Ut(K, N);
+    std::vector<double> dinv(K);
+    for (int i = 0; i < K; ++i) {
+        const float4 *row = Up + factor_size(i);   // i (i + 1) / 2
+        for (int k = 0; k < i; ++k) {
+            Ut.r(k)[i] = U.r(i)[k] = (double)row[k].x + (double)row[k].z;
+            Ut.i(k)[i] = U.i(i)[k] = (double)row[k].y + (double)row[k].w;
         }
+        dinv[i] = (double)row[i].x + (double)row[i].z;
+    }
     return largest(K, N, [&](const double *vr, const double *vi, double *wr, double *wi) {
-        matvec(Li, K, true, vr, vi, T.r(0), T.i(0));
-        matvec_h_lower(Li, K, T.r(0), T.i(0), wr, wi);
+        std::copy(vr, vr + N, wr);
+        std::copy(vi, vi + N, wi);
+        for (int k = 0; k + 1 < K; ++k) axpy_row(Ut.r(k), Ut.i(k), false, wr[k], wi[k], k + 1, K, wr, wi);
+        for (int i = 0; i < K; ++i) {
+            wr[i] *= dinv[i];
+            wi[i] *= dinv[i];
+        }
+        for (int i = K - 1; i > 0; --i) axpy_row(U.r(i), U.i(i), true, wr[i], wi[i], 0, i, wr, wi);
     });
 }
 
@@ -680,7 +678,7 @@ void free_estimate_workspace(EstimateWorkspace &w)
     cudaFree(w.S);
     cudaFree(w.G);
     cudaFree(w.g);
-    cudaFree(w.L);
+    cudaFree(w.U);
     cudaFree(w.h64);
     cudaFree(w.delta);
     cudaFree(w.d);
@@ -696,18 +694,16 @@ void free_estimate_workspace(EstimateWorkspace &w)
     cudaFree(w.mom);
     cudaFree(w.mom_part);
     cudaFree(w.hm64);
-    cudaFree(w.Linv);
-    cudaFree(w.tmpv);
     cudaFree(w.tabb);
     cudaFree(w.bstreams);
     cudaFree(w.bitems);
     cudaFree(w.badj);
     cudaFree(w.bpart);
     cudaFreeHost(w.h_G);
-    cudaFreeHost(w.h_Linv);
+    cudaFreeHost(w.h_U);
     cudaFreeHost(w.h_info);
     cudaFreeHost(w.h_norm);
-    if (w.ev_L) cudaEventDestroy(w.ev_L);
+    if (w.ev_U) cudaEventDestroy(w.ev_U);
     if (w.ev_G) cudaEventDestroy(w.ev_G);
     w = EstimateWorkspace();
 }
@@ -758,7 +754,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
         if ((st = compute_basis(h, std::vector<int64_t>{n}, s)) != DPD_OK) return st;
     }
     if ((st = run_gram(h, 1, cpp, precision, s, ortho(h) ? nullptr : &pr)) != DPD_OK) return st;
-    // For the statistics, G and (after the factorisation) the inverse factor go
+    // For the statistics, G and (after the factorisation) the factor go
     // to pinned host memory while the device carries on, and so does the pivot
     // status: the host condition estimate (Lanczos on D G D from G, and on its
     // inverse) runs during the factorisation and the refinement instead of
@@ -767,19 +763,14 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if (stats && (cudaMemcpyAsync(w.h_G, w.G, sizeof(double2) * K * K, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                   cudaEventRecord(w.ev_G, s) != cudaSuccess))
         return DPD_ERR_CUDA;
-    if (dpd::launch_chol(w.G, 1, h->K, w.L, w.d, w.info, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol(w.G, 1, h->K, w.U, w.d, w.info, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
     if (cudaMemcpyAsync(w.h_info, w.info, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return DPD_ERR_CUDA;
-    // The solves go through the explicit inverse of L: two parallel
-    // matrix-vector products instead of two K-step sequential chains each.
-    if (dpd::launch_chol_invert(w.L, w.info, K, w.Linv, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if ((stats && cudaMemcpyAsync(w.h_Linv, w.Linv, sizeof(double2) * K * K, cudaMemcpyDeviceToHost, s) !=
+    if ((stats && cudaMemcpyAsync(w.h_U, w.U, sizeof(float4) * factor_size(K), cudaMemcpyDeviceToHost, s) !=
                       cudaSuccess) ||
-        cudaEventRecord(w.ev_L, s) != cudaSuccess)
+        cudaEventRecord(w.ev_U, s) != cudaSuccess)
         return DPD_ERR_CUDA;
-    w.use_inverse = true;
-    if (dpd::launch_solve_inverse(w.Linv, w.d, w.info, w.g, K, w.tmpv, w.h64, 0, s) != cudaSuccess)
-        return DPD_ERR_CUDA;
+    if (dpd::launch_chol_solve(w.U, w.d, w.info, w.g, 1, K, w.h64, 0, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
     for (int i = 0; i < refine_iters; ++i)
         if ((st = refine_once(h, 0, pr.u, pr.t, n, s)) != DPD_OK) return st;
     const double2 *hm = monomial_h(h, 0, 1, s, st);
@@ -788,7 +779,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if (stats && (st = queue_norms(h, 0, pr.u, pr.t, n, s)) != DPD_OK) return st;
     // The two Lanczos runs overlap the queued device work: the one on D G D
     // (a second host thread) as soon as G has landed, the one on the inverse
-    // once the inverse factor has.
+    // once the factor has.
     double lmax = 0.0, linv = 0.0;
     std::thread dgd_run;
     bool threaded = false;
@@ -800,9 +791,9 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
         } catch (const std::system_error &) {   // no thread available: on this one, below
         }
     }
-    const bool synced = cudaEventSynchronize(w.ev_L) == cudaSuccess;
+    const bool synced = cudaEventSynchronize(w.ev_U) == cudaSuccess;
     const int info = synced ? *w.h_info : 0;
-    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_Linv, K);
+    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_U, K);
     if (threaded) dgd_run.join();
     if (!synced) return DPD_ERR_CUDA;
     if (stats && !threaded) lmax = cond::largest_dgd(w.h_G, K);
@@ -844,9 +835,8 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
         return DPD_ERR_CUDA;
     if (ortho(h) && (st = compute_basis(h, std::vector<int64_t>(n, n + count), s)) != DPD_OK) return st;
     if ((st = run_gram(h, count, cpp, precision, s)) != DPD_OK) return st;
-    if (dpd::launch_chol(w.G, count, h->K, w.L, w.d, w.info, s) != cudaSuccess) return DPD_ERR_CUDA;
-    w.use_inverse = false;
-    if (dpd::launch_chol_solve(w.L, w.d, w.info, w.g, count, h->K, w.h64, 0, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol(w.G, count, h->K, w.U, w.d, w.info, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol_solve(w.U, w.d, w.info, w.g, count, h->K, w.h64, 0, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
     // The pivot status comes back here only for the refinement problem by
     // problem, which skips problems that did not factor; refined together, the
     // launches are queued behind the solve without a host round trip and the

@@ -1,0 +1,88 @@
+"""The pair factorisation and solves behind the least-squares estimates, at the
+edges of their panels and row groups, and the problems left to the FP64 kernel."""
+import numpy as np
+import pytest
+
+import dpd_synth as synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1612_09001_gb300 as dpd  # noqa: E402
+
+
+def _fit(P, Q, M, n, seed, precision="fp32"):
+    """(h, G^{-1} g in FP64 from the library's own G and g): without refinement the
+    estimate is the solve alone."""
+    u = torch.from_numpy(synth.clipped_gaussian(n, 0.3, key=(140, seed))).cuda()
+    h0 = synth.coeffs(P, Q, M, key=(141, seed))
+    f = dpd.DPD(P, Q, M)
+    f.set_coeffs(h0)
+    t = f.apply(u)
+    h, st = f.estimate(u, t, precision=precision, refine_iters=0)
+    G, g, _ = f.gram(u, t, precision=precision)
+    hb, info = f.estimate_batched([u] * 9, [t] * 9, precision=precision, refine_iters=0)
+    f.close()
+    assert info == [0] * 9
+    G, g = G.cpu().numpy(), g.cpu().numpy()
+    d = 1.0 / np.sqrt(np.real(np.diag(G)))
+    A = G * d[:, None] * d[None, :]
+    return h.cpu().numpy(), hb.cpu().numpy(), d * np.linalg.solve(A, d * g), np.linalg.cond(A), st
+
+
+@pytest.mark.parametrize("P,Q,M", [(1, 0, 0), (1, 1, 1), (3, 0, 1), (5, 3, 0), (3, 3, 2), (7, 0, 7), (7, 7, 3), (5, 5, 5),
+                                   (9, 0, 7), (7, 7, 7), (9, 9, 6), (11, 11, 7)])
+def test_solve_at_panel_edges(P, Q, M):
+    """K - 1 = 1 .. 96: part panels, whole panels, one row group and one past it.  The
+    error of the solve is cond(A) times the factorisation's backward error, below
+    2^-38 (element error 2^-42, at most 97 of them), and the FP32 rounding of h.  The
+    nine problems of the batch sum their Gram matrix over fewer CTAs: the same result
+    for each, within cond(A) times the FP32 Gram's 2e-6 of the single fit's."""
+    h, hb, ref, cond, st = _fit(P, Q, M, 40000, P + 16 * M)
+    err = np.linalg.norm(h - ref) / np.linalg.norm(ref)
+    print(f"K {len(ref)} cond {cond:.2e} error {err:.2e} batch {np.linalg.norm(hb[0] - ref):.2e}")
+    assert err <= cond * 2.0 ** -38 + 2.0 ** -23, (P, Q, M, cond)
+    assert all(np.array_equal(hb[0], v) for v in hb[1:])
+    assert np.linalg.norm(hb[0] - ref) <= (cond * 2e-6 + 2.0 ** -23) * np.linalg.norm(ref), (P, Q, M, cond)
+    assert abs(st["cond_est"] - cond) <= (1e-6 + cond * 2.0 ** -38) * cond
+
+
+def test_scales_at_the_edge_of_fp32():
+    """Samples of 1e-16 (no constant in the target): Gram entries of 1e-29 to 1e-32
+    beside the constant column's, split by their bits or through FP64 on either side of
+    the limits, to the same coefficients."""
+    n = 20000
+    u0 = synth.clipped_gaussian(n, 0.3, key=(142, 0))
+    f = dpd.DPD(1, 1, 3)
+    h0 = synth.coeffs(1, 1, 3, key=(142, 1))
+    h0[-1] = 0.0
+    f.set_coeffs(h0)
+    res = []
+    for scale in (1.0, 1e-16):
+        u = torch.from_numpy((u0 * np.float32(scale)).astype(np.complex64)).cuda()
+        t = f.apply(u)
+        h, _ = f.estimate(u, t, precision="fp32", refine_iters=2)
+        res.append(h.cpu().numpy()[:-1])
+    f.close()
+    assert np.linalg.norm(res[0] - res[1]) <= 1e-4 * np.linalg.norm(res[0])
+
+
+def test_collinear_columns_go_to_fp64():
+    """A real-valued input makes the two branches' columns equal: pivots at rounding
+    level, below the pair kernel's limit.  Whatever the FP64 kernel decides, the call
+    returns as for any other fit (a status, or coefficients)."""
+    n = 20000
+    u = torch.from_numpy(np.abs(synth.clipped_gaussian(n, 0.3, key=(143, 0))).astype(np.complex64)).cuda()
+    f = dpd.DPD(3, 3, 1)
+    try:
+        h, st = f.estimate(u, u, precision="fp32", refine_iters=0)
+        assert h.numel() == f.K and st["cond_est"] > 1e6
+    except dpd.DPDError as e:
+        assert e.code == 6
+    good = torch.from_numpy(synth.clipped_gaussian(n, 0.3, key=(143, 1))).cuda()
+    hb, info = f.estimate_batched([good, u, good], [good, u, good], precision="fp32", refine_iters=0)
+    assert info[0] == 0 and info[2] == 0
+    e0 = np.zeros(f.K)
+    e0[0] = 1.0
+    assert np.abs(hb[0].cpu().numpy() - e0).max() <= 1e-3 and np.array_equal(hb[0].cpu().numpy(), hb[2].cpu().numpy())
+    f.close()
