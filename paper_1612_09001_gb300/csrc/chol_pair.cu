@@ -12,6 +12,7 @@
 
 #include "dpd_device.cuh"
 #include "dpd_gram.cuh"
+#include "dpd_table.cuh"
 
 namespace dpd {
 
@@ -122,23 +123,9 @@ __device__ __noinline__ float4 scaled_fp64(double2 g, double s)
     return make_float4(re.x, im.x, re.y, im.y);
 }
 
-// 1/sqrt(x) for x in (1e-30, 1e30): the FP32 hardware estimate refined by two
-// Newton-Raphson steps y <- y (3 - x y^2) / 2 in FP64.
-__device__ __forceinline__ double rsqrt_newton(double x)
-{
-    double y = (double)rsqrtf((float)x);
-    const double hx = 0.5 * x;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double q = hx * y;
-        const double e = fma(-q, y, 0.5);   // 1/2 - x y^2 / 2
-        y = fma(y, e, y);
-    }
-    return y;
-}
 __device__ __forceinline__ double equilibration(double g)   // g^{-1/2}, or 0
 {
-    return g > 1e-30 && g < 1e30 ? rsqrt_newton(g) : g > 0.0 ? 1.0 / sqrt(g) : 0.0;
+    return g > 0.0 ? inv_sqrt(g) : 0.0;
 }
 
 // NG: row groups of 32, and rounds of panels (columns 32 c + 4 warp + q).
@@ -433,7 +420,7 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
             if (!(piv > 1e-30 && piv < 1e30)) {   // not positive definite (or numerically singular)
                 bad = j + 1;
             } else {
-                const double ri = rsqrt_newton(piv);
+                const double ri = inv_sqrt(piv);
                 A[tri_row(j) + j] = make_double2(piv * ri, 0.0);
                 rinv = ri;
             }
@@ -573,6 +560,24 @@ __device__ __forceinline__ float4 row_sum(const CPair &v)
     }
     return make_float4(re.x, im.x, re.y, im.y);
 }
+// Element j of a coefficient vector in the other basis (both branches, every tap; the
+// constant unchanged), U upper triangular with rows of kMaxB:
+//   MONOMIAL:  h[(a, k)] = sum_{b >= a} U[a][b] h_U[(b, k)]    (W h)
+//   otherwise: g_U[(a, k)] = sum_{c <= a} U[c][a] g[(c, k)]    (W^T g, right-hand sides)
+template <bool MONOMIAL>
+__device__ __forceinline__ double2 basis_transform(const double2 *x, const double *U, int j, int K, int Bp, int Bq, int T)
+{
+    if (j == K - 1) return x[j];
+    const bool conj = j >= Bp * T;
+    const int base = conj ? Bp * T : 0, nb = conj ? Bq : Bp, jj = j - base, a = jj / T, k = jj % T;
+    double2 v = make_double2(0.0, 0.0);
+    for (int b = MONOMIAL ? a : 0; b < (MONOMIAL ? nb : a + 1); ++b) {
+        const double u = MONOMIAL ? U[a * kMaxB + b] : U[b * kMaxB + a];
+        v.x += u * x[base + b * T + k].x;
+        v.y += u * x[base + b * T + k].y;
+    }
+    return v;
+}
 __device__ __forceinline__ float4 cpair_add(const float4 &a, const float4 &b)
 {
     const float2 re = pair_add(make_float2(a.x, a.z), make_float2(b.x, b.z));
@@ -583,12 +588,13 @@ __device__ __forceinline__ float4 cpair_add(const float4 &a, const float4 &b)
 
 __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restrict__ Uall,
                                                          const double *__restrict__ dall,
-                                                         const int *__restrict__ info,
-                                                         const double2 *__restrict__ rhs, int K,
-                                                         double2 *__restrict__ h, int accumulate, int *status)
+                                                         const int *__restrict__ info, int K, SolveIo io,
+                                                         int *status)
 {
     extern __shared__ __align__(128) float4 Us[];   // U, lower triangle packed by rows (tri_row), 1 / pivots on the diagonal
     __shared__ float4 w[kCholMaxK];
+    __shared__ double2 mono[kCholMaxK];      // a vector before and after a change of basis
+    __shared__ float4 part[8][kCholMaxK];    // sums of rows by warp
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) {
         mbar_init(smem_addr(&bar), 1);
@@ -602,13 +608,45 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     if (info[p] != 0) return;   // uniform over the CTA
     const float4 *U = Uall + (size_t)p * tri_row(K);
     const double *d = dall + (size_t)p * K;
-    const double2 *b = rhs + (size_t)p * K;
+    const double *W = io.basis ? io.basis + (size_t)p * kUSize : nullptr;
     if (tid == 0) {   // the whole factor in one bulk copy
         mbar_arrive_expect_tx(smem_addr(&bar), (uint32_t)(tri_row(K) * sizeof(float4)));
         bulk_copy_g2s(smem_addr(Us), U, (uint32_t)(tri_row(K) * sizeof(float4)), smem_addr(&bar));
     }
+    if (io.rows) {
+        // Warp w adds rows w, w + 8, ..., in order, as exact pairs (about 2^-48); thread i
+        // then adds the eight sums of coefficient i.
+        const float2 *rows = io.rows + (size_t)p * io.nrows * K;
+        CPair acc[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 8
+        for (int r = warp; r < io.nrows; r += 8)
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (lane + 32 * m < K) {
+                    const float2 v = rows[(size_t)r * K + lane + 32 * m];
+                    two_sum_acc(acc[m].h.x, acc[m].l.x, v.x);
+                    two_sum_acc(acc[m].h.y, acc[m].l.y, v.y);
+                }
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (lane + 32 * m < K)
+                part[warp][lane + 32 * m] = make_float4(acc[m].h.x, acc[m].h.y, acc[m].l.x, acc[m].l.y);
+        __syncthreads();
+        if (tid < K) {
+            float4 v = part[0][tid];
+#pragma unroll
+            for (int q = 1; q < 8; ++q) v = cpair_add(v, part[q][tid]);
+            mono[tid] = make_double2(to_double(v.x, v.z), to_double(v.y, v.w));
+        }
+        __syncthreads();
+    }
     if (tid < K) {
-        const float2 re = to_pair(b[tid].x * d[tid]), im = to_pair(b[tid].y * d[tid]);
+        const double2 v = !io.rows ? io.rhs[(size_t)p * K + tid]
+                          : W      ? basis_transform<false>(mono, W, tid, K, io.Bp, io.Bq, io.T)
+                                   : mono[tid];
+        const float2 re = to_pair(v.x * d[tid]), im = to_pair(v.y * d[tid]);
         w[tid] = make_float4(re.x, im.x, re.y, im.y);
     }
     if (!mbar_wait(smem_addr(&bar), 0u, status)) {   // the copy lands before the CTA leaves, within the limit
@@ -691,23 +729,37 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
         }
         __syncthreads();
     }
-    double2 *out = h + (size_t)p * K;
     if (tid < K) {
         const float4 v = w[tid];
-        const double2 x = make_double2(to_double(v.x, v.z) * d[tid], to_double(v.y, v.w) * d[tid]);
-        out[tid] = accumulate ? make_double2(out[tid].x + x.x, out[tid].y + x.y) : x;
+        double2 x = make_double2(to_double(v.x, v.z) * d[tid], to_double(v.y, v.w) * d[tid]);
+        double2 *h = io.h + (size_t)p * K + tid;
+        if (io.accumulate) x = make_double2(h->x + x.x, h->y + x.y);
+        *h = x;
+        mono[tid] = x;
     }
+    __syncthreads();
+    // The monomial coefficients in FP32, and their forward table.
+    float2 *hf = reinterpret_cast<float2 *>(w);
+    double2 x = make_double2(0.0, 0.0);
+    if (tid < K) x = W ? basis_transform<true>(mono, W, tid, K, io.Bp, io.Bq, io.T) : mono[tid];
+    if (tid < K) {
+        hf[tid] = make_float2((float)x.x, (float)x.y);
+        io.out[(size_t)p * K + tid] = hf[tid];
+    }
+    __syncthreads();
+    const int B = io.Bp > io.Bq ? io.Bp : io.Bq;
+    wl_table_entry([hf](int i) { return hf[i]; }, tid, io.Bp, io.Bq, io.T, B, io.tab + (size_t)p * io.tstride, nullptr);
 }
 
-cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, const double2 *rhs, int nprob, int K,
-                              double2 *h, int accumulate, int *status, cudaStream_t s)
+cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, int nprob, int K, const SolveIo &io,
+                              int *status, cudaStream_t s)
 {
     if (K < 1 || K > kCholMaxK) return cudaErrorInvalidValue;
     const size_t smem = sizeof(float4) * (size_t)tri_row(K);
     static SmemAttr smem_rec;
     const cudaError_t e = ensure_smem(smem_rec, (const void *)chol_solve_kernel, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(chol_solve_kernel, dim3((unsigned)nprob), 256, smem, s, U, d, info, rhs, K, h, accumulate, status);
+    return launch_pdl(chol_solve_kernel, dim3((unsigned)nprob), 256, smem, s, U, d, info, K, io, status);
 }
 
 }  // namespace dpd

@@ -43,6 +43,20 @@ __device__ __forceinline__ float2 shfl_xor_pair(float2 v, int o)
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
 
+// 1/sqrt(x), x > 0, in FP64: the FP32 hardware estimate refined by two Newton-Raphson
+// steps y <- y (3 - x y^2) / 2 (each squares the relative error: about 2^-22 -> 2^-44 ->
+// FP64 rounding), six FP64 operations on a sequential path instead of a full FP64 square
+// root and division.
+__device__ __forceinline__ double inv_sqrt(double x)
+{
+    if (!(x > 1e-30 && x < 1e30)) return 1.0 / sqrt(x);
+    double y = (double)rsqrtf((float)x);
+    const double hx = 0.5 * x;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(y, fma(-hx * y, y, 0.5), y);
+    return y;
+}
+
 __device__ __forceinline__ uint64_t global_ns()
 {
     uint64_t t;

@@ -100,9 +100,10 @@ cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *pro
 // G (K x K, row-major), g (K) and t^H t per problem from S.
 cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int B, int T, double2 *G, double2 *g,
                                  double *tt, cudaStream_t s);
-// Power sums of r = |u|^2 per problem: mom[p][k - 1] = sum_n r_n^k, k = 1 .. 2 B - 1
-// (zero up to kMomK), in a fixed order: exact FP32 two-sum pairs within a block,
-// then FP64 (part: nprob * moments_blocks(nprob) * kMomK doubles of scratch).
+// Orthonormal basis U of every problem (Sec. 2.1; kUSize per problem, FP32 and the same
+// values in FP64) from the power sums sum_n r_n^k, k = 1 .. 2 B - 1, of r = |u|^2: exact
+// FP32 two-sum pairs within a warp, then FP64, in a fixed order (part: max(nprob,
+// kMomBlocks) * kMomK doubles of scratch).  probs may be null for the one problem `one`;
 // nmax: the longest problem.
 constexpr int kMomK = 2 * kMaxB - 1;
 constexpr int kMomBlocks = 456;   // over all problems: three per SM at 152 SMs
@@ -110,14 +111,8 @@ __host__ __device__ constexpr int moments_blocks(int nprob)   // blocks a proble
 {
     return nprob < kMomBlocks ? kMomBlocks / nprob : 1;
 }
-cudaError_t launch_moments(const GramProblem *probs, int nprob, int64_t nmax, int B, double *part, double *mom,
-                           cudaStream_t s);
-// Coefficient vectors between the monomial basis and the basis U (both
-// branches, every tap; the constant unchanged), per problem:
-//   to_monomial: out = W in       (h = W h_U)
-//   otherwise:   out = W^T in     (g_U = W^T g for right-hand sides)
-cudaError_t launch_basis_transform(const double2 *in, double2 *out, const double *U, int nprob, int K, int Bp,
-                                   int Bq, int T, int to_monomial, cudaStream_t s);
+cudaError_t launch_basis(const GramProblem *probs, GramProblem one, int nprob, int64_t nmax, int B, double *part,
+                         float *ubasis, double *ubasis64, cudaStream_t s);
 // CTAs per row chunk the launch wants for nprob problems of up to n rows.
 int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
 // Equilibrated factorisation of every G: D G D = U Delta U^H, D = diag(G)^{-1/2}, U
@@ -125,22 +120,27 @@ int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
 // by rows, each an FP32 pair {re.hi, im.hi, re.lo, im.lo}, with 1 / Delta on the
 // diagonal; d: K per problem; info[p] = 0 or the failing pivot + 1.
 cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, int *status, cudaStream_t s);
-// x = G^{-1} rhs using the factorisation; if accumulate, h += x instead of h = x.
-// Skips problems that did not factor.
-cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, const double2 *rhs, int nprob,
-                              int K, double2 *h, int accumulate, int *status, cudaStream_t s);
-// Complex64 copy of the FP64 coefficients.
-cudaError_t launch_h_to_f32(const double2 *h, int n, float2 *out, cudaStream_t s);
+// x = G^{-1} rhs using the factorisation (problems that did not factor are skipped).
+// Every pointer: `nprob` consecutive vectors, K apart unless stated.
+struct SolveIo {
+    const double2 *rhs;      // right-hand sides, or null: the sums of ...
+    const float2 *rows;      // ... nrows rows per problem, in the monomial basis
+    int nrows;
+    const double *basis;     // basis U of the system (kUSize per problem), or null: monomials
+    double2 *h;              // x, or h + x with `accumulate`, in that basis
+    int accumulate;
+    float2 *out;             // the monomial coefficients
+    float *tab;              // their forward tables, tstride floats apart
+    int tstride;
+    int Bp, Bq, T;
+};
+cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, int nprob, int K, const SolveIo &io,
+                              int *status, cudaStream_t s);
 // e = t - y (n samples).
 cudaError_t launch_residual(const float2 *t, const float2 *y, int64_t n, float2 *e, cudaStream_t s);
 // e = t - y together with out[0] = sum |e|^2, out[1] = sum |t|^2 in FP64
 // (part: 2 * 1024 doubles of scratch).
 cudaError_t launch_residual_norm(const float2 *t, const float2 *y, int64_t n, float2 *e, double *part, double *out,
                                  cudaStream_t s);
-// Like launch_adj_finalize, summed to FP64.
-cudaError_t launch_adj_finalize64(const float2 *partials, int rows, int K, double2 *out, cudaStream_t s);
-// The same for `count` problems, each with `rows` rows (outputs K apart).
-cudaError_t launch_adj_finalize64_many(const float2 *partials, int rows, int K, int count, double2 *out,
-                                       cudaStream_t s);
 
 }  // namespace dpd

@@ -17,20 +17,17 @@ struct EstimateWorkspace {
     float *partials = nullptr;    // [nprob * cpp][kGramRows][kGramPartCols]
     double *S = nullptr;          // [nprob][kGramS][kGramPartCols]: summed P and Q blocks
     double *Clag = nullptr;       // [nprob][kLagEntries]: summed lag sums (tensor-core Gram)
-    double2 *G = nullptr, *g = nullptr, *h64 = nullptr, *delta = nullptr;
+    double2 *G = nullptr, *g = nullptr, *h64 = nullptr;
     float4 *U = nullptr;          // [nprob][K (K + 1) / 2] factors (launch_chol)
     double *d = nullptr, *tt = nullptr;
     int *info = nullptr;
-    float2 *hf = nullptr;         // coefficients of the refinement pass (complex64)
-    float *tab = nullptr;         // their forward table
+    float *tab = nullptr;         // [nprob][table_stride] forward tables of the current coefficients
     float2 *y = nullptr, *e = nullptr;
     double *norm_part = nullptr;  // 2 * kFwdNormSlots partial sums, 2 results, a counter
     // orthogonal-polynomial basis (DPD_BASIS_ORTHOGONAL)
     float *ubasis = nullptr;      // [nprob][kUSize] basis coefficients used by the Gram kernels
     double *ubasis64 = nullptr;   // the same values in FP64, for the coefficient transforms
-    double *mom = nullptr;        // [nprob][kMomK] power sums of |u|^2
     double *mom_part = nullptr;   // [nprob][blocks][kMomK], max(nprob, kMomBlocks) rows in all
-    double2 *hm64 = nullptr;      // [nprob][K] monomial-basis coefficients / transformed right-hand sides
     // pinned host copies read back by dpd_estimate (single problem)
     int hK = 0;                   // K the host buffers were sized for
     double2 *h_G = nullptr;       // Gram matrix G, K x K (condition estimate on the host)
@@ -38,10 +35,8 @@ struct EstimateWorkspace {
     int *h_info = nullptr;        // pivot status of the factorisation
     double *h_norm = nullptr;     // ||t - Psi h||^2, ||t||^2
     cudaEvent_t ev_G = nullptr;   // h_G has landed
-    // batched refinement (dpd_estimate_batched): per-problem forward tables,
-    // work lists of the batched forward and coefficient-gradient launches
-    float *tabb = nullptr;        // [problems][tstride]
-    size_t tabb_cap = 0;
+    // batched refinement (dpd_estimate_batched): work lists of the batched forward and
+    // coefficient-gradient launches
     void *bstreams = nullptr;     // dpd::BatchStream [problems]
     void *bitems = nullptr;       // dpd::BatchItem [items]
     void *badj = nullptr;         // dpd::AdjArgs [problems]

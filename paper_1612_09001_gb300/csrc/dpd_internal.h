@@ -134,11 +134,6 @@ cudaError_t launch_fwd_any(int B, int T, const FwdArgs &a, const FwdLaunch &L, i
 
 // Build the forward widely-linear table and the adjoint table from the stacked
 // coefficient vector h (K complex); adj_tab may be null.
-// The forward table straight from FP64 coefficients (rounded to FP32 first);
-// _many: `count` problems, coefficients hstride and tables tstride apart.
-cudaError_t launch_wl_table_f64(const double2 *h, int Bp, int Bq, int T, float *tab, cudaStream_t s);
-cudaError_t launch_wl_table_f64_many(const double2 *h, int count, int hstride, int Bp, int Bq, int T, float *tab,
-                                     int tstride, cudaStream_t s);
 cudaError_t launch_wl_table(const float2 *h, int Bp, int Bq, int T, float *tab, float *adj_tab,
                             cudaStream_t s);
 

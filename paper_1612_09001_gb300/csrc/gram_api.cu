@@ -18,6 +18,8 @@ namespace {
 
 bool aligned8(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
 
+// Floats between the forward tables of a batch (16-byte aligned).
+size_t table_stride(dpd_handle h) { return ((size_t)dpd::wl_table_floats(h->B, h->T) + 3) & ~(size_t)3; }
 size_t factor_size(int K) { return (size_t)K * (K + 1) / 2; }   // values of a packed factor
 
 template <class T>
@@ -43,15 +45,14 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
         ok = ok && grow(w.partials, 0, parts * dpd::kGramRows * dpd::kGramPartCols);
         ok = ok && grow(w.S, 0, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, 0, np * dpd::kLagEntries);
         ok = ok && grow(w.G, 0, np * K * K) && grow(w.U, 0, np * factor_size(K));
-        ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K) && grow(w.delta, 0, np * K);
+        ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K);
         ok = ok && grow(w.d, 0, np * K) && grow(w.tt, 0, np) && grow(w.info, 0, np);
-        ok = ok && grow(w.hf, 0, (size_t)K) && grow(w.tab, 0, (size_t)dpd::wl_table_floats(h->B, h->T));
+        ok = ok && grow(w.tab, 0, np * table_stride(h));
         // partial pairs, the two results, the completion counter (zero)
         ok = ok && grow(w.norm_part, 0, (size_t)2 * dpd::kFwdNormSlots + 3) &&
              cudaMemset(w.norm_part, 0, ((size_t)2 * dpd::kFwdNormSlots + 3) * sizeof(double)) == cudaSuccess;
         ok = ok && grow(w.ubasis, 0, np * dpd::kUSize) && grow(w.ubasis64, 0, np * dpd::kUSize);
-        ok = ok && grow(w.mom, 0, np * dpd::kMomK) && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
-        ok = ok && grow(w.hm64, 0, np * K);
+        ok = ok && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         if (!ok) return DPD_ERR_ALLOC;
         w.nprob = nprob;
         w.cpp = cpp;
@@ -88,80 +89,43 @@ bool valid_precision(int p) { return p == DPD_PREC_FP32 || p == DPD_PREC_TF32X3 
 
 bool ortho(dpd_handle h) { return h->est_basis == DPD_BASIS_ORTHOGONAL; }
 
-// Basis of statistically orthogonal polynomials (Sec. 2.1) for every problem
-// in w.probs: with mu_k = sum_n r_n^k (r = |u|^2), the moment matrix
-// M[a][b] = mu_{a+b+1} / n is the Gram matrix of the monomials |u|^{2a} u;
-// M = L L^T (FP64 Cholesky on the host) and U = L^{-T} make
-// sum_a U[a][b] |u|^{2a} u orthonormal.  U is rounded to FP32 for the Gram
-// kernels and the same values are kept in FP64 for the coefficient
-// transforms.  A problem whose moment matrix is not positive definite keeps
-// the monomials (U = I).
-dpd_status compute_basis(dpd_handle h, const std::vector<int64_t> &n, cudaStream_t s)
+// Basis of statistically orthogonal polynomials for the problems in w.probs, or the one
+// problem *one.
+dpd_status compute_basis(dpd_handle h, const dpd::GramProblem *one, int nprob, int64_t nmax, cudaStream_t s)
 {
     EstimateWorkspace &w = h->est;
-    const int nprob = (int)n.size(), B = h->B;
-    if (dpd::launch_moments(static_cast<const dpd::GramProblem *>(w.probs), nprob, *std::max_element(n.begin(), n.end()), B,
-                            w.mom_part, w.mom, s) != cudaSuccess)
-        return DPD_ERR_CUDA;
-    std::vector<double> mom((size_t)nprob * dpd::kMomK);
-    if (cudaMemcpyAsync(mom.data(), w.mom, sizeof(double) * mom.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return DPD_ERR_CUDA;
-    std::vector<float> uf((size_t)nprob * dpd::kUSize, 0.f);
-    std::vector<double> ud((size_t)nprob * dpd::kUSize, 0.0);
-    for (int p = 0; p < nprob; ++p) {
-        double M[dpd::kMaxB][dpd::kMaxB], L[dpd::kMaxB][dpd::kMaxB] = {}, U[dpd::kMaxB][dpd::kMaxB] = {};
-        for (int a = 0; a < B; ++a)
-            for (int b = 0; b < B; ++b) M[a][b] = mom[(size_t)p * dpd::kMomK + a + b] / (double)n[p];
-        bool spd = true;
-        for (int i = 0; i < B && spd; ++i)
-            for (int j = 0; j <= i; ++j) {
-                double v = M[i][j];
-                for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-                if (i == j) {
-                    if (!(v > 0.0) || !std::isfinite(v)) {
-                        spd = false;
-                        break;
-                    }
-                    L[i][i] = std::sqrt(v);
-                } else {
-                    L[i][j] = v / L[j][j];
-                }
-            }
-        if (spd) {   // U = L^{-T}: L^T U = I, solved column by column (back substitution)
-            for (int b = 0; b < B; ++b)
-                for (int a = B - 1; a >= 0; --a) {
-                    double v = a == b ? 1.0 : 0.0;
-                    for (int k = a + 1; k < B; ++k) v -= L[k][a] * U[k][b];
-                    U[a][b] = v / L[a][a];
-                }
-        }
-        for (int a = 0; a < dpd::kMaxB; ++a)
-            for (int b = 0; b < dpd::kMaxB; ++b) {
-                const double v = (a < B && b < B) ? (spd ? U[a][b] : (a == b ? 1.0 : 0.0)) : 0.0;
-                uf[(size_t)p * dpd::kUSize + a * dpd::kMaxB + b] = (float)v;
-                ud[(size_t)p * dpd::kUSize + a * dpd::kMaxB + b] = (double)(float)v;
-            }
-    }
-    if (cudaMemcpyAsync(w.ubasis, uf.data(), sizeof(float) * uf.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(w.ubasis64, ud.data(), sizeof(double) * ud.size(), cudaMemcpyHostToDevice, s) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return DPD_ERR_CUDA;
-    return DPD_OK;
+    return dpd::launch_basis(one ? nullptr : static_cast<const dpd::GramProblem *>(w.probs),
+                             one ? *one : dpd::GramProblem{nullptr, nullptr, 0}, nprob, nmax, h->B, w.mom_part, w.ubasis,
+                             w.ubasis64, s) == cudaSuccess
+               ? DPD_OK
+               : DPD_ERR_CUDA;
 }
 
-// FP64 coefficients of problems [p0, p0 + np) in the monomial basis (w.hm64).
-const double2 *monomial_h(dpd_handle h, int p0, int np, cudaStream_t s, dpd_status &st)
+// Solve for problems [p0, p0 + np): right-hand sides g (w.g), or `rows` rows per problem
+// of coefficient-gradient partials added to the coefficients.  Leaves the coefficients in
+// w.h64, their FP32 monomial form in `out` (K per problem, of problem 0) and their forward
+// tables in w.tab.
+dpd_status solve(dpd_handle h, int p0, int np, const float2 *rows, int nrows, float2 *out, cudaStream_t s)
 {
     EstimateWorkspace &w = h->est;
     const size_t off = (size_t)p0 * h->K;
-    st = DPD_OK;
-    if (!ortho(h)) return w.h64 + off;
-    if (dpd::launch_basis_transform(w.h64 + off, w.hm64 + off, w.ubasis64 + (size_t)p0 * dpd::kUSize, np, h->K,
-                                    h->Bp, h->Bq, h->T, 1, s) != cudaSuccess)
-        st = DPD_ERR_CUDA;
-    return w.hm64 + off;
+    dpd::SolveIo io;
+    io.rhs = rows ? nullptr : w.g + off;
+    io.rows = rows;
+    io.nrows = nrows;
+    io.basis = ortho(h) ? w.ubasis64 + (size_t)p0 * dpd::kUSize : nullptr;
+    io.h = w.h64 + off;
+    io.accumulate = rows ? 1 : 0;
+    io.out = out + off;
+    io.tstride = (int)table_stride(h);
+    io.tab = w.tab + p0 * table_stride(h);
+    io.Bp = h->Bp;
+    io.Bq = h->Bq;
+    io.T = h->T;
+    return dpd::launch_chol_solve(w.U + p0 * factor_size(h->K), w.d + off, w.info + p0, np, h->K, io, h->d_status, s) ==
+                   cudaSuccess
+               ? DPD_OK
+               : DPD_ERR_CUDA;
 }
 
 int gram_cpp(dpd_handle h, int nprob, int64_t n, int precision)
@@ -204,22 +168,18 @@ dpd_status run_gram(dpd_handle h, int nprob, int cpp, int precision, cudaStream_
     return DPD_OK;
 }
 
-// e = t - Psi(u) h for the current FP64 coefficients of problem p (FP32 filter);
-// with `norms`, only ||e||^2 and ||t||^2 into w.norm_part + 2 kFwdNormSlots
+// e = t - Psi(u) h for the current coefficients of problem p (its table in w.tab; FP32
+// filter); with `norms`, only ||e||^2 and ||t||^2 into w.norm_part + 2 kFwdNormSlots
 // (e itself is not written).
 dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, int64_t n, cudaStream_t s,
                        bool norms = false)
 {
     EstimateWorkspace &w = h->est;
-    dpd_status st = DPD_OK;
-    const double2 *hm = monomial_h(h, p, 1, s, st);
-    if (st != DPD_OK) return st;
-    if (dpd::launch_wl_table_f64(hm, h->Bp, h->Bq, h->T, w.tab, s) != cudaSuccess) return DPD_ERR_CUDA;
     dpd::FwdArgs fa;
     fa.x = u;
     fa.y = w.y;
     fa.n = n;
-    fa.tab = w.tab;
+    fa.tab = w.tab + p * table_stride(h);
     fa.status = h->d_status;
     fa.vec_store = 1;
     fa.host_tab = nullptr;
@@ -258,7 +218,7 @@ dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, in
 }
 
 // One refinement step of problem p:  h64[p] += G^{-1} Psi^H (t - Psi h).
-dpd_status refine_once(dpd_handle h, int p, const float2 *u, const float2 *t, int64_t n, cudaStream_t s)
+dpd_status refine_once(dpd_handle h, int p, const float2 *u, const float2 *t, int64_t n, float2 *out, cudaStream_t s)
 {
     EstimateWorkspace &w = h->est;
     const int K = h->K;
@@ -278,34 +238,21 @@ dpd_status refine_once(dpd_handle h, int p, const float2 *u, const float2 *t, in
     if (al.gh_blocks > h->rows_max) al.gh_blocks = h->rows_max;
     if (al.gh_blocks < 1) al.gh_blocks = 1;
     if (dpd::launch_adj_any(h->B, aa, al, h->T, h->Bp, h->Bq, K, h->sm_count, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if (dpd::launch_adj_finalize64(h->d_partials, al.gh_blocks, K, w.delta, s) != cudaSuccess) return DPD_ERR_CUDA;
-    const double2 *rhs = w.delta;   // Psi^H (t - Psi h) in the monomial basis
-    if (ortho(h)) {                 // W^T of it, the right-hand side in the working basis
-        if (dpd::launch_basis_transform(w.delta, w.hm64 + (size_t)p * K, w.ubasis64 + (size_t)p * dpd::kUSize, 1,
-                                        K, h->Bp, h->Bq, h->T, 0, s) != cudaSuccess)
-            return DPD_ERR_CUDA;
-        rhs = w.hm64 + (size_t)p * K;
-    }
-    if (dpd::launch_chol_solve(w.U + p * factor_size(K), w.d + (size_t)p * K, w.info + p, rhs, 1, K,
-                               w.h64 + (size_t)p * K, 1, h->d_status, s) != cudaSuccess)
-        return DPD_ERR_CUDA;
-    return DPD_OK;
+    return solve(h, p, 1, h->d_partials, al.gh_blocks, out, s);   // Psi^H (t - Psi h): the sum of the rows
 }
 
 // Refinement of all problems of a batch together, each step one launch per
-// kernel: the per-problem forward tables, the batched forward filter (6
-// samples per thread, 16 warps in groups of 8, 4 stages) into the residual
-// buffers, e = t - Psi h in place, the coefficient gradients of all problems
-// (one CTA per problem and tap group), their FP64 sums, the basis transform
-// (orthogonal basis) and the batched Cholesky solve.  Needs 16-byte aligned
-// inputs u (the bulk-copy pipelines); the caller checks that.
+// kernel: the batched forward filter (6 samples per thread, 16 warps in groups of
+// 8, 4 stages) into the residual buffers, e = t - Psi h, the coefficient gradients
+// of all problems (one CTA per problem and tap group) and the batched solve.
+// Needs 16-byte aligned inputs u (the bulk-copy pipelines); the caller checks that.
 dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &probs, int64_t nmax, int iters,
-                          cudaStream_t s)
+                          float2 *out, cudaStream_t s)
 {
     EstimateWorkspace &w = h->est;
     const int K = h->K, count = (int)probs.size();
     const int64_t stride = (nmax + 1) & ~int64_t(1);   // keeps every e_p 16-byte aligned
-    const int tfl = dpd::wl_table_floats(h->B, h->T), tstride = (tfl + 3) & ~3;
+    const int tstride = (int)table_stride(h);
     constexpr int V = 6, warps = 16, group = 8, stages = 4;
     const int S = warps * 32 * V;
     std::vector<dpd::BatchStream> st((size_t)count);
@@ -329,15 +276,12 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
         cudaFree(w.bstreams);
         cudaFree(w.badj);
         cudaFree(w.bpart);
-        cudaFree(w.tabb);
         w.bstreams = w.badj = nullptr;
         w.bpart = nullptr;
-        w.tabb = nullptr;
         w.bprob_cap = 0;
         if (cudaMalloc(&w.bstreams, sizeof(dpd::BatchStream) * count) != cudaSuccess ||
             cudaMalloc(&w.badj, sizeof(dpd::AdjArgs) * count) != cudaSuccess ||
-            cudaMalloc(&w.bpart, sizeof(float2) * (size_t)count * K) != cudaSuccess ||
-            cudaMalloc(&w.tabb, sizeof(float) * (size_t)count * tstride) != cudaSuccess)
+            cudaMalloc(&w.bpart, sizeof(float2) * (size_t)count * K) != cudaSuccess)
             return DPD_ERR_ALLOC;
         w.bprob_cap = (size_t)count;
     }
@@ -364,32 +308,20 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     ba.items = static_cast<const dpd::BatchItem *>(w.bitems);
     ba.nitems = (int)items.size();
     ba.nstreams = count;
-    ba.tabs = w.tabb;
+    ba.tabs = w.tab;
     ba.tab_floats = (int64_t)count * tstride;
     ba.status = h->d_status;
     ba.gw = group;
     const bool small = h->B <= 5 && h->T <= 7;
-    dpd_status stt = DPD_OK;
     for (int it = 0; it < iters; ++it) {
-        const double2 *hm = monomial_h(h, 0, count, s, stt);
-        if (stt != DPD_OK) return stt;
-        if (dpd::launch_wl_table_f64_many(hm, count, K, h->Bp, h->Bq, h->T, w.tabb, tstride, s) != cudaSuccess)
-            return DPD_ERR_CUDA;
         const cudaError_t fe = small ? dpd::launch_batched_57(ba, V, warps, stages, 0, h->sm_count, s)
                                      : dpd::launch_batched_68(ba, V, warps, stages, 0, h->sm_count, s);
         if (fe != cudaSuccess) return DPD_ERR_CUDA;   // the filter wrote e_p = t_p - Psi h_p
         if (dpd::launch_adj_gh_many_any(h->B, static_cast<const dpd::AdjArgs *>(w.badj), count, 1, h->adj.tap_group,
                                         h->T, h->Bp, h->Bq, K, s) != cudaSuccess)
             return DPD_ERR_CUDA;
-        if (dpd::launch_adj_finalize64_many(w.bpart, 1, K, count, w.delta, s) != cudaSuccess) return DPD_ERR_CUDA;
-        const double2 *rhs = w.delta;   // Psi^H (t - Psi h) in the monomial basis
-        if (ortho(h)) {                 // W^T of it, the right-hand sides in the working basis
-            if (dpd::launch_basis_transform(w.delta, w.hm64, w.ubasis64, count, K, h->Bp, h->Bq, h->T, 0, s) !=
-                cudaSuccess)
-                return DPD_ERR_CUDA;
-            rhs = w.hm64;
-        }
-        if (dpd::launch_chol_solve(w.U, w.d, w.info, rhs, count, K, w.h64, 1, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+        const dpd_status st2 = solve(h, 0, count, w.bpart, 1, out, s);
+        if (st2 != DPD_OK) return st2;
     }
     return DPD_OK;
 }
@@ -680,21 +612,16 @@ void free_estimate_workspace(EstimateWorkspace &w)
     cudaFree(w.g);
     cudaFree(w.U);
     cudaFree(w.h64);
-    cudaFree(w.delta);
     cudaFree(w.d);
     cudaFree(w.tt);
     cudaFree(w.info);
-    cudaFree(w.hf);
     cudaFree(w.tab);
     cudaFree(w.y);
     cudaFree(w.e);
     cudaFree(w.norm_part);
     cudaFree(w.ubasis);
     cudaFree(w.ubasis64);
-    cudaFree(w.mom);
     cudaFree(w.mom_part);
-    cudaFree(w.hm64);
-    cudaFree(w.tabb);
     cudaFree(w.bstreams);
     cudaFree(w.bitems);
     cudaFree(w.badj);
@@ -749,11 +676,8 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if ((st = reserve(h, 1, cpp, (refine_iters > 0 || stats) ? n : 0)) != DPD_OK) return st;
     EstimateWorkspace &w = h->est;
     const dpd::GramProblem pr{static_cast<const float2 *>(u), static_cast<const float2 *>(t), n};
-    if (ortho(h)) {
-        if (cudaMemcpyAsync(w.probs, &pr, sizeof(pr), cudaMemcpyHostToDevice, s) != cudaSuccess) return DPD_ERR_CUDA;
-        if ((st = compute_basis(h, std::vector<int64_t>{n}, s)) != DPD_OK) return st;
-    }
-    if ((st = run_gram(h, 1, cpp, precision, s, ortho(h) ? nullptr : &pr)) != DPD_OK) return st;
+    if (ortho(h) && (st = compute_basis(h, &pr, 1, n, s)) != DPD_OK) return st;
+    if ((st = run_gram(h, 1, cpp, precision, s, &pr)) != DPD_OK) return st;
     // For the statistics, G and (after the factorisation) the factor go
     // to pinned host memory while the device carries on, and so does the pivot
     // status: the host condition estimate (Lanczos on D G D from G, and on its
@@ -770,12 +694,10 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
                       cudaSuccess) ||
         cudaEventRecord(w.ev_U, s) != cudaSuccess)
         return DPD_ERR_CUDA;
-    if (dpd::launch_chol_solve(w.U, w.d, w.info, w.g, 1, K, w.h64, 0, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+    float2 *out = static_cast<float2 *>(h_out);
+    if ((st = solve(h, 0, 1, nullptr, 0, out, s)) != DPD_OK) return st;
     for (int i = 0; i < refine_iters; ++i)
-        if ((st = refine_once(h, 0, pr.u, pr.t, n, s)) != DPD_OK) return st;
-    const double2 *hm = monomial_h(h, 0, 1, s, st);
-    if (st != DPD_OK) return st;
-    if (dpd::launch_h_to_f32(hm, K, static_cast<float2 *>(h_out), s) != cudaSuccess) return DPD_ERR_CUDA;
+        if ((st = refine_once(h, 0, pr.u, pr.t, n, out, s)) != DPD_OK) return st;
     if (stats && (st = queue_norms(h, 0, pr.u, pr.t, n, s)) != DPD_OK) return st;
     // The two Lanczos runs overlap the queued device work: the one on D G D
     // (a second host thread) as soon as G has landed, the one on the inverse
@@ -833,10 +755,11 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
     if (cudaMemcpyAsync(w.probs, probs.data(), sizeof(dpd::GramProblem) * count, cudaMemcpyHostToDevice, s) !=
         cudaSuccess)
         return DPD_ERR_CUDA;
-    if (ortho(h) && (st = compute_basis(h, std::vector<int64_t>(n, n + count), s)) != DPD_OK) return st;
+    if (ortho(h) && (st = compute_basis(h, nullptr, count, nmax, s)) != DPD_OK) return st;
     if ((st = run_gram(h, count, cpp, precision, s)) != DPD_OK) return st;
     if (dpd::launch_chol(w.G, count, h->K, w.U, w.d, w.info, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if (dpd::launch_chol_solve(w.U, w.d, w.info, w.g, count, h->K, w.h64, 0, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+    float2 *out = static_cast<float2 *>(h_out);
+    if ((st = solve(h, 0, count, nullptr, 0, out, s)) != DPD_OK) return st;
     // The pivot status comes back here only for the refinement problem by
     // problem, which skips problems that did not factor; refined together, the
     // launches are queued behind the solve without a host round trip and the
@@ -847,16 +770,13 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
                       cudaStreamSynchronize(s) != cudaSuccess))
         return DPD_ERR_CUDA;
     if (together) {   // problems that did not factor keep unspecified coefficients
-        if ((st = refine_batched(h, probs, nmax, refine_iters, s)) != DPD_OK) return st;
+        if ((st = refine_batched(h, probs, nmax, refine_iters, out, s)) != DPD_OK) return st;
     } else {
         for (int it = 0; it < refine_iters; ++it)
             for (int p = 0; p < count; ++p)
-                if (info[p] == 0 && (st = refine_once(h, p, probs[p].u, probs[p].t, probs[p].n, s)) != DPD_OK)
+                if (info[p] == 0 && (st = refine_once(h, p, probs[p].u, probs[p].t, probs[p].n, out, s)) != DPD_OK)
                     return st;
     }
-    const double2 *hm = monomial_h(h, 0, count, s, st);
-    if (st != DPD_OK) return st;
-    if (dpd::launch_h_to_f32(hm, count * h->K, static_cast<float2 *>(h_out), s) != cudaSuccess) return DPD_ERR_CUDA;
     if (together &&
         cudaMemcpyAsync(info.data(), w.info, sizeof(int) * count, cudaMemcpyDeviceToHost, s) != cudaSuccess)
         return DPD_ERR_CUDA;

@@ -63,10 +63,10 @@ cudaError_t launch_gram_reduce(const float *partials, int nprob, int cpp, int D,
 constexpr int kMomThreads = 256;
 
 template <int NK>
-__global__ void __launch_bounds__(kMomThreads) moments_kernel(const GramProblem *__restrict__ probs,
+__global__ void __launch_bounds__(kMomThreads) moments_kernel(const GramProblem *__restrict__ probs, GramProblem one,
                                                               double *__restrict__ part)
 {
-    const GramProblem pr = probs[blockIdx.y];
+    const GramProblem pr = probs ? probs[blockIdx.y] : one;
     float2 sum[NK];   // (sum, error)
 #pragma unroll
     for (int k = 0; k < NK; ++k) sum[k] = make_float2(0.f, 0.f);
@@ -112,81 +112,95 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const GramProblem 
     }
 }
 
-// One warp per power: lane l adds blocks l, l + 32, ... in order, then a fixed
-// shuffle tree.  Powers past nk are zero.
-__global__ void __launch_bounds__(32 * kMomK) moments_sum_kernel(const double *__restrict__ part, int blocks, int nk,
-                                                                 double *__restrict__ mom)
+// Basis of statistically orthogonal polynomials (Sec. 2.1) of a problem per block.
+// Power sums mu_k: one warp per power, lane l adds blocks l, l + 32, ... in order, then a
+// fixed shuffle tree.  Then one warp: the moment matrix M[a][b] = mu_{a+b+1} / n is the
+// Gram matrix of the monomials |u|^{2a} u; M = L L^T (lane i holds row i) and U = L^{-T}
+// (lane b solves for column b) make sum_a U[a][b] |u|^{2a} u orthonormal.  U is rounded
+// to FP32 for the Gram kernels and the same values are kept in FP64 for the coefficient
+// transforms.  A moment matrix that is not positive definite gives the monomials (U = I).
+// FP64's latency (64 cycles) bounds it: 13 us; a kernel for the sums, two copies, two
+// synchronisations and the same factorisation on the host took about 45.
+__global__ void __launch_bounds__(32 * kMomK) basis_kernel(const GramProblem *__restrict__ probs, GramProblem one,
+                                                           const double *__restrict__ part, int blocks, int B,
+                                                           float *__restrict__ ubasis, double *__restrict__ ubasis64)
 {
+    __shared__ double mu[kMomK], L[kMaxB][kMaxB], rinv[kMaxB];
+    grid_dep_wait();
     const int p = blockIdx.x, k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    if (k < nk) {
+    if (k < 2 * B - 1) {
 #pragma unroll 4
         for (int b = lane; b < blocks; b += 32) s += part[((size_t)p * blocks + b) * kMomK + k];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) mom[(size_t)p * kMomK + k] = s;
+    if (lane == 0) mu[k] = s / (double)(probs ? probs[p].n : one.n);
+    __syncthreads();
+    if (k != 0) return;
+    const int i = lane;
+    double row[kMaxB];
+#pragma unroll
+    for (int j = 0; j < kMaxB; ++j) row[j] = i < B && j < B ? mu[i + j] : 0.0;
+    bool spd = true;
+#pragma unroll
+    for (int j = 0; j < kMaxB; ++j)
+        if (j < B && spd) {
+            const double piv = __shfl_sync(0xffffffffu, row[j], j);
+            spd = piv > 0.0 && isfinite(piv);
+            const double r = spd ? inv_sqrt(piv) : 0.0;
+            const double l = row[j] * r;
+            if (i >= j && i < B) L[i][j] = l;
+            if (i == j) rinv[j] = r;
+#pragma unroll
+            for (int q = j + 1; q < kMaxB; ++q) row[q] = fma(-l, __shfl_sync(0xffffffffu, l, q), row[q]);
+        }
+    __syncwarp();
+    double u[kMaxB];   // column i of U
+#pragma unroll
+    for (int a = kMaxB - 1; a >= 0; --a) {
+        u[a] = 0.0;
+        if (a < B && i < B) {
+            double v = a == i ? 1.0 : 0.0;
+            if (spd) {
+#pragma unroll
+                for (int q = a + 1; q < kMaxB; ++q)
+                    if (q < B) v = fma(-L[q][a], u[q], v);
+                v *= rinv[a];
+            }
+            u[a] = v;
+        }
+    }
+    if (i < kMaxB)
+#pragma unroll
+        for (int a = 0; a < kMaxB; ++a) {
+            const size_t at = (size_t)p * kUSize + a * kMaxB + i;
+            ubasis[at] = (float)u[a];
+            ubasis64[at] = (double)(float)u[a];
+        }
 }
 
-cudaError_t launch_moments(const GramProblem *probs, int nprob, int64_t nmax, int B, double *part, double *mom,
-                           cudaStream_t s)
+cudaError_t launch_basis(const GramProblem *probs, GramProblem one, int nprob, int64_t nmax, int B, double *part,
+                         float *ubasis, double *ubasis64, cudaStream_t s)
 {
     // At least a thousand samples (four per thread) a block.
     const int64_t need = (nmax + 4 * kMomThreads - 1) / (4 * kMomThreads);
     const int blocks = (int)(need < moments_blocks(nprob) ? need : moments_blocks(nprob));
     const dim3 grid((unsigned)blocks, (unsigned)nprob);
     switch (B) {
-    case 1: moments_kernel<1><<<grid, kMomThreads, 0, s>>>(probs, part); break;
-    case 2: moments_kernel<3><<<grid, kMomThreads, 0, s>>>(probs, part); break;
-    case 3: moments_kernel<5><<<grid, kMomThreads, 0, s>>>(probs, part); break;
-    case 4: moments_kernel<7><<<grid, kMomThreads, 0, s>>>(probs, part); break;
-    case 5: moments_kernel<9><<<grid, kMomThreads, 0, s>>>(probs, part); break;
-    case 6: moments_kernel<11><<<grid, kMomThreads, 0, s>>>(probs, part); break;
+    case 1: moments_kernel<1><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
+    case 2: moments_kernel<3><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
+    case 3: moments_kernel<5><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
+    case 4: moments_kernel<7><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
+    case 5: moments_kernel<9><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
+    case 6: moments_kernel<11><<<grid, kMomThreads, 0, s>>>(probs, one, part); break;
     default: return cudaErrorInvalidValue;
     }
     count_launch();
-    moments_sum_kernel<<<nprob, 32 * kMomK, 0, s>>>(part, blocks, 2 * B - 1, mom);
-    count_launch();
-    return cudaGetLastError();
-}
-
-__global__ void basis_transform_kernel(const double2 *__restrict__ in, double2 *__restrict__ out,
-                                       const double *__restrict__ Uall, int K, int Bp, int Bq, int T, int to_monomial)
-{
-    const int p = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= K) return;
-    const double2 *x = in + (size_t)p * K;
-    const double *U = Uall + (size_t)p * kUSize;
-    double2 v;
-    if (j == K - 1) {
-        v = x[j];
-    } else {
-        const bool conj = j >= Bp * T;
-        const int base = conj ? Bp * T : 0, nb = conj ? Bq : Bp, jj = j - base, a = jj / T, k = jj % T;
-        v = make_double2(0.0, 0.0);
-        if (to_monomial) {   // h[(a, k)] = sum_{b >= a} U[a][b] h_U[(b, k)]
-            for (int b = a; b < nb; ++b) {
-                const double u = U[a * kMaxB + b];
-                v.x += u * x[base + b * T + k].x;
-                v.y += u * x[base + b * T + k].y;
-            }
-        } else {             // g_U[(a, k)] = sum_{c <= a} U[c][a] g[(c, k)]
-            for (int c = 0; c <= a; ++c) {
-                const double u = U[c * kMaxB + a];
-                v.x += u * x[base + c * T + k].x;
-                v.y += u * x[base + c * T + k].y;
-            }
-        }
-    }
-    out[(size_t)p * K + j] = v;
-}
-
-cudaError_t launch_basis_transform(const double2 *in, double2 *out, const double *U, int nprob, int K, int Bp,
-                                   int Bq, int T, int to_monomial, cudaStream_t s)
-{
-    basis_transform_kernel<<<dim3((K + 127) / 128, nprob), 128, 0, s>>>(in, out, U, K, Bp, Bq, T, to_monomial);
-    count_launch();
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_pdl(basis_kernel, dim3((unsigned)nprob), 32 * kMomK, 0, s, probs, one, part, blocks, B, ubasis,
+                      ubasis64);
 }
 
 // <x, y> for two signed distinct-column references: S = P + Q + Q^T from the
@@ -228,19 +242,6 @@ cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int 
 {
     dim3 grid((K * K + K + 1 + 255) / 256, nprob);
     gram_assemble_kernel<<<grid, 256, 0, s>>>(S, K, Bp, B, T, G, g, tt);
-    count_launch();
-    return cudaGetLastError();
-}
-
-__global__ void h_to_f32_kernel(const double2 *__restrict__ h, int n, float2 *__restrict__ out)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = make_float2((float)h[i].x, (float)h[i].y);
-}
-
-cudaError_t launch_h_to_f32(const double2 *h, int n, float2 *out, cudaStream_t s)
-{
-    h_to_f32_kernel<<<(n + 127) / 128, 128, 0, s>>>(h, n, out);
     count_launch();
     return cudaGetLastError();
 }
