@@ -92,11 +92,12 @@ cudaError_t launch_gram_reduce(const float *partials, int nprob, int cpp, int D,
 // (a < 15, b < 14, d < kMaxT), each an FP32 pair (sum, rounding error); this sums them per
 // problem into C (FP64, fixed order).
 // G, g and t^H t are assembled from C directly (the entries of S on the fly), into G / g
-// / tt at K x K, K, 1 per problem; probs may be null for one problem passed as `one`.
+// / tt at K x K, K, 1 per problem; probs may be null for one problem passed as `one`;
+// `lower`: only the lower triangle of G (what the factorisation reads).
 constexpr int kLagEntries = 15 * 14 * kMaxT;
 cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *probs, GramProblem one,
-                                   const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, double *C,
-                                   double2 *G, double2 *g, double *tt, cudaStream_t s);
+                                   const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, bool lower,
+                                   double *C, double2 *G, double2 *g, double *tt, cudaStream_t s);
 // G (K x K, row-major), g (K) and t^H t per problem from S.
 cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int B, int T, double2 *G, double2 *g,
                                  double *tt, cudaStream_t s);

@@ -10,11 +10,11 @@
 
 // Device workspace of dpd_estimate, grown on demand.
 struct EstimateWorkspace {
-    int cpp = 0;                  // Gram CTAs per problem the partials were sized for
     int nprob = 0;                // problems the per-problem arrays were sized for
     int64_t nsamp = 0;            // samples the y / e buffers hold
     void *probs = nullptr;        // GramProblem[nprob]
-    float *partials = nullptr;    // [nprob * cpp][kGramRows][kGramPartCols]
+    size_t partials_cap = 0;      // floats
+    float *partials = nullptr;    // per Gram CTA: [kGramRows][kGramPartCols], or kLagEntries pairs
     double *S = nullptr;          // [nprob][kGramS][kGramPartCols]: summed P and Q blocks
     double *Clag = nullptr;       // [nprob][kLagEntries]: summed lag sums (tensor-core Gram)
     double2 *G = nullptr, *g = nullptr, *h64 = nullptr;
@@ -40,8 +40,8 @@ struct EstimateWorkspace {
     void *bstreams = nullptr;     // dpd::BatchStream [problems]
     void *bitems = nullptr;       // dpd::BatchItem [items]
     void *badj = nullptr;         // dpd::AdjArgs [problems]
-    float2 *bpart = nullptr;      // coefficient-gradient partials, [problems][K]
-    size_t bprob_cap = 0, bitems_cap = 0;
+    float2 *bpart = nullptr;      // coefficient-gradient partials, [problems][rows][K]
+    size_t bprob_cap = 0, bitems_cap = 0, bpart_cap = 0;   // problems, items, rows
     cudaEvent_t ev_U = nullptr;   // h_info (and h_U) have landed
 };
 

@@ -31,18 +31,27 @@ bool grow(T *&p, size_t have, size_t need)
     return cudaMalloc(&p, std::max<size_t>(need, 1) * sizeof(T)) == cudaSuccess;
 }
 
-// Make sure the workspace holds nprob problems with cpp Gram CTAs each and
-// nsamp samples of refinement buffers.  Synchronises the device when it grows.
-dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
+// Make sure the workspace holds nprob problems with cpp Gram CTAs each at this
+// precision and nsamp samples of refinement buffers.  Synchronises the device when it
+// grows.
+dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsamp)
 {
     EstimateWorkspace &w = h->est;
     const int K = h->K;
     bool ok = true;
-    if (nprob > w.nprob || cpp * nprob > w.cpp * w.nprob) {
+    const size_t part = precision == dpd::kPrecFP32 ? (size_t)dpd::kGramRows * dpd::kGramPartCols
+                                                    : (size_t)2 * dpd::kLagEntries;   // floats per CTA
+    const size_t parts = (size_t)nprob * cpp * part;
+    if (parts > w.partials_cap) {
         cudaDeviceSynchronize();
-        const size_t np = (size_t)nprob, parts = (size_t)nprob * cpp;
+        w.partials_cap = 0;
+        if (!grow(w.partials, 0, parts)) return DPD_ERR_ALLOC;
+        w.partials_cap = parts;
+    }
+    if (nprob > w.nprob) {
+        cudaDeviceSynchronize();
+        const size_t np = (size_t)nprob;
         ok = ok && grow(reinterpret_cast<dpd::GramProblem *&>(w.probs), 0, np);
-        ok = ok && grow(w.partials, 0, parts * dpd::kGramRows * dpd::kGramPartCols);
         ok = ok && grow(w.S, 0, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, 0, np * dpd::kLagEntries);
         ok = ok && grow(w.G, 0, np * K * K) && grow(w.U, 0, np * factor_size(K));
         ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K);
@@ -55,7 +64,6 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int64_t nsamp)
         ok = ok && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         if (!ok) return DPD_ERR_ALLOC;
         w.nprob = nprob;
-        w.cpp = cpp;
     }
     if (w.hK != K || !w.h_G) {
         cudaFreeHost(w.h_G);
@@ -162,7 +170,7 @@ dpd_status run_gram(dpd_handle h, int nprob, int cpp, int precision, cudaStream_
             dpd::launch_gram_assemble(w.S, nprob, h->K, h->Bp, h->B, h->T, G, g, w.tt, s) != cudaSuccess)
             return DPD_ERR_CUDA;
     } else if (dpd::launch_gram_lag_finish(w.partials, a.probs, a.one, a.ubasis, nprob, cpp, h->K, h->Bp, h->B, h->T,
-                                           w.Clag, G, g, w.tt, s) != cudaSuccess) {
+                                           nprob > 1, w.Clag, G, g, w.tt, s) != cudaSuccess) {
         return DPD_ERR_CUDA;
     }
     return DPD_OK;
@@ -244,7 +252,7 @@ dpd_status refine_once(dpd_handle h, int p, const float2 *u, const float2 *t, in
 // Refinement of all problems of a batch together, each step one launch per
 // kernel: the batched forward filter (6 samples per thread, 16 warps in groups of
 // 8, 4 stages) into the residual buffers, e = t - Psi h, the coefficient gradients
-// of all problems (one CTA per problem and tap group) and the batched solve.
+// of all problems (a few CTAs per problem and tap group) and the batched solve.
 // Needs 16-byte aligned inputs u (the bulk-copy pipelines); the caller checks that.
 dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &probs, int64_t nmax, int iters,
                           float2 *out, cudaStream_t s)
@@ -254,7 +262,27 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     const int64_t stride = (nmax + 1) & ~int64_t(1);   // keeps every e_p 16-byte aligned
     const int tstride = (int)table_stride(h);
     constexpr int V = 6, warps = 16, group = 8, stages = 4;
-    const int S = warps * 32 * V;
+    // Two sub-blocks of 3,072 samples to an item where that leaves four items per SM
+    // (256 x 2^16 at K = 97: 139 us against 147 with one).
+    int64_t total = 0;
+    for (const dpd::GramProblem &pr : probs) total += pr.n / (2 * warps * 32 * V);
+    const int nsub = total >= 4 * (int64_t)h->sm_count ? dpd::batch_nsub(warps, group, stages, V) : 1;
+    const int S = nsub * warps * 32 * V;
+    // CTAs of a problem and tap group in the coefficient gradient, one per SM: the rounds
+    // that the launch takes, each a share of the samples and a CTA's start and end, about
+    // kCtaSamples samples' time.
+    const int groups = (h->T + h->adj.tap_group - 1) / h->adj.tap_group;
+    int rows = 1;
+    int64_t best = INT64_MAX;
+    for (int r = 1; r <= std::max(8, h->sm_count / (groups * count)); ++r) {
+        constexpr int64_t kCtaSamples = 7000;
+        const int64_t rounds = ((int64_t)groups * count * r + h->sm_count - 1) / h->sm_count;
+        const int64_t cost = rounds * ((nmax + r - 1) / r + kCtaSamples);
+        if (cost < best) {
+            best = cost;
+            rows = r;
+        }
+    }
     std::vector<dpd::BatchStream> st((size_t)count);
     std::vector<dpd::BatchItem> items;
     std::vector<dpd::AdjArgs> adj((size_t)count);
@@ -275,15 +303,18 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
         cudaDeviceSynchronize();
         cudaFree(w.bstreams);
         cudaFree(w.badj);
-        cudaFree(w.bpart);
         w.bstreams = w.badj = nullptr;
-        w.bpart = nullptr;
         w.bprob_cap = 0;
         if (cudaMalloc(&w.bstreams, sizeof(dpd::BatchStream) * count) != cudaSuccess ||
-            cudaMalloc(&w.badj, sizeof(dpd::AdjArgs) * count) != cudaSuccess ||
-            cudaMalloc(&w.bpart, sizeof(float2) * (size_t)count * K) != cudaSuccess)
+            cudaMalloc(&w.badj, sizeof(dpd::AdjArgs) * count) != cudaSuccess)
             return DPD_ERR_ALLOC;
         w.bprob_cap = (size_t)count;
+    }
+    if ((size_t)count * rows > w.bpart_cap) {
+        cudaDeviceSynchronize();
+        w.bpart_cap = 0;
+        if (!grow(w.bpart, 0, (size_t)count * rows * K)) return DPD_ERR_ALLOC;
+        w.bpart_cap = (size_t)count * rows;
     }
     if (items.size() > w.bitems_cap) {
         cudaDeviceSynchronize();
@@ -293,7 +324,7 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
         if (cudaMalloc(&w.bitems, sizeof(dpd::BatchItem) * items.size()) != cudaSuccess) return DPD_ERR_ALLOC;
         w.bitems_cap = items.size();
     }
-    for (int p = 0; p < count; ++p) adj[p].partials = w.bpart + (size_t)p * K;   // one row per problem
+    for (int p = 0; p < count; ++p) adj[p].partials = w.bpart + (size_t)p * rows * K;
     // Stream-ordered uploads from pageable memory: the runtime stages the host
     // data before each call returns (no device synchronisation), so the vectors
     // may go out of scope and the host goes on enqueuing the launches.
@@ -312,15 +343,16 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     ba.tab_floats = (int64_t)count * tstride;
     ba.status = h->d_status;
     ba.gw = group;
+    ba.nsub = nsub;
     const bool small = h->B <= 5 && h->T <= 7;
     for (int it = 0; it < iters; ++it) {
         const cudaError_t fe = small ? dpd::launch_batched_57(ba, V, warps, stages, 0, h->sm_count, s)
                                      : dpd::launch_batched_68(ba, V, warps, stages, 0, h->sm_count, s);
         if (fe != cudaSuccess) return DPD_ERR_CUDA;   // the filter wrote e_p = t_p - Psi h_p
-        if (dpd::launch_adj_gh_many_any(h->B, static_cast<const dpd::AdjArgs *>(w.badj), count, 1, h->adj.tap_group,
+        if (dpd::launch_adj_gh_many_any(h->B, static_cast<const dpd::AdjArgs *>(w.badj), count, rows, h->adj.tap_group,
                                         h->T, h->Bp, h->Bq, K, s) != cudaSuccess)
             return DPD_ERR_CUDA;
-        const dpd_status st2 = solve(h, 0, count, w.bpart, 1, out, s);
+        const dpd_status st2 = solve(h, 0, count, w.bpart, rows, out, s);
         if (st2 != DPD_OK) return st2;
     }
     return DPD_OK;
@@ -652,7 +684,7 @@ dpd_status dpd_gram(dpd_handle h, const void *u, const void *t, int64_t n, int p
     if (!G || !aligned8(G) || (g && (!t || !aligned8(g)))) return DPD_ERR_INVALID_ARGUMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int cpp = gram_cpp(h, 1, n, precision);
-    if ((st = reserve(h, 1, cpp, 0)) != DPD_OK) return st;
+    if ((st = reserve(h, 1, cpp, precision, 0)) != DPD_OK) return st;
     // Psi of Eq. 2 (the monomial basis, whatever the handle's estimate basis);
     // the problem travels by value in the kernel arguments.
     const dpd::GramProblem pr{static_cast<const float2 *>(u), static_cast<const float2 *>(t), n};
@@ -673,7 +705,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if (!t || !h_out || !aligned8(h_out) || refine_iters < 0 || refine_iters > 100) return DPD_ERR_INVALID_ARGUMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int cpp = gram_cpp(h, 1, n, precision);
-    if ((st = reserve(h, 1, cpp, (refine_iters > 0 || stats) ? n : 0)) != DPD_OK) return st;
+    if ((st = reserve(h, 1, cpp, precision, (refine_iters > 0 || stats) ? n : 0)) != DPD_OK) return st;
     EstimateWorkspace &w = h->est;
     const dpd::GramProblem pr{static_cast<const float2 *>(u), static_cast<const float2 *>(t), n};
     if (ortho(h) && (st = compute_basis(h, &pr, 1, n, s)) != DPD_OK) return st;
@@ -749,7 +781,7 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
     bool together = refine_iters > 0 && count > 1;
     for (int i = 0; i < count && together; ++i) together = (reinterpret_cast<uintptr_t>(u[i]) & 15u) == 0;
     const int64_t nsamp = refine_iters > 0 ? (together ? ((nmax + 1) & ~int64_t(1)) * count : nmax) : 0;
-    dpd_status st = reserve(h, count, cpp, nsamp);
+    dpd_status st = reserve(h, count, cpp, precision, nsamp);
     if (st != DPD_OK) return st;
     EstimateWorkspace &w = h->est;
     if (cudaMemcpyAsync(w.probs, probs.data(), sizeof(dpd::GramProblem) * count, cudaMemcpyHostToDevice, s) !=

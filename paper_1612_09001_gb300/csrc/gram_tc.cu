@@ -3,6 +3,9 @@
 // basis and target signals, split BF16 / TF32 operands) with the kernels that
 // turn its sums into S, and the plain FP32 CUDA-core form it is compared
 // against.
+#include <algorithm>
+#include <cstdint>
+
 #include <cuda_bf16.h>
 
 #include "dpd_gram.cuh"
@@ -524,6 +527,24 @@ __global__ void __launch_bounds__(256) gram_lag_reduce_kernel(const float2 *__re
     }
 }
 
+// The same for the few CTAs of a problem of a batch: one thread per entry.
+constexpr int kLagFew = 8;
+__global__ void __launch_bounds__(256) gram_lag_reduce_few_kernel(const float2 *__restrict__ partials, int cpp,
+                                                                  double *__restrict__ C)
+{
+    const int p = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= kLagEntries) return;
+    const float2 *base = partials + (size_t)p * cpp * kLagEntries + e;
+    float2 v[kLagFew];
+#pragma unroll
+    for (int k = 0; k < kLagFew; ++k) v[k] = k < cpp ? base[(size_t)k * kLagEntries] : make_float2(0.f, 0.f);
+    float2 t = v[0];
+#pragma unroll
+    for (int k = 1; k < kLagFew; ++k)
+        if (k < cpp) t = pair_add(t, v[k]);
+    C[(size_t)p * kLagEntries + e] = (double)t.x + (double)t.y;
+}
+
 // Signal and tap of distinct column d (the order of dpd_gram.cuh).
 __device__ __forceinline__ void lag_source(int d, int B, int T, int &sig, int &tap)
 {
@@ -538,16 +559,18 @@ __device__ __forceinline__ void lag_source(int d, int B, int T, int &sig, int &t
     }
 }
 
-// G, g and t^H t of each problem from its lag sums; grid (entries / 256,
-// problems).  An entry of S is C less the end products, which come from the
+// G, g and t^H t of each problem from its lag sums; grid (blocks, problems), the
+// blocks of a problem sharing its entries; with `lower` only the lower triangle of G.
+// An entry of S is C less the end products, which come from the
 // last T - 1 samples of every signal evaluated as the tensor kernel evaluates
 // them; they are a few of the N products of an entry, so they are summed in
 // FP32 and only the difference is formed in FP64.
 __global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__restrict__ Call,
                                                                 const GramProblem *__restrict__ probs,
                                                                 GramProblem one, const float *__restrict__ ubasis,
-                                                                int K, int Bp, int B, int T, double2 *__restrict__ G,
-                                                                double2 *__restrict__ g, double *__restrict__ tt)
+                                                                int K, int Bp, int B, int T, int lower,
+                                                                double2 *__restrict__ G, double2 *__restrict__ g,
+                                                                double *__restrict__ tt)
 {
     __shared__ float xt[kLagSigA][kMaxT];   // x_s(N - 8 + i), zero before the record
     __shared__ float su_buf[kUSize];
@@ -643,33 +666,43 @@ __global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__
     // x + y and x - y of two such values
     auto sum = [](Pair x, Pair y) { return (x.c + y.c) - (double)(x.t + y.t); };
     auto diff = [](Pair x, Pair y) { return (x.c - y.c) - (double)(x.t - y.t); };
-    const int idx = blockIdx.x * blockDim.x + tid;
     const ColRef tre{2 * B * T + 1, 1}, tim{2 * B * T + 2, 1};
-    if (idx < K * K) {
-        const int a = idx / K, b = idx % K;
-        ColRef ar, ai, br, bi;
-        psi_column_refs(a, K, Bp, B, T, ar, ai);
-        psi_column_refs(b, K, Bp, B, T, br, bi);
-        G[(size_t)p * K * K + idx] = make_double2(sum(dot(ar, br), dot(ai, bi)), diff(dot(ar, bi), dot(ai, br)));
-    } else if (idx < K * K + K) {
-        const int a = idx - K * K;
-        ColRef ar, ai;
-        psi_column_refs(a, K, Bp, B, T, ar, ai);
-        if (g) g[(size_t)p * K + a] = make_double2(sum(dot(ar, tre), dot(ai, tim)), diff(dot(ar, tim), dot(ai, tre)));
-    } else if (idx == K * K + K) {
-        if (tt) tt[p] = sum(dot(tre, tre), dot(tim, tim));
+    for (int idx = blockIdx.x * blockDim.x + tid; idx <= K * K + K; idx += gridDim.x * blockDim.x) {
+        if (idx < K * K) {
+            const int a = idx / K, b = idx % K;
+            if (lower && b > a) continue;
+            ColRef ar, ai, br, bi;
+            psi_column_refs(a, K, Bp, B, T, ar, ai);
+            psi_column_refs(b, K, Bp, B, T, br, bi);
+            G[(size_t)p * K * K + idx] = make_double2(sum(dot(ar, br), dot(ai, bi)), diff(dot(ar, bi), dot(ai, br)));
+        } else if (idx < K * K + K) {
+            const int a = idx - K * K;
+            ColRef ar, ai;
+            psi_column_refs(a, K, Bp, B, T, ar, ai);
+            if (g)
+                g[(size_t)p * K + a] = make_double2(sum(dot(ar, tre), dot(ai, tim)), diff(dot(ar, tim), dot(ai, tre)));
+        } else {
+            if (tt) tt[p] = sum(dot(tre, tre), dot(tim, tim));
+        }
     }
 }
 
 cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *probs, GramProblem one,
-                                   const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, double *C,
-                                   double2 *G, double2 *g, double *tt, cudaStream_t s)
+                                   const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, bool lower,
+                                   double *C, double2 *G, double2 *g, double *tt, cudaStream_t s)
 {
-    gram_lag_reduce_kernel<<<dim3((kLagEntries + 31) / 32, nprob), 256, 0, s>>>(
-        reinterpret_cast<const float2 *>(partials), cpp, C);
+    const float2 *parts = reinterpret_cast<const float2 *>(partials);
+    if (cpp <= kLagFew && nprob > 1)
+        gram_lag_reduce_few_kernel<<<dim3((kLagEntries + 255) / 256, nprob), 256, 0, s>>>(parts, cpp, C);
+    else
+        gram_lag_reduce_kernel<<<dim3((kLagEntries + 31) / 32, nprob), 256, 0, s>>>(parts, cpp, C);
     count_launch();
-    gram_lag_assemble_kernel<<<dim3((K * K + K + 1 + 255) / 256, nprob), 256, 0, s>>>(C, probs, one, ubasis, K, Bp,
-                                                                                       B, T, G, g, tt);
+    // A block's start (the record's last samples in every signal) takes longer than an
+    // entry: one entry per thread for one problem, about eight blocks per SM for many
+    // (256 problems at K = 97: 45.4 us; 63.1 with one entry of the whole G per thread).
+    const int full = (K * K + K + 1 + 255) / 256, share = 8 * 152 / nprob;
+    const int blocks = share < 1 ? 1 : share < full ? share : full;
+    gram_lag_assemble_kernel<<<dim3(blocks, nprob), 256, 0, s>>>(C, probs, one, ubasis, K, Bp, B, T, lower ? 1 : 0, G, g, tt);
     count_launch();
     return cudaGetLastError();
 }
@@ -804,15 +837,29 @@ size_t gram_fp32_smem() { return (size_t)kF32Rows * kF32Stride * 4 + (kMaxB * kP
 
 int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n)
 {
-    // tensor kernel: one CTA per SM in total; FP32 kernel: four (small CTAs);
-    // at least one per problem, no more than row blocks
-    const int total = precision == kPrecFP32 ? 4 * sm_count : sm_count;
-    int cpp = total / (nprob > 0 ? nprob : 1);
-    if (cpp < 1) cpp = 1;
+    // FP32 kernel: four small CTAs per SM in all, at least one per problem.  Tensor
+    // kernel: one CTA per SM, so a launch takes as many rounds as its CTAs fill the SMs,
+    // each round a share of the stages and the start and end of a CTA, about kCtaStages
+    // stages' time.  256 problems of 2^16 samples (TF32: 256 stages) on 152 SMs, us:
+    // 1 CTA each (2 rounds) 617, 4 (7 rounds) 568, 7 (12 rounds) 590.
     const int rows = precision == kPrecFP32   ? kF32Rows
                      : precision == kPrecBF16x3 ? LagGeom<kFmtBF16>::R
                                                 : LagGeom<kFmtTF32>::R;   // samples per stage
     const int64_t blocks = (n + rows - 1) / rows;
+    const int even = std::max((precision == kPrecFP32 ? 4 * sm_count : sm_count) / std::max(nprob, 1), 1);
+    int cpp = even;
+    if (precision != kPrecFP32 && nprob > 1) {
+        constexpr int64_t kCtaStages = 5;
+        int64_t best = INT64_MAX;
+        for (int c = 1; c <= std::max(even, 8); ++c) {
+            const int64_t rounds = ((int64_t)nprob * c + sm_count - 1) / sm_count;
+            const int64_t cost = rounds * ((blocks + c - 1) / c + kCtaStages);
+            if (cost < best) {
+                best = cost;
+                cpp = c;
+            }
+        }
+    }
     if (cpp > blocks) cpp = (int)(blocks > 1 ? blocks : 1);
     return cpp;
 }
