@@ -386,9 +386,9 @@ __global__ void __launch_bounds__(kCholThreads, 1)
 // many lanes it has).
 constexpr int kChol64Threads = 256;
 
-__global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *__restrict__ Gall, int K,
-                                                              float4 *__restrict__ Uall, double *__restrict__ dall,
-                                                              int *__restrict__ info)
+__global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *__restrict__ Gall, int K, float4 *Uall,
+                                                                double *__restrict__ dall, int *info, float4 *Uhost,
+                                                                int *info_host)
 {
     extern __shared__ double2 A[];   // lower triangle of K x K, packed by rows (tri_row)
     __shared__ double dsh[kCholMaxK];
@@ -396,7 +396,17 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
     __shared__ int bad;
     grid_dep_wait();
     const int p = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    if (info[p] != kNeedFp64) return;
+    // Host copies of the first problem, whichever kernel factored it.
+    auto to_host = [&](int status) {
+        if (p != 0 || !Uhost) return;
+        for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = Uall[e];
+        if (tid == 0) *info_host = status;
+    };
+    const int before = info[p];
+    if (before != kNeedFp64) {
+        to_host(before);
+        return;
+    }
     const int tx = tid & 15, ty = tid >> 4, nty = nt >> 4;
     const double2 *G = Gall + (size_t)p * K * K;
     if (tid == 0) bad = 0;
@@ -480,9 +490,12 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
         }
     for (int i = tid; i < K; i += nt) dall[(size_t)p * K + i] = dsh[i];
     if (tid == 0) info[p] = bad;
+    __syncthreads();   // U and every thread's read of info
+    to_host(bad);
 }
 
-cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, int *status, cudaStream_t s)
+cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, float4 *Uhost,
+                        int *info_host, int *status, cudaStream_t s)
 {
     if (K < 2 || K > kCholMaxK) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)nprob);
@@ -497,7 +510,7 @@ cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d
     static SmemAttr smem_rec;
     e = ensure_smem(smem_rec, (const void *)chol64_kernel, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(chol64_kernel, grid, kChol64Threads, smem, s, G, K, U, d, info);
+    return launch_pdl(chol64_kernel, grid, kChol64Threads, smem, s, G, K, U, d, info, Uhost, info_host);
 }
 
 // One CTA per problem: x = D U^{-H} Delta^{-1} U^{-1} D rhs, in FP32 pairs.  The CTA

@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(fwd_lb_threads<SH>(), fwd_lb_blocks<SH>())
             pt = pair_add(pt, shfl_xor_pair(pt, o));
         }
         float4 *part = reinterpret_cast<float4 *>(a.norms);
-        unsigned *count = reinterpret_cast<unsigned *>(a.norms + 2 * kFwdNormSlots + 2);
+        unsigned *count = reinterpret_cast<unsigned *>(a.norms + 2 * kFwdNormSlots);
         int last = 0;
         if (lane == 0) {
             part[blockIdx.x] = make_float4(pe.x, pe.y, pt.x, pt.y);
@@ -516,8 +516,8 @@ __global__ void __launch_bounds__(fwd_lb_threads<SH>(), fwd_lb_blocks<SH>())
             pt = pair_add(pt, shfl_xor_pair(pt, o));
         }
         if (lane == 0) {
-            a.norms[2 * kFwdNormSlots] = (double)pe.x + (double)pe.y;
-            a.norms[2 * kFwdNormSlots + 1] = (double)pt.x + (double)pt.y;
+            a.norms_out[0] = (double)pe.x + (double)pe.y;
+            a.norms_out[1] = (double)pt.x + (double)pt.y;
             *count = 0u;
         }
     }
@@ -631,7 +631,7 @@ cudaError_t launch_fwd_tv(const FwdArgs &a, const FwdLaunch &L, int sm_count, cu
             int64_t grid = (int64_t)sm_count * cps;
             if (grid > ntiles) grid = ntiles;
             if constexpr ((MODE & kModeNorms) != 0)
-                if (!a.norms || grid > kFwdNormSlots || L.warps > kFwdMaxWarps) return cudaErrorInvalidValue;
+                if (!a.norms || !a.norms_out || grid > kFwdNormSlots || L.warps > kFwdMaxWarps) return cudaErrorInvalidValue;
             // Programmatic dependent launch: this grid may begin launching while
             // the previous one in the stream drains (the kernel waits for it
             // before touching global memory).

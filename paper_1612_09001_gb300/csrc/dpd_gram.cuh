@@ -93,14 +93,15 @@ cudaError_t launch_gram_reduce(const float *partials, int nprob, int cpp, int D,
 // problem into C (FP64, fixed order).
 // G, g and t^H t are assembled from C directly (the entries of S on the fly), into G / g
 // / tt at K x K, K, 1 per problem; probs may be null for one problem passed as `one`;
-// `lower`: only the lower triangle of G (what the factorisation reads).
+// `lower`: only the lower triangle of G (what the factorisation reads).  Ghost: a copy
+// of the first problem's G in mapped host memory, or null.
 constexpr int kLagEntries = 15 * 14 * kMaxT;
 cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *probs, GramProblem one,
                                    const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, bool lower,
-                                   double *C, double2 *G, double2 *g, double *tt, cudaStream_t s);
+                                   double *C, double2 *G, double2 *g, double *tt, double2 *Ghost, cudaStream_t s);
 // G (K x K, row-major), g (K) and t^H t per problem from S.
 cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int B, int T, double2 *G, double2 *g,
-                                 double *tt, cudaStream_t s);
+                                 double *tt, double2 *Ghost, cudaStream_t s);
 // Orthonormal basis U of every problem (Sec. 2.1; kUSize per problem, FP32 and the same
 // values in FP64) from the power sums sum_n r_n^k, k = 1 .. 2 B - 1, of r = |u|^2: exact
 // FP32 two-sum pairs within a warp, then FP64, in a fixed order (part: max(nprob,
@@ -119,8 +120,10 @@ int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
 // Equilibrated factorisation of every G: D G D = U Delta U^H, D = diag(G)^{-1/2}, U
 // unit lower triangular, Delta diagonal.  U per problem: K (K + 1) / 2 values packed
 // by rows, each an FP32 pair {re.hi, im.hi, re.lo, im.lo}, with 1 / Delta on the
-// diagonal; d: K per problem; info[p] = 0 or the failing pivot + 1.
-cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, int *status, cudaStream_t s);
+// diagonal; d: K per problem; info[p] = 0 or the failing pivot + 1.  Uhost, info_host:
+// copies of the first problem's factor and status in mapped host memory, or null.
+cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, float4 *Uhost,
+                        int *info_host, int *status, cudaStream_t s);
 // x = G^{-1} rhs using the factorisation (problems that did not factor are skipped).
 // Every pointer: `nprob` consecutive vectors, K apart unless stated.
 struct SolveIo {

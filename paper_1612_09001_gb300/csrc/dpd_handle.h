@@ -23,18 +23,18 @@ struct EstimateWorkspace {
     int *info = nullptr;
     float *tab = nullptr;         // [nprob][table_stride] forward tables of the current coefficients
     float2 *y = nullptr, *e = nullptr;
-    double *norm_part = nullptr;  // 2 * kFwdNormSlots partial sums, 2 results, a counter
+    double *norm_part = nullptr;  // 2 * kFwdNormSlots partial sums, a counter
     // orthogonal-polynomial basis (DPD_BASIS_ORTHOGONAL)
     float *ubasis = nullptr;      // [nprob][kUSize] basis coefficients used by the Gram kernels
     double *ubasis64 = nullptr;   // the same values in FP64, for the coefficient transforms
     double *mom_part = nullptr;   // [nprob][blocks][kMomK], max(nprob, kMomBlocks) rows in all
-    // pinned host copies read back by dpd_estimate (single problem)
+    // pinned, mapped host memory that the kernels of dpd_estimate write (single problem)
     int hK = 0;                   // K the host buffers were sized for
     double2 *h_G = nullptr;       // Gram matrix G, K x K (condition estimate on the host)
     float4 *h_U = nullptr;        // factor of D G D (launch_chol)
     int *h_info = nullptr;        // pivot status of the factorisation
     double *h_norm = nullptr;     // ||t - Psi h||^2, ||t||^2
-    cudaEvent_t ev_G = nullptr;   // h_G has landed
+    cudaEvent_t ev_G = nullptr;   // h_G is written
     // batched refinement (dpd_estimate_batched): work lists of the batched forward and
     // coefficient-gradient launches
     void *bstreams = nullptr;     // dpd::BatchStream [problems]
@@ -42,7 +42,7 @@ struct EstimateWorkspace {
     void *badj = nullptr;         // dpd::AdjArgs [problems]
     float2 *bpart = nullptr;      // coefficient-gradient partials, [problems][rows][K]
     size_t bprob_cap = 0, bitems_cap = 0, bpart_cap = 0;   // problems, items, rows
-    cudaEvent_t ev_U = nullptr;   // h_info (and h_U) have landed
+    cudaEvent_t ev_U = nullptr;   // h_info and h_U are written
 };
 
 // Device staging of dpd_apply_host's copy / compute pipeline, created on first use.

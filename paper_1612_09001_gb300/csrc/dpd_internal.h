@@ -73,12 +73,12 @@ struct FwdArgs {
     const HostTab *host_tab;   // host copy of the table (param-bank modes), or null
     const float2 *sub = nullptr;   // kModeSubtract: minuend, n samples, 16-byte aligned
     // kModeNorms: kFwdNormSlots partial sums (one float4 per CTA: the FP32
-    // (hi, lo) pairs of both sums, the size of two doubles), then the two
-    // results in FP64 (sum |sub - y|^2, sum |sub|^2), then a completion counter
-    // (an unsigned in the next double; zero between launches).  The last CTA to
-    // finish adds the partials in a fixed order, writes the results and clears
-    // the counter.
+    // (hi, lo) pairs of both sums, the size of two doubles), then a completion
+    // counter (an unsigned in the next double; zero between launches).  The last
+    // CTA to finish adds the partials in a fixed order, writes the results in FP64
+    // (sum |sub - y|^2, sum |sub|^2) to norms_out and clears the counter.
     double *norms = nullptr;
+    double *norms_out = nullptr;   // kModeNorms: the two results (mapped host memory allowed)
     // kHalo samples in front of x[0], replaced by those in front of the next
     // block, or null: zero history (bulk-copy kernel only).
     float2 *hist = nullptr;

@@ -57,9 +57,9 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsam
         ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K);
         ok = ok && grow(w.d, 0, np * K) && grow(w.tt, 0, np) && grow(w.info, 0, np);
         ok = ok && grow(w.tab, 0, np * table_stride(h));
-        // partial pairs, the two results, the completion counter (zero)
-        ok = ok && grow(w.norm_part, 0, (size_t)2 * dpd::kFwdNormSlots + 3) &&
-             cudaMemset(w.norm_part, 0, ((size_t)2 * dpd::kFwdNormSlots + 3) * sizeof(double)) == cudaSuccess;
+        // partial pairs, the completion counter (zero)
+        ok = ok && grow(w.norm_part, 0, (size_t)2 * dpd::kFwdNormSlots + 1) &&
+             cudaMemset(w.norm_part, 0, ((size_t)2 * dpd::kFwdNormSlots + 1) * sizeof(double)) == cudaSuccess;
         ok = ok && grow(w.ubasis, 0, np * dpd::kUSize) && grow(w.ubasis64, 0, np * dpd::kUSize);
         ok = ok && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         if (!ok) return DPD_ERR_ALLOC;
@@ -147,7 +147,7 @@ int gram_cpp(dpd_handle h, int nprob, int64_t n, int precision)
 // handle's estimate basis, or the monomials of Eq. 2 with `monomial`.
 dpd_status run_gram(dpd_handle h, int nprob, int cpp, int precision, cudaStream_t s,
                     const dpd::GramProblem *one = nullptr, double2 *G_out = nullptr, double2 *g_out = nullptr,
-                    bool monomial = false)
+                    bool monomial = false, double2 *G_host = nullptr)
 {
     EstimateWorkspace &w = h->est;
     dpd::GramArgs a;
@@ -167,18 +167,18 @@ dpd_status run_gram(dpd_handle h, int nprob, int cpp, int precision, cudaStream_
     const int D = dpd::gram_distinct(h->B, h->T);
     if (precision == dpd::kPrecFP32) {
         if (dpd::launch_gram_reduce(w.partials, nprob, cpp, D, w.S, s) != cudaSuccess ||
-            dpd::launch_gram_assemble(w.S, nprob, h->K, h->Bp, h->B, h->T, G, g, w.tt, s) != cudaSuccess)
+            dpd::launch_gram_assemble(w.S, nprob, h->K, h->Bp, h->B, h->T, G, g, w.tt, G_host, s) != cudaSuccess)
             return DPD_ERR_CUDA;
     } else if (dpd::launch_gram_lag_finish(w.partials, a.probs, a.one, a.ubasis, nprob, cpp, h->K, h->Bp, h->B, h->T,
-                                           nprob > 1, w.Clag, G, g, w.tt, s) != cudaSuccess) {
+                                           nprob > 1, w.Clag, G, g, w.tt, G_host, s) != cudaSuccess) {
         return DPD_ERR_CUDA;
     }
     return DPD_OK;
 }
 
 // e = t - Psi(u) h for the current coefficients of problem p (its table in w.tab; FP32
-// filter); with `norms`, only ||e||^2 and ||t||^2 into w.norm_part + 2 kFwdNormSlots
-// (e itself is not written).
+// filter); with `norms`, only ||e||^2 and ||t||^2 into the pinned w.h_norm (e itself is not
+// written).
 dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, int64_t n, cudaStream_t s,
                        bool norms = false)
 {
@@ -209,6 +209,7 @@ dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, in
         fa.y = w.e;
         fa.sub = t;
         fa.norms = w.norm_part;
+        fa.norms_out = w.h_norm;
         return dpd::launch_fwd_any(h->B, h->T, fa, L, h->sm_count, s) == cudaSuccess ? DPD_OK : DPD_ERR_CUDA;
     }
     if ((reinterpret_cast<uintptr_t>(u) & 15u) != 0) {
@@ -217,7 +218,7 @@ dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, in
     }
     if (dpd::launch_fwd_any(h->B, h->T, fa, L, h->sm_count, s) != cudaSuccess) return DPD_ERR_CUDA;
     if (norms)
-        return dpd::launch_residual_norm(t, w.y, n, nullptr, w.norm_part, w.norm_part + 2 * dpd::kFwdNormSlots, s) ==
+        return dpd::launch_residual_norm(t, w.y, n, nullptr, w.norm_part, w.h_norm, s) ==
                        cudaSuccess
                    ? DPD_OK
                    : DPD_ERR_CUDA;
@@ -608,21 +609,6 @@ double largest_inverse(const float4 *Up, int K)
 
 }  // namespace cond
 
-// Statistics of a problem: ||t - Psi h||^2 and ||t||^2 of the final
-// coefficients (FP32 residual summed in FP64 on the device), queued on s and
-// read back into the pinned w.h_norm.
-dpd_status queue_norms(dpd_handle h, int p, const float2 *u, const float2 *t, int64_t n, cudaStream_t s)
-{
-    EstimateWorkspace &w = h->est;
-    dpd_status st = residual_of(h, p, u, t, n, s, true);
-    if (st != DPD_OK) return st;
-    if (cudaMemcpyAsync(w.h_norm, w.norm_part + 2 * dpd::kFwdNormSlots, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                        s) !=
-        cudaSuccess)
-        return DPD_ERR_CUDA;
-    return DPD_OK;
-}
-
 dpd_status check_inputs(dpd_handle h, const void *u, const void *t, int64_t n, int precision)
 {
     if (!h || n < 1 || !u || !aligned8(u) || (t && !aligned8(t))) return DPD_ERR_INVALID_ARGUMENT;
@@ -709,28 +695,23 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     EstimateWorkspace &w = h->est;
     const dpd::GramProblem pr{static_cast<const float2 *>(u), static_cast<const float2 *>(t), n};
     if (ortho(h) && (st = compute_basis(h, &pr, 1, n, s)) != DPD_OK) return st;
-    if ((st = run_gram(h, 1, cpp, precision, s, &pr)) != DPD_OK) return st;
-    // For the statistics, G and (after the factorisation) the factor go
-    // to pinned host memory while the device carries on, and so does the pivot
-    // status: the host condition estimate (Lanczos on D G D from G, and on its
-    // inverse) runs during the factorisation and the refinement instead of
-    // after them, and the solves skip a failed factorisation on the device.
+    // For the statistics the kernels write G, the factor and the sums of squares to
+    // pinned host memory too (a copy in the stream would hold up the kernel behind it),
+    // and the pivot status: the host condition estimate (Lanczos on D G D from G, and on
+    // its inverse) runs during the factorisation and the refinement instead of after
+    // them, and the solves skip a failed factorisation on the device.
     const int K = h->K;
-    if (stats && (cudaMemcpyAsync(w.h_G, w.G, sizeof(double2) * K * K, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                  cudaEventRecord(w.ev_G, s) != cudaSuccess))
-        return DPD_ERR_CUDA;
-    if (dpd::launch_chol(w.G, 1, h->K, w.U, w.d, w.info, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if (cudaMemcpyAsync(w.h_info, w.info, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return DPD_ERR_CUDA;
-    if ((stats && cudaMemcpyAsync(w.h_U, w.U, sizeof(float4) * factor_size(K), cudaMemcpyDeviceToHost, s) !=
-                      cudaSuccess) ||
+    if ((st = run_gram(h, 1, cpp, precision, s, &pr, nullptr, nullptr, false, stats ? w.h_G : nullptr)) != DPD_OK)
+        return st;
+    if (stats && cudaEventRecord(w.ev_G, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol(w.G, 1, K, w.U, w.d, w.info, w.h_U, w.h_info, h->d_status, s) != cudaSuccess ||
         cudaEventRecord(w.ev_U, s) != cudaSuccess)
         return DPD_ERR_CUDA;
     float2 *out = static_cast<float2 *>(h_out);
     if ((st = solve(h, 0, 1, nullptr, 0, out, s)) != DPD_OK) return st;
     for (int i = 0; i < refine_iters; ++i)
         if ((st = refine_once(h, 0, pr.u, pr.t, n, out, s)) != DPD_OK) return st;
-    if (stats && (st = queue_norms(h, 0, pr.u, pr.t, n, s)) != DPD_OK) return st;
+    if (stats && (st = residual_of(h, 0, pr.u, pr.t, n, s, true)) != DPD_OK) return st;
     // The two Lanczos runs overlap the queued device work: the one on D G D
     // (a second host thread) as soon as G has landed, the one on the inverse
     // once the factor has.
@@ -789,7 +770,7 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
         return DPD_ERR_CUDA;
     if (ortho(h) && (st = compute_basis(h, nullptr, count, nmax, s)) != DPD_OK) return st;
     if ((st = run_gram(h, count, cpp, precision, s)) != DPD_OK) return st;
-    if (dpd::launch_chol(w.G, count, h->K, w.U, w.d, w.info, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol(w.G, count, h->K, w.U, w.d, w.info, nullptr, nullptr, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
     float2 *out = static_cast<float2 *>(h_out);
     if ((st = solve(h, 0, count, nullptr, 0, out, s)) != DPD_OK) return st;
     // The pivot status comes back here only for the refinement problem by

@@ -215,7 +215,8 @@ __device__ __forceinline__ double dot(const double *SPQ, ColRef x, ColRef y)
 }
 
 __global__ void gram_assemble_kernel(const double *__restrict__ Sall, int K, int Bp, int B, int T,
-                                     double2 *__restrict__ G, double2 *__restrict__ g, double *__restrict__ tt)
+                                     double2 *__restrict__ G, double2 *__restrict__ g, double *__restrict__ tt,
+                                     double2 *Ghost)
 {
     const int p = blockIdx.y;
     const double *S = Sall + (size_t)p * kGramS * kGramPartCols;
@@ -226,7 +227,9 @@ __global__ void gram_assemble_kernel(const double *__restrict__ Sall, int K, int
         ColRef ar, ai, br, bi;
         psi_column_refs(a, K, Bp, B, T, ar, ai);
         psi_column_refs(b, K, Bp, B, T, br, bi);
-        G[(size_t)p * K * K + idx] = make_double2(dot(S, ar, br) + dot(S, ai, bi), dot(S, ar, bi) - dot(S, ai, br));
+        const double2 v = make_double2(dot(S, ar, br) + dot(S, ai, bi), dot(S, ar, bi) - dot(S, ai, br));
+        G[(size_t)p * K * K + idx] = v;
+        if (Ghost && p == 0) Ghost[idx] = v;
     } else if (idx < K * K + K) {
         const int a = idx - K * K;
         ColRef ar, ai;
@@ -238,10 +241,10 @@ __global__ void gram_assemble_kernel(const double *__restrict__ Sall, int K, int
 }
 
 cudaError_t launch_gram_assemble(const double *S, int nprob, int K, int Bp, int B, int T, double2 *G, double2 *g,
-                                 double *tt, cudaStream_t s)
+                                 double *tt, double2 *Ghost, cudaStream_t s)
 {
     dim3 grid((K * K + K + 1 + 255) / 256, nprob);
-    gram_assemble_kernel<<<grid, 256, 0, s>>>(S, K, Bp, B, T, G, g, tt);
+    gram_assemble_kernel<<<grid, 256, 0, s>>>(S, K, Bp, B, T, G, g, tt, Ghost);
     count_launch();
     return cudaGetLastError();
 }

@@ -495,6 +495,7 @@ __global__ void __launch_bounds__(256) gram_lag_reduce_kernel(const float2 *__re
                                                               double *__restrict__ C)
 {
     __shared__ double grp[8][32];
+    grid_dep_wait();
     const int p = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int e = blockIdx.x * 32 + lane;
     double s = 0.0;
@@ -532,6 +533,7 @@ constexpr int kLagFew = 8;
 __global__ void __launch_bounds__(256) gram_lag_reduce_few_kernel(const float2 *__restrict__ partials, int cpp,
                                                                   double *__restrict__ C)
 {
+    grid_dep_wait();
     const int p = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
     if (e >= kLagEntries) return;
     const float2 *base = partials + (size_t)p * cpp * kLagEntries + e;
@@ -570,8 +572,9 @@ __global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__
                                                                 GramProblem one, const float *__restrict__ ubasis,
                                                                 int K, int Bp, int B, int T, int lower,
                                                                 double2 *__restrict__ G, double2 *__restrict__ g,
-                                                                double *__restrict__ tt)
+                                                                double *__restrict__ tt, double2 *Ghost)
 {
+    grid_dep_wait();
     __shared__ float xt[kLagSigA][kMaxT];   // x_s(N - 8 + i), zero before the record
     __shared__ float su_buf[kUSize];
     __shared__ int2 src[kGramS];             // (signal, tap) of each distinct column
@@ -674,7 +677,9 @@ __global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__
             ColRef ar, ai, br, bi;
             psi_column_refs(a, K, Bp, B, T, ar, ai);
             psi_column_refs(b, K, Bp, B, T, br, bi);
-            G[(size_t)p * K * K + idx] = make_double2(sum(dot(ar, br), dot(ai, bi)), diff(dot(ar, bi), dot(ai, br)));
+            const double2 v = make_double2(sum(dot(ar, br), dot(ai, bi)), diff(dot(ar, bi), dot(ai, br)));
+            G[(size_t)p * K * K + idx] = v;
+            if (Ghost && p == 0) Ghost[idx] = v;
         } else if (idx < K * K + K) {
             const int a = idx - K * K;
             ColRef ar, ai;
@@ -689,22 +694,22 @@ __global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__
 
 cudaError_t launch_gram_lag_finish(const float *partials, const GramProblem *probs, GramProblem one,
                                    const float *ubasis, int nprob, int cpp, int K, int Bp, int B, int T, bool lower,
-                                   double *C, double2 *G, double2 *g, double *tt, cudaStream_t s)
+                                   double *C, double2 *G, double2 *g, double *tt, double2 *Ghost, cudaStream_t s)
 {
     const float2 *parts = reinterpret_cast<const float2 *>(partials);
-    if (cpp <= kLagFew && nprob > 1)
-        gram_lag_reduce_few_kernel<<<dim3((kLagEntries + 255) / 256, nprob), 256, 0, s>>>(parts, cpp, C);
-    else
-        gram_lag_reduce_kernel<<<dim3((kLagEntries + 31) / 32, nprob), 256, 0, s>>>(parts, cpp, C);
-    count_launch();
+    const unsigned np = (unsigned)nprob;
+    const cudaError_t e =
+        cpp <= kLagFew && nprob > 1
+            ? launch_pdl(gram_lag_reduce_few_kernel, dim3((kLagEntries + 255) / 256, np), 256, 0, s, parts, cpp, C)
+            : launch_pdl(gram_lag_reduce_kernel, dim3((kLagEntries + 31) / 32, np), 256, 0, s, parts, cpp, C);
+    if (e != cudaSuccess) return e;
     // A block's start (the record's last samples in every signal) takes longer than an
     // entry: one entry per thread for one problem, about eight blocks per SM for many
     // (256 problems at K = 97: 45.4 us; 63.1 with one entry of the whole G per thread).
     const int full = (K * K + K + 1 + 255) / 256, share = 8 * 152 / nprob;
     const int blocks = share < 1 ? 1 : share < full ? share : full;
-    gram_lag_assemble_kernel<<<dim3(blocks, nprob), 256, 0, s>>>(C, probs, one, ubasis, K, Bp, B, T, lower ? 1 : 0, G, g, tt);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(gram_lag_assemble_kernel, dim3((unsigned)blocks, np), 256, 0, s, C, probs, one, ubasis, K, Bp, B, T,
+                      lower ? 1 : 0, G, g, tt, Ghost);
 }
 
 // ------------------------------------------------------------------ FP32 CUDA cores
