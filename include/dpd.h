@@ -230,6 +230,13 @@ dpd_status dpd_sq_error(dpd_handle h, const void *y, const void *x, int64_t n, f
                         double scale, float *loss, void *gy, void *stream);
 
 /*
+ * The gradient of dpd_sq_error's loss alone, times the gradient dl of what follows (one
+ * device float): gy[n] = dl 2 scale (y_n - g x_n).  Buffers as there; gy required.
+ */
+dpd_status dpd_sq_error_grad(dpd_handle h, const void *y, const void *x, int64_t n, float gain_re, float gain_im,
+                             double scale, const float *dl, void *gy, void *stream);
+
+/*
  * One Adam step (Kingma and Ba, Algorithm 1; no weight decay) of n float
  * parameters on the device, for coefficient vectors trained by direct learning:
  *   t = ++step, m = beta1 m + (1 - beta1) grad, v = beta2 v + (1 - beta2) grad^2,

@@ -54,6 +54,7 @@ SIGNATURES = {
     "dpd_apply_stream": [_vp, _vp, _vp, _i64, _vp],
     "dpd_set_estimate_basis": [_vp, _i],
     "dpd_sq_error": [_vp, _vp, _vp, _i64, ctypes.c_float, ctypes.c_float, ctypes.c_double, _vp, _vp, _vp],
+    "dpd_sq_error_grad": [_vp, _vp, _vp, _i64, ctypes.c_float, ctypes.c_float, ctypes.c_double, _vp, _vp, _vp],
     "dpd_adam_step": [_vp, _vp, _vp, _vp, _vp, _i64, _vp, ctypes.c_double, ctypes.c_double, ctypes.c_double, _vp],
     "dpd_reset_stream": [_vp, _vp],
     "dpd_set_fwd_launch": [_vp, _i, _i, _i, _i, _i, _i, _i],

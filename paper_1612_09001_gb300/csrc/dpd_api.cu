@@ -597,18 +597,33 @@ dpd_status dpd_apply_stream(dpd_handle h, const void *x, void *y, int64_t n, voi
     return apply_block(h, x, y, n, stream, h ? h->d_hist : nullptr);
 }
 
+// The buffers of the loss and its gradient.
+static bool sq_error_args(dpd_handle h, const void *y, const void *x, int64_t n, const void *gy)
+{
+    if (!h || n < 0) return false;
+    if (n > 0 && (!y || !x || !aligned(y, 8) || !aligned(x, 8))) return false;
+    if (n > (int64_t)(INT64_MAX / sizeof(float2))) return false;
+    const size_t bytes = (size_t)n * sizeof(float2);
+    return !gy || (aligned(gy, 8) && !overlap(gy, bytes, x, bytes) && !overlap(gy, bytes, y, bytes));
+}
+
 dpd_status dpd_sq_error(dpd_handle h, const void *y, const void *x, int64_t n, float gain_re, float gain_im,
                         double scale, float *loss, void *gy, void *stream)
 {
-    if (!h || n < 0 || !loss || !aligned(loss, 4)) return DPD_ERR_INVALID_ARGUMENT;
-    if (n > 0 && (!y || !x || !aligned(y, 8) || !aligned(x, 8))) return DPD_ERR_INVALID_ARGUMENT;
-    if (n > (int64_t)(INT64_MAX / sizeof(float2))) return DPD_ERR_INVALID_ARGUMENT;
-    const size_t bytes = (size_t)n * sizeof(float2);
-    if (gy && (!aligned(gy, 8) || overlap(gy, bytes, x, bytes) || overlap(gy, bytes, y, bytes)))
-        return DPD_ERR_INVALID_ARGUMENT;
+    if (!sq_error_args(h, y, x, n, gy) || !loss || !aligned(loss, 4)) return DPD_ERR_INVALID_ARGUMENT;
     return cuda_status(dpd::launch_sq_error(static_cast<const float2 *>(y), static_cast<const float2 *>(x), n,
                                             make_float2(gain_re, gain_im), scale, h->d_loss_part, loss,
                                             static_cast<float2 *>(gy), static_cast<cudaStream_t>(stream)));
+}
+
+dpd_status dpd_sq_error_grad(dpd_handle h, const void *y, const void *x, int64_t n, float gain_re, float gain_im,
+                             double scale, const float *dl, void *gy, void *stream)
+{
+    if (!sq_error_args(h, y, x, n, gy) || !dl || !aligned(dl, 4) || (n > 0 && !gy)) return DPD_ERR_INVALID_ARGUMENT;
+    if (n == 0) return DPD_OK;
+    return cuda_status(dpd::launch_sq_error_grad(static_cast<const float2 *>(y), static_cast<const float2 *>(x), n,
+                                                 make_float2(gain_re, gain_im), scale, dl, static_cast<float2 *>(gy),
+                                                 static_cast<cudaStream_t>(stream)));
 }
 
 dpd_status dpd_adam_step(float *param, const float *grad, float *m, float *v, float *step, int64_t n, const float *lr,

@@ -91,10 +91,13 @@ void free_host_pipeline(HostPipeline &p);
 
 
 namespace dpd {
-constexpr int kLossBlocks = 296;   // 2 per SM at 148-152 SMs
+constexpr int kLossBlocks = 304;   // 2 per SM at 152 SMs
 // loss[0] = (float)(scale * sum |y - g x|^2) (FP64 sum, fixed order); gy = 2 scale (y - g x) if non-null.
 cudaError_t launch_sq_error(const float2 *y, const float2 *x, int64_t n, float2 g, double scale, double *part,
                             float *loss, float2 *gy, cudaStream_t s);
+// gy = dl[0] 2 scale (y - g x): the gradient alone, times dL.
+cudaError_t launch_sq_error_grad(const float2 *y, const float2 *x, int64_t n, float2 g, double scale, const float *dl,
+                                 float2 *gy, cudaStream_t s);
 // One Adam step of n FP32 parameters; m, v: moments, step: the count (one float), advanced.
 cudaError_t launch_adam(float *param, const float *grad, float *m, float *v, float *step, int64_t n, const float *lr,
                         double beta1, double beta2, double eps, cudaStream_t s);

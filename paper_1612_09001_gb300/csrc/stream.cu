@@ -57,13 +57,14 @@ cudaError_t launch_stream_head(const float *tab, int B, int T, const float2 *x, 
 // Squared-error loss of direct learning and its gradient in one pass.  Each
 // thread sums |e|^2 as an FP32 (sum, rounding error) pair with an exact two-sum
 // per addition (about 2^-48 relative; FP64 runs at about two operations per clock
-// per SM on this GPU), or in FP64 where that leaves FP32's range; the threads'
-// totals are added in FP64 in a fixed order, and the last block to finish adds the
-// block sums in block order, writes the loss and clears the counter for the next
-// launch.  Four samples' loads in
-// flight per thread.  GB300, 2^20 samples from DRAM: 11.1 us (FP64 sums and a
-// second launch for the block sums: 11.4 + 4.4).
-constexpr int kLossThreads = 256;
+// per SM on this GPU), the warp adds its pairs, or its FP64 sums where a pair leaves
+// FP32's range; the warps' totals are added in FP64 in a fixed order, and the last
+// block to finish adds the block sums in block order, writes the loss and clears the
+// counter for the next launch.  Four samples' loads in
+// flight per thread.  GB300, 2^20 samples from DRAM, us: 9.3 without the
+// gradient (11.3 with the threads' totals added in FP64; 11.4 + 4.4 with FP64 sums and a
+// second launch for the block sums).
+constexpr int kLossThreads = 512;
 
 __global__ void __launch_bounds__(kLossThreads)
     sq_error_kernel(const float2 *__restrict__ y, const float2 *__restrict__ x, int64_t n, float2 g, double scale,
@@ -91,19 +92,21 @@ __global__ void __launch_bounds__(kLossThreads)
             }
         }
     }
-    double s = (double)acc.x + (double)acc.y;
-    if (!isfinite(acc.x)) {
+    __shared__ double red[kLossThreads / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2 w = acc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w = pair_add(w, shfl_xor_pair(w, o));
+    double s = (double)w.x + (double)w.y;
+    if (__any_sync(0xffffffffu, !isfinite(w.x))) {
         s = 0.0;
         for (int64_t i = (int64_t)blockIdx.x * kLossThreads + threadIdx.x; i < n; i += stride) {
             const float2 a = x[i], b = y[i];
             const float er = b.x - (g.x * a.x - g.y * a.y), ei = b.y - (g.x * a.y + g.y * a.x);
             s += (double)(er * er + ei * ei);
         }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
-    __shared__ double red[kLossThreads / 32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) red[warp] = s;
     __syncthreads();
     if (warp != 0) return;
@@ -129,6 +132,37 @@ __global__ void __launch_bounds__(kLossThreads)
     }
 }
 
+// The loss's gradient on its own, scaled by dL (one device float): gy = dL 2 scale (y - g x).
+__global__ void __launch_bounds__(kLossThreads)
+    sq_error_grad_kernel(const float2 *__restrict__ y, const float2 *__restrict__ x, int64_t n, float2 g, double scale,
+                         const float *__restrict__ dl, float2 *__restrict__ gy)
+{
+    grid_dep_wait();
+    const float s2 = (float)(2.0 * scale), l = dl[0];
+    const int64_t stride = (int64_t)gridDim.x * kLossThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * kLossThreads + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        float2 a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            a[q] = i < n ? x[i] : make_float2(0.f, 0.f);
+            b[q] = i < n ? y[i] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            const float er = b[q].x - (g.x * a[q].x - g.y * a[q].y), ei = b[q].y - (g.x * a[q].y + g.y * a[q].x);
+            if (i < n) gy[i] = make_float2(s2 * er * l, s2 * ei * l);
+        }
+    }
+}
+
+cudaError_t launch_sq_error_grad(const float2 *y, const float2 *x, int64_t n, float2 g, double scale, const float *dl,
+                                 float2 *gy, cudaStream_t s)
+{
+    return launch_pdl(sq_error_grad_kernel, dim3(kLossBlocks), kLossThreads, 0, s, y, x, n, g, scale, dl, gy);
+}
+
 cudaError_t launch_sq_error(const float2 *y, const float2 *x, int64_t n, float2 g, double scale, double *part,
                             float *loss, float2 *gy, cudaStream_t s)
 {
@@ -137,10 +171,21 @@ cudaError_t launch_sq_error(const float2 *y, const float2 *x, int64_t n, float2 
 
 // One Adam step (Kingma and Ba, "Adam: A Method for Stochastic Optimization",
 // Algorithm 1) of a short parameter vector, in FP64 between the FP32 loads and
-// stores.  One block: it has the step count to advance.  beta^t comes from
-// repeated squaring (t is a whole number), about 2 log2 t FP64 products instead
-// of pow()'s hundreds of FP64 operations, which at FP64's rate on this GPU made
-// the library optimiser's step 39.4 us; here 7.5 us (66 parameters).
+// stores.  One block: it has the step count to advance.  beta^t comes from repeated
+// squaring (t is a whole number), about 2 log2 t FP64 products, and the roots and the
+// quotient from Newton-Raphson steps on FP32 estimates: an FP64 operation takes 64
+// cycles on this GPU, and pow(), square root and division are tens to hundreds of them
+// (the library optimiser's step took 39.4 us; here 6.1 us from cold caches, 7.5 with the functions
+// called).
+__device__ __forceinline__ double inv_newton(double x)   // 1 / x, x > 0
+{
+    if (!(x > 1e-30 && x < 1e30)) return 1.0 / x;
+    double y = (double)(1.f / (float)x);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(y, fma(-x, y, 1.0), y);
+    return y;
+}
+
 __global__ void __launch_bounds__(256)
     adam_kernel(float *__restrict__ param, const float *__restrict__ grad, float *__restrict__ m,
                 float *__restrict__ v, float *__restrict__ step, int64_t n, const float *__restrict__ lr, double beta1,
@@ -163,14 +208,17 @@ __global__ void __launch_bounds__(256)
         p = pow(base, (double)t);
     }
     const double c1 = 1.0 - __shfl_sync(0xffffffffu, p, 0), c2 = 1.0 - __shfl_sync(0xffffffffu, p, 1);
-    const double rate = (double)lr[0] / c1, inv2 = 1.0 / sqrt(c2);
+    // 1 - beta^t > 0; sqrt(v / c2) = v / sqrt(v c2)
+    const double rate = (double)lr[0] * inv_newton(c1);
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
         const double gd = (double)grad[i];
         const double mi = beta1 * (double)m[i] + (1.0 - beta1) * gd;
         const double vi = beta2 * (double)v[i] + (1.0 - beta2) * gd * gd;
         m[i] = (float)mi;
         v[i] = (float)vi;
-        param[i] = (float)((double)param[i] - rate * mi / (sqrt(vi) * inv2 + eps));
+        const double root = vi > 0.0 ? vi * inv_sqrt(vi * c2) : sqrt(vi);
+        const double den = root + eps;
+        param[i] = (float)((double)param[i] - (den > 0.0 ? rate * mi * inv_newton(den) : rate * mi / den));
     }
 }
 

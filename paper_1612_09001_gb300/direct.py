@@ -29,21 +29,26 @@ from .autograd import DPDFunction
 
 
 class SqErrorLoss(torch.autograd.Function):
-    """L = scale * ||y - gain x||^2 with its gradient produced in the same device
-    pass (dpd_sq_error); backward scales the saved gradient by dL."""
+    """L = scale * ||y - gain x||^2 (dpd_sq_error); backward forms the gradient from the
+    same y and x, scaled by dL, in one pass (dpd_sq_error_grad)."""
 
     @staticmethod
     def forward(ctx, y, x, filt, gain, scale):
-        gy = torch.empty_like(y)
-        loss = filt.sq_error(y, x, gain=gain, scale=scale, gy=gy)
-        ctx.save_for_backward(gy)
+        loss = filt.sq_error(y, x, gain=gain, scale=scale)
+        ctx.save_for_backward(y, x)
+        ctx.args = filt, complex(gain), float(scale)
         return loss[0]
 
     @staticmethod
     def backward(ctx, gl):
-        (gy,) = ctx.saved_tensors
-        # real by real: the complex product's kernel takes twice as long
-        return torch.view_as_complex(torch.view_as_real(gy) * gl), None, None, None, None
+        y, x = ctx.saved_tensors
+        filt, g, scale = ctx.args
+        gl = gl.to(device=y.device, dtype=torch.float32)   # as it comes, unless a caller passed another kind
+        gy = torch.empty_like(y)
+        _lib.check("dpd_sq_error_grad", lib().dpd_sq_error_grad(
+            filt.handle, y.data_ptr(), x.data_ptr(), y.numel(), g.real, g.imag, scale, gl.data_ptr(), gy.data_ptr(),
+            _stream_ptr(None)))
+        return gy, None, None, None, None
 
 
 class Transmitter:

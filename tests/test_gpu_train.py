@@ -39,7 +39,7 @@ def test_adam_step_against_fp64(n, t0):
         assert np.all(np.abs(got.cpu().numpy() - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-44)
 
 
-@pytest.mark.parametrize("n", [1, 31, 256, 257, 4 * 296 * 256, 4 * 296 * 256 + 1, 300007])
+@pytest.mark.parametrize("n", [1, 31, 256, 257, 4 * 304 * 512, 4 * 304 * 512 + 1, 300007])
 def test_sq_error_block_edges(n):
     y, x = synth.ofdm2(n, key=(131, n)), synth.ofdm2(n, key=(132, n))
     f = dpd.DPD(1, 0, 0)
@@ -51,13 +51,18 @@ def test_sq_error_block_edges(n):
         ref = 0.5 * np.sum(np.abs(e) ** 2)
         assert abs(float(loss[0]) - ref) <= 1e-6 * ref
         assert np.abs(gy.cpu().numpy() - e).max() <= 1e-6 * np.abs(e).max()
+    dl = torch.tensor(-1.75, device="cuda")   # the gradient alone, times dL
+    _lib.check("dpd_sq_error_grad", dpd.lib().dpd_sq_error_grad(
+        f.handle, yd.data_ptr(), xd.data_ptr(), n, 0.95, -0.02, 0.5, dl.data_ptr(), gy.data_ptr(),
+        torch.cuda.current_stream().cuda_stream))
+    assert np.abs(gy.cpu().numpy() + 1.75 * e).max() <= 1e-6 * np.abs(e).max()
     f.close()
 
 
 @pytest.mark.parametrize("big", [3e19, float("inf")])
 def test_sq_error_outside_fp32_sums(big):
     """Squares whose FP32 sum overflows are summed in FP64; an infinity stays one."""
-    x = torch.zeros(400000, dtype=torch.complex64, device="cuda")   # four or more samples per thread
+    x = torch.zeros(800000, dtype=torch.complex64, device="cuda")   # four or more samples per thread
     y = torch.full_like(x, 1e19 if big != float("inf") else 1.0)
     y[::7777] = big if big == float("inf") else 1e19
     f = dpd.DPD(1, 0, 0)
@@ -65,7 +70,7 @@ def test_sq_error_outside_fp32_sums(big):
     if big == float("inf"):
         assert loss == float("inf")
     else:
-        assert abs(loss - 4e37) <= 1e-5 * 4e37   # 4e5 samples of 1e38, scale 1e-6
+        assert abs(loss - 8e37) <= 1e-5 * 8e37   # 8e5 samples of 1e38, scale 1e-6
     f.close()
 
 
