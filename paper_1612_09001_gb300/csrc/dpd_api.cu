@@ -304,27 +304,49 @@ dpd_status dpd_set_coeffs(dpd_handle h, const void *coeffs, int K, int where, vo
     return DPD_OK;
 }
 
-// Launch shape for n samples.  With the default shape, an input too short to
-// give every SM a few tiles gets 4 samples per thread and fewer warps per tile
-// (tiles of 128 to 512 samples): such calls are bound by latency, and more,
-// smaller tiles spread them over more SMs.
+// Launch shape for n samples (the default shape; one set explicitly stays).  The cost of
+// a sample is B T quadruples of multiply-adds against 16 bytes, so the choice goes by
+// B T, by the samples per SM, and by where the coefficients come from: 8 samples per
+// thread need the fewest instructions, but their window loads are 4-way bank conflicts
+// and with a table in shared memory they spill; 6 have neither; 4 give the most CTAs.
+// GB300 (152 SMs), us, the alternatives at the lines drawn below:
+//   V = 4, 4 warps and fewer: short inputs, bound by latency and spread over more SMs
+//     (2^18 samples, B T = 16: 2.5 against 2.8 for tiles of 3,072), and models of little
+//     arithmetic (2^23, B T = 6: 18.9 against 23.4 for V = 8; 8 warps past 2^23, B T = 9:
+//     43.7 against 48.1 at 2^24)
+//   V = 6, 4 warps: the middle (2^21, B T = 16: 6.9 against 7.6 for V = 4; B T = 25 9.2
+//     against 9.8; 3 2^20, B T = 48 20.2 against 23.1 for V = 8)
+//   V = 6, 16 warps in groups of 8: long inputs (2^23, B T = 48: 50.8 against 52.6 for V
+//     = 8; 2^24, B T = 15 42.4 against 44.5), for tables in shared memory above all (2^22,
+//     B T = 48: 29.3 against 41.5; 2^24, B T = 25 63.4 against 72.2), with fewer warps
+//     where there is little arithmetic (2^24, B T = 9: 43.4 against 47.6)
+//   V = 8, 16 warps in groups of 4: long inputs at B T = 20 .. 25 with coefficients in the
+//     parameter bank, whose multiply-adds fill the pipe (2^24, B T = 25: 54.4 against 57.7)
 static dpd::FwdLaunch launch_for(dpd_handle h, int64_t n, bool param_tab)
 {
     dpd::FwdLaunch L = h->fwd;
     if (!param_tab) L.mode &= ~dpd::kModeParamCoef;
-    const int64_t tile = (int64_t)L.warps * 32 * L.V;
-    if (h->fwd_auto && (n + tile - 1) / tile < 4 * (int64_t)h->sm_count) {
-        L.V = 4;
-        L.warps = 1;
+    if (!h->fwd_auto) return L;
+    const int64_t per = n / h->sm_count;   // samples per SM
+    const int bt = h->B * h->T;
+    const bool light = bt <= (param_tab ? 12 : 4);
+    auto shape = [&](int V, int warps, int stages, int group) {
+        L.V = V;
+        L.warps = warps;
+        L.stages = stages;
+        L.group = group;
+        return L;
+    };
+    if (light && per >= 80000) return shape(4, 8, 3, 0);
+    if (light || per < (param_tab ? 8500 : 3000)) {
         for (int w : {4, 2})
-            if ((n + w * 128 - 1) / (w * 128) * 2 >= 3 * (int64_t)h->sm_count) {
-                L.warps = w;
-                break;
-            }
-        L.stages = L.warps >= 4 ? 3 : 2;
-        L.group = 0;
+            if ((n + w * 128 - 1) / (w * 128) * 2 >= 3 * (int64_t)h->sm_count) return shape(4, w, w == 4 ? 3 : 2, 0);
+        return shape(4, 1, 2, 0);
     }
-    return L;
+    if (!param_tab && bt < 12) return per < 80000 ? shape(6, 4, 3, 0) : shape(6, 8, 2, 4);
+    if (per < 24000) return shape(6, 4, 3, 0);
+    if (param_tab && bt >= 20 && bt <= 25) return L;
+    return shape(6, 16, 4, 8);
 }
 
 // y = DPD(x) with the samples in `hist` in front of x[0], which is updated, or

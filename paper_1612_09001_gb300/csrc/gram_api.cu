@@ -191,16 +191,18 @@ dpd_status residual_of(dpd_handle h, int p, const float2 *u, const float2 *t, in
     fa.status = h->d_status;
     fa.vec_store = 1;
     fa.host_tab = nullptr;
-    // Coefficients live on the device (shared-memory table): 6 samples per
-    // thread, 16 warps in two groups of 8, 4 stages (measured best for these
-    // shapes on GB300: 31.6 us per 2^22 samples at P = Q = 11, M = 7, against
-    // about 42 at the single-stream default of 8 samples per thread).
+    // Coefficients live on the device (shared-memory table): 6 samples per thread, 16
+    // warps in two groups of 8, 4 stages (GB300, us per 2^22 samples at P = Q = 11, M = 7:
+    // 29.3, against 41.5 at the single-stream default of 8 samples per thread); fewer than
+    // eight tiles of 3,072 samples per SM go to CTAs of 4 warps (an estimate of 2^18 samples
+    // at P = Q = 7, M = 3: 151.0 us against 154.3, with 86 tiles for 152 SMs).
     dpd::FwdLaunch L;
+    const bool few = n < 8 * 3072 * (int64_t)h->sm_count;
     L.mode = dpd::kModePackedFma;
     L.V = 6;
-    L.warps = 16;
-    L.group = 8;
-    L.stages = 4;
+    L.warps = few ? 4 : 16;
+    L.group = few ? 0 : 8;
+    L.stages = few ? 3 : 4;
     const bool aligned16 = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(t)) & 15u) == 0;
     if (aligned16) {
         // The filter writes e = t - Psi(u) h itself (no separate residual
