@@ -399,7 +399,8 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
     // Host copies of the first problem, whichever kernel factored it.
     auto to_host = [&](int status) {
         if (p != 0 || !Uhost) return;
-        for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = Uall[e];
+#pragma unroll 8
+        for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = __ldcg(Uall + e);
         if (tid == 0) *info_host = status;
     };
     const int before = info[p];
