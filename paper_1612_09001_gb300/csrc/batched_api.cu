@@ -28,6 +28,16 @@ struct dpd_plan_s {
 
 namespace {
 
+// An item's sub-blocks in BatchItem::tile: first * 4 + (count - 1).
+constexpr int64_t kMaxBlocks = (int64_t)1 << 29;
+int batch_tile(int64_t block, int nsub) { return (int)(block * 4 + nsub - 1); }
+
+// Whether the launch runs one CTA per SM (its ring takes more than half of the shared memory).
+bool one_per_sm(int V, int warps, int group, int stages, int nsub)
+{
+    return dpd::batch_smem(warps, group > 0 ? group : warps, stages, V, nsub) > dpd::kBatchSmemMax / 2;
+}
+
 int nbranch(int order) { return order > 0 ? (order + 1) / 2 : 0; }
 bool aligned(const void *p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 bool overlap(const void *a, size_t na, const void *b, size_t nb)
@@ -36,21 +46,19 @@ bool overlap(const void *a, size_t na, const void *b, size_t nb)
     return na && nb && x < y + nb && y < x + na;
 }
 
-// Launch shape of a new plan.  Long batches: 6 samples per thread (the 16-byte
-// window loads of a quarter warp on distinct banks), 16 warps in groups of 4,
-// items of 12,288 samples.  That needs enough items that the last round of
-// them is a small part of a CTA's work, so batches with fewer than four such
-// items per SM take 4 samples per thread, 4 warps and items of 2,048 samples
-// on as many CTAs as fit an SM.  GB300, us per launch, first shape / second
-// shape / 8 samples per thread on 8 warps (items of 8,192): 64 streams, 36.7 M
-// samples 140.8 / 150 / 217.7; 24 streams, 12.2 M 56.2 / 57.7 / 89.3; 33
-// streams, 3.8 M 40.1 / 29.1 / 49.5; 16 streams, 1.3 M 19.3 / 17.5 / 23.1; 8
-// streams, 0.17 M 17.3 / 10.9 / 15.1.
+// Launch shape of a new plan.  6 samples per thread (the 16-byte window loads of a
+// quarter warp on distinct banks) and 16 warps in groups of 4, one CTA per SM with a
+// run of items of up to 12,288 samples.  Batches that leave an SM fewer than 8,192
+// samples are bound by latency and take 4 samples per thread, 4 warps and items of 2,048
+// samples on as many CTAs as fit an SM.  GB300, us per launch, first shape / second shape
+// / 8 samples per thread on 8 warps with items of 8,192 dealt out in order: 64 streams,
+// 36.7 M samples 125.9 / 150 / 217.7; 24 streams, 12.2 M 47.7 / 57.7 / 89.3; 33 streams, 3.8 M
+// 25.5 / 27.3 / 49.5; 16 streams, 1.3 M 16.9 / 17.1 / 23.1; 8 streams, 0.17 M 12.8 / 11.1 / 15.1.
 void default_shape(dpd_plan p)
 {
-    int64_t units = 0;   // of 1024 samples; an item of the first shape has 12
+    int64_t units = 0;   // of 1024 samples
     for (const dpd::BatchStream &st : p->streams) units += st.n / 1024;
-    const bool large = units >= 4 * 12 * (int64_t)p->sm_count;
+    const bool large = units >= 8 * (int64_t)p->sm_count;
     p->V = large ? 6 : 4;
     p->warps = large ? 16 : 4;
     p->stages = large ? 2 : 3;
@@ -68,14 +76,19 @@ void free_plan(dpd_plan p)
     delete p;
 }
 
-// Work list for tile size S = nsub * warps * 32 * V: streams by decreasing per-sample
-// cost (B * T), every tile of a stream in order.  Launched CTAs take items
-// round-robin.  The list goes to a new device buffer that replaces the plan's
-// only once it holds the list, so on failure the plan keeps its previous list
-// (and tiling) unchanged.
-dpd_status build_items(dpd_plan p, int V, int warps, int nsub)
+// Work list: streams by decreasing per-sample cost (B * T), in items of up to nsub
+// sub-blocks of warps * 32 * V samples.  CTA b of a launch of G takes items b, b + G, ...
+// With a CTA per SM (`contiguous`) those are one run of the ordered list of equal cost
+// for each CTA, so a CTA stays with one model's code (the kernel holds one unrolled
+// body per model, and its instruction fetch was an eighth of the stalls) and the SMs
+// with little arithmetic per sample move their bytes while the others compute: 64
+// streams of mixed models, 36.7 M samples, 121.4 us against 126.0 with full items
+// dealt out in order.  The list goes to a new device buffer that replaces the plan's only
+// once it holds the list, so on failure the plan keeps its previous list (and tiling)
+// unchanged.
+dpd_status build_items(dpd_plan p, int V, int warps, int nsub, bool contiguous)
 {
-    const int S = nsub * warps * 32 * V;
+    const int block = warps * 32 * V;
     std::vector<int> order(p->streams.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     // Costliest models first (B T per sample), and streams of the same model
@@ -87,10 +100,47 @@ dpd_status build_items(dpd_plan p, int V, int warps, int nsub)
         return p->streams[a].B > p->streams[b].B;
     });
     std::vector<dpd::BatchItem> items;
+    auto put = [&](std::vector<dpd::BatchItem> &list, int si, int64_t from, int64_t count) {
+        for (int64_t b = from; b < from + count; b += nsub)
+            list.push_back({si, batch_tile(b, (int)std::min<int64_t>(nsub, from + count - b))});
+    };
+    double total = 0.0;
+    // Cost of a sample: 4 B T multiply-adds, and what a sample takes besides them (about
+    // the time of 28: one model at a time over 5.6 M samples, us per launch, 60
+    // multiply-adds 18.6, 100 26.7, 140 32.9).
+    auto cost = [&](int si) { return 4.0 * p->streams[si].B * p->streams[si].T + 28.0; };
     for (int si : order) {
-        const int64_t nt = (p->streams[si].n + S - 1) / S;
-        if (nt > INT32_MAX) return DPD_ERR_UNSUPPORTED;
-        for (int64_t t = 0; t < nt; ++t) items.push_back({si, (int)t});
+        if ((p->streams[si].n + block - 1) / block > kMaxBlocks) return DPD_ERR_UNSUPPORTED;
+        total += cost(si) * (double)p->streams[si].n;
+    }
+    const int G = p->sm_count;
+    if (!contiguous || total <= 0.0) {
+        for (int si : order) put(items, si, 0, (p->streams[si].n + block - 1) / block);
+    } else {
+        std::vector<std::vector<dpd::BatchItem>> run((size_t)G);
+        int k = 0;            // the CTA being filled
+        double done = 0.0;    // cost given out
+        for (int si : order) {
+            const int64_t n = p->streams[si].n, blocks = (n + block - 1) / block;
+            const double c = cost(si) * block;   // of a sub-block
+            for (int64_t b = 0; b < blocks;) {
+                const double room = total / G * (k + 1) - done;
+                int64_t take = blocks - b;
+                if (k < G - 1) take = std::min(take, (int64_t)(room / c + 0.5));
+                if (take <= 0) {
+                    ++k;
+                    continue;
+                }
+                put(run[(size_t)k], si, b, take);
+                b += take;
+                done += b < blocks ? c * (double)take : c * (double)take - cost(si) * (double)(blocks * block - n);
+            }
+        }
+        size_t rounds = 0;
+        for (const auto &r : run) rounds = std::max(rounds, r.size());
+        items.assign(rounds * (size_t)G, {-1, -1});   // the end of a CTA's list
+        for (int b = 0; b < G; ++b)
+            for (size_t r = 0; r < run[(size_t)b].size(); ++r) items[r * (size_t)G + b] = run[(size_t)b][r];
     }
     if (items.size() > (size_t)INT32_MAX) return DPD_ERR_UNSUPPORTED;
     dpd::BatchItem *d_new = nullptr;
@@ -189,7 +239,7 @@ dpd_status dpd_plan_batched(const dpd_stream_desc *descs, int count, int where, 
         return DPD_ERR_CUDA;
     }
     default_shape(p);
-    dpd_status st = build_items(p, p->V, p->warps, p->nsub);
+    dpd_status st = build_items(p, p->V, p->warps, p->nsub, one_per_sm(p->V, p->warps, p->group, p->stages, p->nsub));
     if (st == DPD_OK && cudaDeviceSynchronize() != cudaSuccess) st = DPD_ERR_CUDA;
     if (st != DPD_OK) {
         free_plan(p);
@@ -208,10 +258,12 @@ dpd_status dpd_plan_set_launch(dpd_plan p, int V, int warps, int stages, int cta
     const int gw = group > 0 ? group : warps;
     if (dpd::batch_smem(warps, gw, stages, V) > dpd::kBatchSmemMax) return DPD_ERR_UNSUPPORTED;
     const int nsub = dpd::batch_nsub(warps, gw, stages, V);
-    if (V != p->V || warps != p->warps || nsub != p->nsub) {
+    const bool single = one_per_sm(V, warps, group, stages, nsub);
+    if (V != p->V || warps != p->warps || nsub != p->nsub ||
+        single != one_per_sm(p->V, p->warps, p->group, p->stages, p->nsub)) {
         // Re-tile first: the new shape is kept only once its work list is on
         // the device; on failure the plan runs with its previous shape.
-        const dpd_status st = build_items(p, V, warps, nsub);
+        const dpd_status st = build_items(p, V, warps, nsub, single);
         if (st != DPD_OK) return st;
     }
     p->V = V;

@@ -1,8 +1,8 @@
 // Batched APH DPD: many independent antenna streams of uneven length and
 // model order (P, Q, M) filtered by ONE persistent launch.
 //
-// The host plan cuts every stream into tiles of S samples and orders the
-// (stream, tile) work items by cost; CTA b takes items b, b + grid, ...  One
+// The host plan cuts every stream into work items of a few sub-blocks and orders
+// them; CTA b takes items b, b + grid, ...  One
 // producer thread per CTA streams each item into a shared-memory ring slot
 // with two bulk copies completed on the slot's mbarrier: the stream's
 // widely-linear coefficient table (see dpd_internal.h) and the tile with its
@@ -29,10 +29,15 @@ struct BatchStream {
     const float2 *sub = nullptr;   // if set, y = sub - filter output (a least-squares residual)
 };
 
+// Work item: sub-blocks [tile / 4, tile / 4 + tile % 4 + 1) of a stream, a sub-block
+// being one run of V samples per consumer thread of the CTA (batch_item packs the
+// pair).  An item of -1, -1 ends the list of the CTA that takes it.
 struct BatchItem {
     int stream;
     int tile;
 };
+constexpr int kBatchMaxSub = 4;
+__host__ __device__ constexpr int batch_tile(int64_t block, int nsub) { return (int)(block * kBatchMaxSub + nsub - 1); }
 
 struct BatchArgs {
     const BatchStream *streams;
@@ -43,7 +48,7 @@ struct BatchArgs {
     int64_t tab_floats;   // size of the table pool
     int *status;
     int gw = 0;           // consumer warps per group (0: one group of all warps)
-    int nsub = 1;         // sub-blocks of V samples per thread and item
+    int nsub = 1;         // sub-blocks per item at most
 };
 
 constexpr int kBatchTabBytes = ((kMaxTabFloats * 4 + 15) / 16) * 16;   // table area of a slot
@@ -55,7 +60,8 @@ struct BatchSlotHeader {
     int64_t n;     // stream length
     int64_t s0;    // first sample of the tile
     int bt;        // B * 16 + T
-    int ok;        // item passed item_ok (else skipped by both sides)
+    int ok;        // item passed item_ok (0: skipped by both sides; -1: end of the CTA's list)
+    int nsub;      // sub-blocks of the item
     const float2 *sub;   // the stream's subtrahend or null
 };
 constexpr int kBatchHdrBytes = 64;
@@ -71,12 +77,12 @@ __host__ __device__ constexpr size_t batch_slot_bytes(int S)
 // the pool and the slot, tile inside the stream, 16-byte aligned input).  The
 // producer and the consumers evaluate the same predicate on the same item, so
 // a bad item is skipped by both sides and no wait is left unmatched.
-__device__ __forceinline__ bool item_ok(const BatchArgs &a, const BatchItem &w, const BatchStream &st, int S)
+__device__ __forceinline__ bool item_ok(const BatchArgs &a, const BatchItem &w, const BatchStream &st, int block)
 {
     return w.stream >= 0 && w.stream < a.nstreams && st.tab_off >= 0 && st.tab_bytes > 0 &&
            st.tab_bytes <= kBatchTabBytes && (st.tab_bytes & 15) == 0 && (st.tab_off & 3) == 0 &&
            (int64_t)st.tab_off + st.tab_bytes / 4 <= a.tab_floats && w.tile >= 0 &&
-           (int64_t)w.tile * S < st.n && ((reinterpret_cast<uintptr_t>(st.x) & 15u) == 0);
+           w.tile % kBatchMaxSub < a.nsub && (int64_t)(w.tile / kBatchMaxSub) * block < st.n && ((reinterpret_cast<uintptr_t>(st.x) & 15u) == 0);
 }
 
 template <int B, int T, int V>
@@ -109,7 +115,7 @@ __device__ __forceinline__ void batched_item(const unsigned char *slot, const Ba
 #define DPD_BCASE(b, t)                                                                            \
     case (b) * 16 + (t):                                                                           \
         if constexpr ((b) <= BMAX && (t) <= TMAX) {                                                \
-            for (int sb = 0; sb < a.nsub; ++sb)                                                    \
+            for (int sb = 0; sb < hd.nsub; ++sb)                                                   \
                 batched_item<(b), (t), V>(slot, hd, SG, sb * gw * 32 + t_in_tile);                 \
             break;                                                                                 \
         }                                                                                          \
@@ -129,9 +135,7 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
     // per group g: full[s] at bars[2 stages g + s], empty[s] at bars[2 stages g + stages + s]
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
     unsigned char *ring = smem + ((2 * ngroups * stages * 8 + 127) / 128) * 128;
-    const int S = a.nsub * nwarps * 32 * V;   // the item's tile
-    const int SG = a.nsub * gw * 32 * V;      // a group's part of it: nsub sub-blocks of gw * 32 * V
-    const size_t slot_bytes = batch_slot_bytes(SG);
+    const size_t slot_bytes = batch_slot_bytes(a.nsub * gw * 32 * V);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
@@ -157,8 +161,12 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
         for (int i = blockIdx.x; i < a.nitems && gfail < 0; i += gridDim.x, ++it) {
             const BatchItem w = a.items[i];
             const BatchStream st = a.streams[(w.stream >= 0 && w.stream < a.nstreams) ? w.stream : 0];
-            const bool good = item_ok(a, w, st, S);
-            if (!good) atomicOr(a.status, kFlagBadWork);
+            const bool end = w.stream == -1 && w.tile == -1;
+            const bool good = !end && item_ok(a, w, st, nwarps * 32 * V);
+            if (!good && !end) atomicOr(a.status, kFlagBadWork);
+            const int nsub = good ? w.tile % kBatchMaxSub + 1 : 0;
+            const int SG = nsub * gw * 32 * V;   // a group's part of the item
+            const int64_t first = (int64_t)(w.tile / kBatchMaxSub) * (nwarps * 32 * V);
             for (int g = 0; g < ngroups; ++g) {
                 uint64_t *gb = bars + 2 * stages * g;
                 if (it >= stages && !mbar_wait(smem_addr(&gb[stages + s]), ph ^ 1u, a.status)) {
@@ -169,13 +177,14 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
                 const uint32_t fb = smem_addr(&gb[s]);
                 unsigned char *slot = ring + ((size_t)g * stages + s) * slot_bytes;
                 BatchSlotHeader *hd = reinterpret_cast<BatchSlotHeader *>(slot);
-                const int64_t s0 = (int64_t)w.tile * S + (int64_t)g * SG;
+                const int64_t s0 = first + (int64_t)g * SG;
                 hd->x = st.x;
                 hd->y = st.y;
                 hd->n = st.n;
                 hd->s0 = s0;
                 hd->bt = st.B * 16 + st.T;
-                hd->ok = good ? 1 : 0;
+                hd->ok = good ? 1 : end ? -1 : 0;
+                hd->nsub = nsub;
                 hd->sub = st.sub;
                 if (!good) {
                     mbar_arrive_expect_tx(fb, 0);   // complete the phase with no copies (releases the header)
@@ -200,6 +209,7 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
                         smem_addr(slot + kBatchHdrBytes + kBatchTabBytes + (size_t)off * sizeof(float2)), st.x + lo,
                         xbytes, fb, pol);
             }
+            if (end) break;
             if (gfail < 0 && ++s == stages) {
                 s = 0;
                 ph ^= 1u;
@@ -228,7 +238,9 @@ __global__ void __launch_bounds__(32 * 17) fwd_batched_kernel(BatchArgs a, int s
         if (!mbar_wait(smem_addr(&gb[s]), ph, a.status)) return;
         const unsigned char *slot = ring + ((size_t)g * stages + s) * slot_bytes;
         const BatchSlotHeader &hd = *reinterpret_cast<const BatchSlotHeader *>(slot);   // read in place
+        if (hd.ok < 0) break;   // nothing follows: the slot needs no release
         bool bad = hd.ok == 0;
+        const int SG = hd.nsub * gw * 32 * V;
         if (!bad && hd.s0 < hd.n) switch (hd.bt) {   // a group past the stream's end has nothing to do
             DPD_BCASES(1)
             DPD_BCASES(2)

@@ -292,7 +292,7 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     for (int p = 0; p < count; ++p) {
         float2 *ep = w.e + (size_t)p * stride;
         st[p] = {probs[p].u, ep, probs[p].n, h->B, h->T, p * tstride, tstride * 4, probs[p].t};   // e = t - Psi h
-        for (int64_t t = 0; t * S < probs[p].n; ++t) items.push_back({p, (int)t});
+        for (int64_t t = 0; t * S < probs[p].n; ++t) items.push_back({p, dpd::batch_tile(t * nsub, nsub)});
         dpd::AdjArgs &a = adj[p];
         a.x = probs[p].u;
         a.gy = ep;
