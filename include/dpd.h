@@ -307,12 +307,11 @@ enum { DPD_BASIS_MONOMIAL = 0, DPD_BASIS_ORTHOGONAL = 1 };
  *       psi_p(x) = sum_{m <= p} u_{m,p} |x|^{m-1} x, with u_{m,p} computed from
  *       the estimation input itself: the power sums of |u|^2 give the Gram
  *       matrix of the monomials, whose Cholesky factor L yields U = L^{-T}
- *       (FP64 on the host), so the basis functions are orthonormal over u.
+ *       (FP64 on the device), so the basis functions are orthonormal over u.
  *       Both branches and every tap use the same U.  The Gram matrix is
  *       formed and solved in that basis (much better conditioned), and the
  *       coefficients are converted back, h = W h_orth, so the output is always
  *       in the monomial stacking order of Sec. 2.2 that dpd_set_coeffs takes.
- *       One extra synchronisation per call (the power sums are read back).
  * dpd_gram always uses the monomials.
  */
 dpd_status dpd_set_estimate_basis(dpd_handle h, int basis);
@@ -320,17 +319,19 @@ dpd_status dpd_set_estimate_basis(dpd_handle h, int basis);
 /*
  * Least-squares coefficients (Sec. 2.2): h = argmin ||Psi(u) h - t||_2, i.e.
  * (Psi^H Psi) h = Psi^H t.  The Gram matrix is formed in `precision`, the
- * system is equilibrated (D = diag(G)^{-1/2}) and solved by an FP64 Cholesky
- * factorisation, then refined `refine_iters` times (0..100) with
+ * system is equilibrated (D = diag(G)^{-1/2}) and solved by a factorisation
+ * U Delta U^H in FP32 (hi, lo) pairs (FP64 where a pivot is below 2^-24 or a
+ * scale outside FP32's range), then refined `refine_iters` times (0..100) with
  * h += G^{-1} Psi^H (t - Psi h), the residual computed by the FP32 filter
  * and adjoint kernels.  In the indirect learning architecture u is the PA
  * output divided by its gain and t the predistorter output.
  *   h_out : device, K complex64, written (the handle's own coefficients are
  *           left unchanged; install the result with dpd_set_coeffs)
  *   stats : host double[2] or NULL: [0] 2-norm condition number of D G D
- *           (Lanczos on the FP64 Cholesky factor, host; about 1e-11 relative),
- *           [1] ||t - Psi h||^2 / ||t||^2 of the returned h (FP32 residual,
- *           FP32 squares summed in runs of 32, runs summed in FP64)
+ *           (Lanczos on D G D and on its inverse through the factor, the latter
+ *           refined against G; host, FP64, about 1e-11 relative),
+ *           [1] ||t - Psi h||^2 / ||t||^2 of the returned h (FP32 residual and
+ *           squares, sums in FP32 pairs, FP64 at the end)
  * Synchronises `stream` once, at the end: the condition estimate runs on the
  * host while the refinement runs on the device.  DPD_ERR_NOT_SPD if G is not
  * positive definite (e.g. u all zero); h_out and stats are then unspecified.
@@ -344,7 +345,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
  * `count` independent estimates for the handle's model (e.g. one per antenna):
  * u[i], t[i] device pointers to n[i] complex64.  One Gram launch covers every
  * problem; h_out receives count*K complex64 (problem-major).  info_out (host,
- * count ints, nullable) gets 0 or the failing Cholesky pivot + 1 per problem;
+ * count ints, nullable) gets 0 or the failing pivot + 1 per problem;
  * any failure returns DPD_ERR_NOT_SPD after the others are solved.
  */
 dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *const *t, const int64_t *n,

@@ -679,7 +679,7 @@ cudaError_t launch_adj_gh_tg(const AdjArgs &a, int blocks, int T, int Bp, int Bq
     return cudaGetLastError();
 }
 
-// gh: the tap-group size (1, 2 or 4 taps per group) and the CTAs per group
+// gh: the tap-group size (1 to 5 taps per group) and the CTAs per group
 // (= rows of partials, already clamped by the caller).
 template <int B>
 cudaError_t launch_adj_gh(const AdjArgs &a, const AdjLaunch &L, int T, int Bp, int Bq, int K, cudaStream_t s)

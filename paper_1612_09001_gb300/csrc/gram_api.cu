@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <limits>
 #include <system_error>
 #include <thread>
 #include <vector>
@@ -382,9 +383,9 @@ inline double hsum(v2d v) { return v[0] + v[1]; }
 // std::vector are 16-byte aligned (the allocator's fundamental alignment on
 // x86-64 and AArch64), so every row starts on a 16-byte boundary.
 struct Split {
-    int N = 0;
+    int rows = 0, N = 0;
     std::vector<double> re, im;
-    Split(int rows, int n) : N(n), re((size_t)rows * n, 0.0), im((size_t)rows * n, 0.0) {}
+    Split(int rows_, int n) : rows(rows_), N(n), re((size_t)rows * n, 0.0), im((size_t)rows * n, 0.0) {}
     double *r(int row) { return re.data() + (size_t)row * N; }
     double *i(int row) { return im.data() + (size_t)row * N; }
     const double *r(int row) const { return re.data() + (size_t)row * N; }
@@ -424,17 +425,54 @@ void matvec(const Split &M, int rows, const double *xr, const double *xi, double
     }
 }
 
-// One step of a column-oriented triangular solve: y[from .. to) -= m[from .. to) z
-// (m conjugated with `conj`), z an element that is final; independent over the
-// elements of the row m.
-void axpy_row(const double *mr, const double *mi, bool conj, double zr, double zi, int from, int to, double *yr,
-              double *yi)
+// Products of rows i .. i + 3 of M (conjugated with CONJ) with x[from .. to), from and to
+// even: every x element is loaded once per four rows.
+template <bool CONJ>
+void dot4(const Split &M, int i, int from, int to, const double *xr, const double *xi, double *sr, double *si)
 {
-    const v2d a = v2d{zr, zr}, b = v2d{zi, zi}, sg = conj ? v2d{-1.0, -1.0} : v2d{1.0, 1.0};
-    for (int k = from & ~1; k < to; k += 2) {   // M is zero outside [from, to)
-        const v2d r = ld2(mr + k), i = sg * ld2(mi + k);
-        st2(yr + k, ld2(yr + k) - (r * a - i * b));
-        st2(yi + k, ld2(yi + k) - (r * b + i * a));
+    v2d ar[4] = {}, ai[4] = {};
+    const double *mr[4], *mi[4];
+    for (int q = 0; q < 4; ++q) {
+        const int row = std::min(i + q, M.rows - 1);
+        mr[q] = M.r(row);
+        mi[q] = M.i(row);
+    }
+    for (int k = from; k < to; k += 2) {
+        const v2d a = ld2(xr + k), b = ld2(xi + k);
+        for (int q = 0; q < 4; ++q) {
+            const v2d r = ld2(mr[q] + k), c = ld2(mi[q] + k);
+            ar[q] += CONJ ? r * a + c * b : r * a - c * b;
+            ai[q] += CONJ ? r * b - c * a : r * b + c * a;
+        }
+    }
+    for (int q = 0; q < 4; ++q) {
+        sr[q] = hsum(ar[q]);
+        si[q] = hsum(ai[q]);
+    }
+}
+
+// x <- T^{-1} x for a unit triangular T: lower (its strict part in L's rows) or, with
+// CONJ, the conjugate transpose of the lower one whose transpose has its strict part in L's
+// rows.  Four rows at a time: the finished elements' products, then the block's own.
+template <bool CONJ>
+void triangular_solve(const Split &L, double *xr, double *xi)
+{
+    const int K = L.rows, N = L.N, last = (K - 1) & ~3;
+    for (int b = 0; b <= last; b += 4) {
+        const int i = CONJ ? last - b : b, rows = std::min(4, K - i);
+        double sr[4], si[4];
+        dot4<CONJ>(L, i, CONJ ? i + 4 : 0, CONJ ? N : i, xr, xi, sr, si);
+        for (int j = 0; j < rows; ++j) {
+            const int q = CONJ ? rows - 1 - j : j;
+            double re = xr[i + q] - sr[q], im = xi[i + q] - si[q];
+            for (int k = CONJ ? q + 1 : 0; k < (CONJ ? rows : q); ++k) {
+                const double mr = L.r(i + q)[i + k], mi = CONJ ? -L.i(i + q)[i + k] : L.i(i + q)[i + k];
+                re -= mr * xr[i + k] - mi * xi[i + k];
+                im -= mr * xi[i + k] + mi * xr[i + k];
+            }
+            xr[i + q] = re;
+            xi[i + q] = im;
+        }
     }
 }
 
@@ -489,6 +527,40 @@ double ritz_max(const std::vector<double> &al, const std::vector<double> &be, do
     return 0.5 * (lo + hi);
 }
 
+// z <- (T - lam)^{-1} z for the Lanczos tridiagonal T, by elimination with partial
+// pivoting (a zero pivot, lam being an eigenvalue, becomes the smallest normal number).
+void tridiagonal_solve(const std::vector<double> &al, const std::vector<double> &be, double lam, std::vector<double> &z)
+{
+    const int n = (int)al.size();
+    std::vector<double> p(n), q(n, 0.0), r(n, 0.0);   // the diagonal and the two above it
+    for (int i = 0; i < n; ++i) p[i] = al[i] - lam;
+    for (int i = 0; i + 1 < n; ++i) q[i] = be[i];
+    auto pivot = [](double v) { return v != 0.0 ? v : std::numeric_limits<double>::min(); };
+    for (int i = 0; i + 1 < n; ++i) {
+        const double s = be[i];
+        if (std::fabs(s) > std::fabs(p[i])) {   // rows i and i + 1 change places
+            const double m = p[i] / s, above = q[i];
+            p[i] = s;
+            q[i] = p[i + 1];
+            r[i] = q[i + 1];
+            p[i + 1] = above - m * q[i];
+            q[i + 1] = -m * r[i];
+            std::swap(z[i], z[i + 1]);
+            z[i + 1] -= m * z[i];
+        } else {
+            const double m = s / pivot(p[i]);
+            p[i + 1] -= m * q[i];
+            z[i + 1] -= m * z[i];
+        }
+    }
+    for (int i = n - 1; i >= 0; --i) {
+        double v = z[i];
+        if (i + 1 < n) v -= q[i] * z[i + 1];
+        if (i + 2 < n) v -= r[i] * z[i + 2];
+        z[i] = v / pivot(p[i]);
+    }
+}
+
 // Largest eigenvalue of the Hermitian positive definite operator `op` (w = op
 // v on padded split vectors of length N, K of them significant) by Lanczos
 // with full reorthogonalisation (classical Gram-Schmidt, repeated once when
@@ -499,8 +571,9 @@ double ritz_max(const std::vector<double> &al, const std::vector<double> &be, do
 // less than 1e-12 relative over five steps (checked at steps 10, 15, ..., at
 // most 40).  On these clustered spectra plain power iterations stay
 // percent-level low after 100 steps; this converges to about 1e-11 in 15-40.
+// `ritz`: the eigenvector's approximation (one row of N), or null.
 template <class Op>
-double largest(int K, int N, Op op)
+double largest(int K, int N, Op op, Split *ritz = nullptr)
 {
     const int m = std::min(K, 40);
     Split Q(m + 1, N), W(1, N);
@@ -559,6 +632,20 @@ double largest(int K, int N, Op op)
             Q.i(j + 1)[k] = wi[k] / bn;
         }
     }
+    if (ritz) {   // two steps of inverse iteration on the tridiagonal, in the Lanczos basis
+        std::vector<double> z(al.size(), 1.0);
+        for (int step = 0; step < 2; ++step) {
+            tridiagonal_solve(al, be, lam, z);
+            double top = 0.0;
+            for (double v : z) top = std::max(top, std::fabs(v));
+            for (double &v : z) v /= top;
+        }
+        for (size_t i = 0; i < z.size(); ++i)
+            for (int k = 0; k < K; ++k) {
+                ritz->r(0)[k] += z[i] * Q.r((int)i)[k];
+                ritz->i(0)[k] += z[i] * Q.i((int)i)[k];
+            }
+    }
     return lam;
 }
 
@@ -582,9 +669,12 @@ double largest_dgd(const double2 *G, int K)
     });
 }
 
-// Largest eigenvalue of (U Delta U^H)^{-1} from the packed factor (launch_chol):
-// two triangular solves per product, by rows of U^T and of U.
-double largest_inverse(const float4 *Up, int K)
+// Largest eigenvalue of (D G D)^{-1} with the packed factor of D G D = U Delta U^H
+// (launch_chol): two triangular solves per product, by rows of U and of U^T.  The factor
+// is a little off (about 2^-42 of the diagonal), and so is the eigenvector that Lanczos
+// finds with it, but the value is then taken as the Rayleigh quotient of that vector with
+// a product refined against G itself, whose error is that of the vector squared.
+double largest_inverse(const float4 *Up, const double2 *G, int K)
 {
     const int N = (K + 1) & ~1;
     Split U(K, N), Ut(K, N);
@@ -597,16 +687,45 @@ double largest_inverse(const float4 *Up, int K)
         }
         dinv[i] = (double)row[i].x + (double)row[i].z;
     }
-    return largest(K, N, [&](const double *vr, const double *vi, double *wr, double *wi) {
+    auto solve = [&](const double *vr, const double *vi, double *wr, double *wi) {
         std::copy(vr, vr + N, wr);
         std::copy(vi, vi + N, wi);
-        for (int k = 0; k + 1 < K; ++k) axpy_row(Ut.r(k), Ut.i(k), false, wr[k], wi[k], k + 1, K, wr, wi);
+        triangular_solve<false>(U, wr, wi);
         for (int i = 0; i < K; ++i) {
             wr[i] *= dinv[i];
             wi[i] *= dinv[i];
         }
-        for (int i = K - 1; i > 0; --i) axpy_row(U.r(i), U.i(i), true, wr[i], wi[i], 0, i, wr, wi);
-    });
+        triangular_solve<true>(Ut, wr, wi);
+    };
+    Split v(1, N), w(1, N), res(1, N), cor(1, N);
+    const double lam = largest(K, N, solve, &v);
+    solve(v.r(0), v.i(0), w.r(0), w.i(0));
+    std::vector<double> d(K), xr(K), xi(K);
+    for (int i = 0; i < K; ++i) {
+        const double gii = G[(size_t)i * K + i].x;
+        d[i] = gii > 0.0 ? 1.0 / std::sqrt(gii) : 0.0;
+        xr[i] = d[i] * w.r(0)[i];
+        xi[i] = d[i] * w.i(0)[i];
+    }
+    for (int i = 0; i < K; ++i) {   // v - D G D w
+        double sr = 0.0, si = 0.0;
+        for (int k = 0; k < K; ++k) {
+            const double2 g = G[(size_t)i * K + k];
+            sr += g.x * xr[k] - g.y * xi[k];
+            si += g.x * xi[k] + g.y * xr[k];
+        }
+        res.r(0)[i] = v.r(0)[i] - d[i] * sr;
+        res.i(0)[i] = v.i(0)[i] - d[i] * si;
+    }
+    solve(res.r(0), res.i(0), cor.r(0), cor.i(0));
+    double num = 0.0, den = 0.0;
+    for (int k = 0; k < K; ++k) {
+        const double a = v.r(0)[k], b = v.i(0)[k];
+        num += a * (w.r(0)[k] + cor.r(0)[k]) + b * (w.i(0)[k] + cor.i(0)[k]);
+        den += a * a + b * b;
+    }
+    const double quotient = num / den;
+    return std::isfinite(quotient) && quotient > 0.0 ? quotient : lam;
 }
 
 }  // namespace cond
@@ -730,7 +849,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     }
     const bool synced = cudaEventSynchronize(w.ev_U) == cudaSuccess;
     const int info = synced ? *w.h_info : 0;
-    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_U, K);
+    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_U, w.h_G, K);
     if (threaded) dgd_run.join();
     if (!synced) return DPD_ERR_CUDA;
     if (stats && !threaded) lmax = cond::largest_dgd(w.h_G, K);

@@ -44,7 +44,9 @@ def test_solve_at_panel_edges(P, Q, M):
     assert err <= cond * 2.0 ** -38 + 2.0 ** -23, (P, Q, M, cond)
     assert all(np.array_equal(hb[0], v) for v in hb[1:])
     assert np.linalg.norm(hb[0] - ref) <= (cond * 2e-6 + 2.0 ** -23) * np.linalg.norm(ref), (P, Q, M, cond)
-    assert abs(st["cond_est"] - cond) <= (1e-6 + cond * 2.0 ** -38) * cond
+    # the condition number is refined against G: Lanczos' 1e-11 and FP64 rounding on both sides
+    print(f"cond error {abs(st['cond_est'] / cond - 1):.2e}")
+    assert abs(st["cond_est"] - cond) <= (1e-10 + cond * 2.0 ** -48) * cond
 
 
 def test_scales_at_the_edge_of_fp32():
