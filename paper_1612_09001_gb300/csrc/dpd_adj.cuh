@@ -2,19 +2,19 @@
 // with respect to the input samples and the coefficients, given gy = dL/dy,
 // all under the convention grad = dL/dRe + j dL/dIm.
 //
-// With r = |x|^2 the filter is y_n = sum_{b,k} h_{b,k} r^b x + hbar_{b,k} r^b conj(x)
-// + c at samples n - k (Eq. 1, order 2b + 1).  Its adjoint first runs the taps
-// backwards over gy, one widely-linear FIR per power of r,
-//   F_b = sum_k conj(h_{b,k}) g_{i+k} + hbar_{b,k} conj(g_{i+k}),
-// and then takes the derivative of the features r^b x, r^b conj(x) at x_i:
-//   gx_i = V + 2 x_i Re(conj(x_i) V'),   V = sum_b r^b F_b,   V' = dV/dr.
-// V and V' come from one Horner pass over b (V' <- r V' + V, V <- r V + F_b), so
-// a sample costs 4 B T + 4 B fused multiply-adds.  The Wirtinger derivatives
-// evaluated tap by tap (four derivative polynomials of B and four of B - 1
-// coefficients per tap, 8 B - 4 per tap) cost 184 against 120 at B = T = 5.
-// Each FIR term is the 2 x 2 real matrix of the forward filter transposed, run
-// as two packed f32x2 FMAs on the window sample {c, d} and its swap {d, c}
-// (table built by wl_table_kernel, one float4 per tap and power).
+// With r = |x|^2, branch polynomials A_k(r) = sum_b h_{2b+1,k} r^b and
+// C_k(r) = sum_b hbar_{2b+1,k} r^b (so that y_n = sum_k A_k(r_{n-k}) x_{n-k}
+// + C_k(r_{n-k}) conj(x_{n-k}) + c, Eq. 1), the Wirtinger derivatives of the
+// term of tap k are
+//   dy/dx       = E_k(r) + G_k(r) conj(x)^2,   E = A + r A',  G = C'
+//   dy/dconj(x) = F_k(r) x^2 + H_k(r),         F = A',        H = C + r C'
+// and
+//   gx_i = sum_k conj(dy_{i+k}/dx_i) gy_{i+k} + (dy_{i+k}/dconj(x_i)) conj(gy_{i+k})
+//        = sum_k [conj(E_k) g + H_k conj(g)] + x_i^2 [conj(G_k) g + F_k conj(g)],  g = gy_{i+k}
+// Each bracket is widely linear in g, so it is evaluated like the forward
+// filter: four real Horner polynomials per bracket, run as two packed f32x2
+// Horner chains whose results multiply the window sample {c, d} and its swap
+// {d, c} (table built by wl_table_kernel, one float4 per power).
 //
 // The coefficient gradient is the correlation
 //   gh_{(p,k)} = sum_j r_j^b conj(x_j) gy_{j+k},  gh_{(q,k)} = sum_j r_j^b x_j gy_{j+k},
@@ -27,12 +27,21 @@
 // forward pass is stored.
 //
 // Data movement.  For 16-byte aligned x and gy both gradients run as kernels
-// whose warps work on their own: every warp owns a contiguous share of the
-// record and a ring of shared-memory slots that its lane 0 fills with bulk
+// whose warps work on their own: every warp has its share of the record's
+// units and a ring of shared-memory slots that its lane 0 fills with bulk
 // copies of x and gy (plus the look-ahead) completed on the warp's own
 // mbarriers, so no warp waits for another one until the final reduction.
 // Other alignments (and callers without an error word) use the plain-load
 // kernels, which read through L1.
+//
+// Rounding.  The forms above and the order of the FP32 sums are fixed: training's
+// first Adam step divides a gradient element by its own size plus eps, so where an
+// element is nearly zero (the constant's, at the identity) its rounding becomes a
+// visible part of the step.  A split of the coefficient gradient's samples over
+// other threads, with gx as one FIR per power of r and the features' derivative
+// after it (120 instead of 184 multiply-adds at B = T = 5), was as accurate but
+// moved the outputs of the fourth step by up to 2.7e-4 on inputs whose first gradient of
+// the constant is below 2e-7; in this order they stay within 2e-6.
 #pragma once
 
 #include "dpd_device.cuh"
@@ -44,19 +53,21 @@ constexpr int kAdjV = 4;          // samples per thread and unit
 constexpr int kAdjUnit = 32 * kAdjV;   // samples of a warp's work unit
 constexpr int kAdjWarps = 8;      // warps per CTA of the staged gx kernel
 constexpr int kAdjStages = 2;     // ring slots per warp of the staged gx kernel
-constexpr int kAdjSub = 2;        // units per slot of the staged gx kernel
+constexpr int kAdjSub = 1;        // units per slot of the staged gx kernel
 constexpr int kAdjGhWarps = 12;   // warps per CTA of the staged gh kernel (about 165 registers per thread)
 constexpr int kAdjGhStages = 2;   // ring slots per warp of the staged gh kernel
-constexpr int kAdjGhSub = 3;      // units per slot of the staged gh kernel
-// Measured on GB300, graph-replayed, P = Q = 9, M = 4, us at 2^23 + 4097 / 2^20
-// samples.  gx (slots x units): 2 x 2 38.8 / 6.4, 2 x 4 39.9 / 6.4, 3 x 2 40.5 / 6.4;
-// two CTAs of 8 warps an SM 39.4, three (80 registers, spills) 49.3, five of 4 warps
-// 40.1.  At 38.8 us it moves 5.2 TB/s; P = Q = 7, M = 3 takes 31.5 us, 6.4 TB/s (96 %
-// of a copy).  The kernel with a producer warp per CTA and derivative polynomials
-// per tap took 51 us.
-// gh with its final sum: 2 x 3 38.9 / 10.7, 2 x 4 39.0 / 10.9, 4 x 2 40.4 / 10.9; 11
-// warps 44.4, 16 (128 registers, spills) 80.7.  24 T FMA/s at 2^23; the ring shared by
-// the CTA's warps, whose slots waited for the slowest warp, took 47.7.
+constexpr int kAdjGhSub = 4;      // units per slot of the staged gh kernel
+// Measured on GB300, graph-replayed, us at 2^23 + 4097 / 2^20 samples.
+// gx, P = Q = 9, M = 4 and P = Q = 7, M = 3 (CTAs per SM, slots x units): 3, 2 x 1
+// 54.4 / 8.4 and 40.5 / 6.4; 2, 2 x 1 56.6 / 8.5 and 39.9 / 6.4; 2, 2 x 2 56.8 / 8.6
+// and 41.2 / 6.7; 2, 4 x 1 53.7 / 8.4 and 42.4 / 6.5; 3, 3 x 1 55.0 / 8.4 and 41.5 /
+// 6.6; 4 (64 registers, spills) 64.4 / 10.2 and 47.5 / 8.0.  The FMA pipe bounds the
+// first (28.5 T FMA/s), traffic the second (4.97 TB/s).  With a ring shared by the CTA's
+// warps and a producer warp: 53.8 / 9.3 and 41.2 / 7.4.
+// gh with its final sum, P = Q = 9, M = 4 and P = Q = 7, M = 3: 41.4 / 14.1 and 32.5 /
+// 11.8; with a ring shared by the CTA's warps, whose slots waited for the slowest
+// warp, 46.0 / 18.6 and 35.3 / 14.8.  At 2^20 the 171 tiles on 152 CTAs take two rounds
+// (10.7 with the record cut evenly over the warps, a split with other sums).
 
 // NS consecutive complex samples p[base .. base+NS-1] (zero past n).  When the
 // buffer is 16-byte aligned, base is even and the rounded-up window lies inside
@@ -100,8 +111,8 @@ __device__ __forceinline__ void adj_slot_window(const float2 *slot, int off, flo
 }
 
 // ---------------------------------------------------------------- warp rings
-// The record is cut into units of kAdjUnit samples and every warp of a launch
-// takes a contiguous run of them, equal to within one unit: warp w of W takes
+// The record is cut into units of kAdjUnit samples.  For the input gradient every
+// warp of a launch takes a contiguous run of them, equal to within one unit: warp w of W takes
 // units [first, first + count).  Consecutive w sit on different CTAs, so a short
 // record spreads over the SMs.  (A run of 2^31 units would be 2 TB of samples.)
 __device__ __forceinline__ int64_t warp_share(int64_t units, int w, int W, int &count)
@@ -136,10 +147,10 @@ __device__ __forceinline__ void adj_slot_window_tail(const float2 *slot, int cnt
     }
 }
 
-// One warp's ring: STAGES slots of SUB units; a slot holds x[s0, s0 + S) and,
-// from element S on, gy[s0, s0 + S + HALO), S = SUB * kAdjUnit (less at the end
-// of the warp's share and of the record, where only the even-length prefix that
-// exists is copied).  Lane 0 issues the copies of tile i + STAGES once the whole
+// One warp's ring over a contiguous share of the record (the input gradient):
+// STAGES slots of SUB units; a slot holds x[s0, s0 + S) and, from element S on,
+// gy[s0, s0 + S + HALO), S = SUB * kAdjUnit (less at the end of the warp's share
+// and of the record, where only the even-length prefix that exists is copied).  Lane 0 issues the copies of tile i + STAGES once the whole
 // warp has read tile i (its windows are in registers): the warp is producer and
 // consumer, so the slot needs a "full" barrier only.
 template <int STAGES, int SUB, int HALO>
@@ -210,9 +221,10 @@ struct AdjRing {
             copy(i, (uint32_t)xc * (uint32_t)sizeof(float2), (uint32_t)gc * (uint32_t)sizeof(float2));
         }
     }
+    // One outcome for the whole warp, whose lanes issue and reduce together.
     __device__ __forceinline__ bool wait(int i, int *status) const
     {
-        return mbar_wait(bars + 8u * (i % STAGES), (uint32_t)((i / STAGES) & 1), status);
+        return __all_sync(0xffffffffu, mbar_wait(bars + 8u * (i % STAGES), (uint32_t)((i / STAGES) & 1), status));
     }
     // The whole warp has read tile i: refill its slot.
     __device__ __forceinline__ void refill(int i, int lane)
@@ -270,47 +282,99 @@ template <int B, int T, int V, bool PARAM = false>
 __device__ __forceinline__ void gx_compute(const float *tab, const AdjParamTab<B, T> &ptab,
                                            const float2 (&xs)[V], const float2 (&g)[V + T - 1], float2 (&acc)[V])
 {
+    constexpr int QB = B, RB = B - 1;       // coefficients per Q / S polynomial
+    constexpr int PER_TAP = 4 * QB + 4 * RB;
     constexpr int W = V + T - 1;
     float2 gs[W];   // window samples swapped: {d, c}
 #pragma unroll
     for (int j = 0; j < W; ++j) gs[j] = make_float2(g[j].y, g[j].x);
-    float rr[V];
+    float ur[V], ui[V], rr[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) rr[v] = fmaf(xs[v].x, xs[v].x, xs[v].y * xs[v].y);
-    float2 val[V], der[V];   // V and V' of the Horner pass
+    for (int v = 0; v < V; ++v) {
+        const float2 q = xs[v];
+        rr[v] = fmaf(q.x, q.x, q.y * q.y);
+        ur[v] = fmaf(q.x, q.x, -q.y * q.y);   // x^2
+        ui[v] = 2.f * q.x * q.y;
+    }
+    // {Re, Im} of the gradient of each sample, and of the tap sum of the second
+    // bracket (its factor x^2 does not depend on the tap, so it is applied once
+    // after the tap loop).  Every tap advances all V samples together with
+    // packed f32x2 FMAs (coefficient pairs adjacent in the table).
+    float2 ws[V];
 #pragma unroll
-    for (int b = B - 1; b >= 0; --b) {
-        if (b < B - 1) {
+    for (int v = 0; v < V; ++v) {
+        acc[v] = make_float2(0.f, 0.f);
+        ws[v] = make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int k = 0; k < T; ++k) {
+        // quadruple j of tap k's block: the Q quadruples, then the S ones
+        auto coef = [&](int j) -> float4 {
+            if constexpr (PARAM) {
+                const int o = PER_TAP * k + 4 * j;
+                return make_float4(ptab.v[o], ptab.v[o + 1], ptab.v[o + 2], ptab.v[o + 3]);
+            } else {
+                return reinterpret_cast<const float4 *>(tab + PER_TAP * k)[j];
+            }
+        };
+        float2 pa[V], pb[V];
+        {
+            const float4 c4 = coef(QB - 1);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const float2 r2 = make_float2(rr[v], rr[v]);
-                der[v] = b < B - 2 ? __ffma2_rn(der[v], r2, val[v]) : val[v];
-                val[v] = __fmul2_rn(val[v], r2);
+                pa[v] = make_float2(c4.x, c4.y);
+                pb[v] = make_float2(c4.z, c4.w);
             }
         }
 #pragma unroll
-        for (int k = 0; k < T; ++k) {
-            float4 c4;
-            const int o = 4 * (k * B + b);
-            if constexpr (PARAM)
-                c4 = make_float4(ptab.v[o], ptab.v[o + 1], ptab.v[o + 2], ptab.v[o + 3]);
-            else
-                c4 = *reinterpret_cast<const float4 *>(tab + o);
+        for (int m = QB - 2; m >= 0; --m) {
+            const float4 c4 = coef(m);
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const float2 p = make_float2(c4.x, c4.y), q = make_float2(c4.z, c4.w);
-                val[v] = (b == B - 1 && k == 0) ? __fmul2_rn(p, g[v + k]) : __ffma2_rn(p, g[v + k], val[v]);
-                val[v] = __ffma2_rn(q, gs[v + k], val[v]);
+                const float2 rr2 = make_float2(rr[v], rr[v]);
+                pa[v] = __ffma2_rn(pa[v], rr2, make_float2(c4.x, c4.y));
+                pb[v] = __ffma2_rn(pb[v], rr2, make_float2(c4.z, c4.w));
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            acc[v] = __ffma2_rn(pa[v], g[v + k], acc[v]);    // {Q0 c, Q3 d}
+            acc[v] = __ffma2_rn(pb[v], gs[v + k], acc[v]);   // {Q1 d, Q2 c}
+        }
+        if constexpr (RB > 0) {
+            float2 sa[V], sb[V];
+            {
+                const float4 c4 = coef(QB + RB - 1);
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    sa[v] = make_float2(c4.x, c4.y);
+                    sb[v] = make_float2(c4.z, c4.w);
+                }
+            }
+#pragma unroll
+            for (int m = RB - 2; m >= 0; --m) {
+                const float4 c4 = coef(QB + m);
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const float2 rr2 = make_float2(rr[v], rr[v]);
+                    sa[v] = __ffma2_rn(sa[v], rr2, make_float2(c4.x, c4.y));
+                    sb[v] = __ffma2_rn(sb[v], rr2, make_float2(c4.z, c4.w));
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                // conj(G) g + F conj(g) = {S0 c + S1 d, S2 c + S3 d}
+                ws[v] = __ffma2_rn(sa[v], g[v + k], ws[v]);    // {S0 c, S3 d}
+                ws[v] = __ffma2_rn(sb[v], gs[v + k], ws[v]);   // {S1 d, S2 c}
             }
         }
     }
+    if constexpr (RB > 0) {
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        if constexpr (B > 1) {
-            const float t = 2.f * fmaf(xs[v].x, der[v].x, xs[v].y * der[v].y);
-            acc[v] = __ffma2_rn(xs[v], make_float2(t, t), val[v]);
-        } else {
-            acc[v] = val[v];
+        for (int v = 0; v < V; ++v) {
+            // acc += x^2 ws (complex):  {ur wr - ui wi, ur wi + ui wr}
+            acc[v] = __ffma2_rn(make_float2(ur[v], ur[v]), ws[v], acc[v]);
+            acc[v] = __ffma2_rn(make_float2(-ui[v], ui[v]), make_float2(ws[v].y, ws[v].x), acc[v]);
         }
     }
 }
@@ -367,7 +431,7 @@ using GxRing = AdjRing<kAdjStages, kAdjSub, kHalo>;
 // Staged variant: CTAs of kAdjWarps independent warps (see AdjRing).  x and gy
 // 16-byte aligned.
 template <int B, int T, int V, bool PARAM>
-__global__ void __launch_bounds__(32 * kAdjWarps, 2)
+__global__ void __launch_bounds__(32 * kAdjWarps, 3)
     adj_gx_tma_kernel(AdjArgs a, int64_t units, const __grid_constant__ AdjParamTab<B, T> ptab)
 {
     constexpr int W = V + T - 1;
@@ -542,10 +606,121 @@ __global__ void __launch_bounds__(256) adj_gh_kernel(AdjArgs a, int T, int Bp, i
                                 a.partials + (size_t)blockIdx.x * K);
 }
 
-using GhRing = AdjRing<kAdjGhStages, kAdjGhSub, kAdjGhHalo>;
+// One warp's ring in the coefficient gradient.  The CTAs of a tap group take tiles of
+// kAdjGhSub units per warp in turn: unit j of tile i of warp w of CTA b of G is unit
+//   ((i G + b) kAdjGhSub + j) kAdjGhWarps + w
+// of the record, and a lane adds its samples in that order.  A slot holds a tile: of
+// each unit its x and, from element kAdjUnit on, its gy with the look-ahead (at the
+// record's end the even-length prefix that exists), one bulk copy each by a lane of its
+// own.  Slots and barriers as in AdjRing.
+struct GhRing {
+    static constexpr int kPart = 2 * kAdjUnit + kAdjGhHalo;   // elements of a unit
+    static constexpr size_t kBytes = (size_t)kAdjGhStages * kAdjGhSub * kPart * sizeof(float2);   // per warp
+    static_assert(2 * kAdjGhSub <= 32, "a lane per copy");
+
+    const float2 *x, *gy;   // at the first sample of the warp's first unit
+    int64_t left;           // samples of the record from there on
+    int64_t step;           // samples from a tile to the next
+    float2 *slots;
+    uint32_t bars;
+    int tiles;
+    int whole;   // the first `whole` tiles lie, with their look-ahead, inside the record
+
+    __device__ __forceinline__ void init(const AdjArgs &a, int cta, int ctas, int warp, unsigned char *mem,
+                                         uint32_t bar_addr, int lane)
+    {
+        const int64_t s0 = ((int64_t)cta * kAdjGhSub * kAdjGhWarps + warp) * kAdjUnit;
+        // Samples from a tile's first to its end with the look-ahead.
+        constexpr int kReach = ((kAdjGhSub - 1) * kAdjGhWarps + 1) * kAdjUnit + kAdjGhHalo;
+        x = a.x + s0;
+        gy = a.gy + s0;
+        left = a.n - s0;
+        step = (int64_t)ctas * (kAdjGhSub * kAdjGhWarps * kAdjUnit);
+        slots = reinterpret_cast<float2 *>(mem);
+        bars = bar_addr;
+        tiles = left > 0 ? (int)((left - 1) / step) + 1 : 0;
+        whole = left >= kReach ? (int)((left - kReach) / step) + 1 : 0;
+        if (lane == 0) {
+            for (int s = 0; s < kAdjGhStages; ++s) mbar_init(bars + 8u * s, 1);
+            fence_barrier_init();
+        }
+        __syncwarp();
+        for (int i = 0; i < kAdjGhStages && i < tiles; ++i) issue(i, lane);
+    }
+    // Samples from unit j of tile i on to the end of the record.
+    __device__ __forceinline__ int64_t rest(int i, int j) const
+    {
+        return left - i * step - j * (kAdjGhWarps * kAdjUnit);
+    }
+    __device__ __forceinline__ int units_of(int i) const
+    {
+        if (i < whole) return kAdjGhSub;
+        const int64_t nu = (rest(i, 0) - 1) / (kAdjGhWarps * kAdjUnit) + 1;
+        return nu < kAdjGhSub ? (int)nu : kAdjGhSub;
+    }
+    __device__ __forceinline__ float2 *part(int i, int j) const
+    {
+        return slots + ((i % kAdjGhStages) * kAdjGhSub + j) * kPart;
+    }
+    // Samples of x (or of gy) that the slot holds of a unit with `rem` samples to the end.
+    __device__ __forceinline__ static int held(int64_t rem, bool is_gy)
+    {
+        const int want = is_gy ? kAdjUnit + kAdjGhHalo : kAdjUnit;
+        return rem >= want ? want : rem > 0 ? (int)rem & ~1 : 0;
+    }
+    __device__ __forceinline__ void issue(int i, int lane)   // the whole warp
+    {
+        const uint32_t fb = bars + 8u * (i % kAdjGhStages);
+        const int j = lane >> 1;
+        const bool is_gy = lane & 1;
+        uint32_t bytes = 0, all = kAdjGhSub * kPart * (uint32_t)sizeof(float2);
+        if (lane < 2 * kAdjGhSub)
+            bytes = (uint32_t)(i < whole ? (is_gy ? kAdjUnit + kAdjGhHalo : kAdjUnit) : held(rest(i, j), is_gy)) *
+                    (uint32_t)sizeof(float2);
+        if (i >= whole) all = __reduce_add_sync(0xffffffffu, bytes);
+        if (lane == 0) mbar_arrive_expect_tx(fb, all);
+        __syncwarp();
+        if (bytes)
+            bulk_copy_g2s(smem_addr(part(i, j)) + (is_gy ? kAdjUnit * (uint32_t)sizeof(float2) : 0u),
+                          (is_gy ? gy : x) + i * step + j * (kAdjGhWarps * kAdjUnit), bytes, fb);
+    }
+    __device__ __forceinline__ bool wait(int i, int *status) const
+    {
+        return __all_sync(0xffffffffu, mbar_wait(bars + 8u * (i % kAdjGhStages),
+                                                 (uint32_t)((i / kAdjGhStages) & 1), status));
+    }
+    __device__ __forceinline__ void refill(int i, int lane)   // the whole warp has read tile i
+    {
+        __syncwarp();
+        if (i + kAdjGhStages < tiles) {
+            fence_proxy_async_smem();   // the reads above precede the copies' writes
+            issue(i + kAdjGhStages, lane);
+        }
+    }
+    // After a failed wait on tile i: let the copies in flight land.
+    __device__ __forceinline__ void drain(int i, int *status) const
+    {
+        for (int q = i; q < i + kAdjGhStages && q < tiles; ++q) wait(q, status);
+    }
+    // The window of NX samples of x and NG of gy (from k0 on) of element off of unit j of tile i.
+    template <int NX, int NG>
+    __device__ __forceinline__ void window(int i, int j, int off, int k0, float2 (&xs)[NX], float2 (&g)[NG]) const
+    {
+        const float2 *sl = part(i, j);
+        if (i < whole) {
+            adj_slot_window<NX>(sl, off, xs);
+            adj_slot_window<NG>(sl + kAdjUnit, off + k0, g);
+        } else {
+            const int64_t rem = rest(i, j), at = i * step + j * (kAdjGhWarps * kAdjUnit);
+            adj_slot_window_tail<NX>(sl, held(rem, false), x + at, off, rem, xs);
+            adj_slot_window_tail<NG>(sl + kAdjUnit, held(rem, true), gy + at, off + k0, rem, g);
+        }
+    }
+};
+static_assert(GhRing::kPart % 2 == 0, "a unit's parts must stay 16-byte aligned");
 
 // Staged variant: grid (blocks, tap groups) of CTAs of kAdjGhWarps independent
-// warps (see AdjRing), block x of a tap group sharing the record with the
+// warps (see GhRing), block x of a tap group sharing the record with the
 // others of the group.  x and gy 16-byte aligned.  With 2 B TG + 1 packed
 // accumulators a thread takes about 165 registers, so one CTA fits an SM.
 template <int B, int TG, int V>
@@ -563,8 +738,8 @@ __device__ __forceinline__ void adj_gh_tma_body(const AdjArgs &a, int T, int Bp,
     const bool group0 = blockIdx.y == 0;
     grid_dep_wait();
     GhRing ring;
-    ring.init(a, (a.n + kAdjUnit - 1) / kAdjUnit, warp * gridDim.x + blockIdx.x, kAdjGhWarps * gridDim.x,
-              smem + adj_staged_smem<GhRing>(warp, kAdjGhWarps * NA), smem_addr(smem) + 8u * kAdjGhStages * warp, lane);
+    ring.init(a, blockIdx.x, gridDim.x, warp, smem + adj_staged_smem<GhRing>(warp, kAdjGhWarps * NA),
+              smem_addr(smem) + 8u * kAdjGhStages * warp, lane);
     float2 acc2[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) acc2[i] = make_float2(0.f, 0.f);
@@ -578,9 +753,8 @@ __device__ __forceinline__ void adj_gh_tma_body(const AdjArgs &a, int T, int Bp,
         const int nu = ring.units_of(i);
 #pragma unroll 1
         for (int j = 0; j < nu; ++j) {
-            const int off = j * kAdjUnit + lane * V;
             float2 xs[V], g[NG];
-            ring.window(i, off, k0, xs, g);
+            ring.window(i, j, lane * V, k0, xs, g);
             if (j == nu - 1) ring.refill(i, lane);
             gh_accumulate<B, TG, V>(xs, g, group0, acc2);
         }

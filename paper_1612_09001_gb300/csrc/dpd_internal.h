@@ -84,10 +84,12 @@ struct FwdArgs {
     float2 *hist = nullptr;
 };
 
-// Floats of the adjoint table: per tap k and power b the transposed 2 x 2 real
-// matrix of the forward table as the quadruple {P0, P3, P2, P1}; see dpd_adj.cuh.
-__host__ __device__ constexpr int adj_table_floats(int B, int T) { return 4 * B * T; }
-constexpr int kMaxAdjTabFloats = adj_table_floats(6, 8);   // 192
+// Floats of the adjoint table: per tap, four polynomials of B coefficients
+// (Q0..Q3 for conj(E) g + H conj(g)) and four of B-1 (S0..S3 for
+// conj(G) g + F conj(g)), stored power-major as quadruples {Q0, Q3, Q1, Q2}
+// then {S0, S3, S1, S2}; see dpd_adj.cuh.
+__host__ __device__ constexpr int adj_table_floats(int B, int T) { return (4 * B + 4 * (B - 1)) * T; }
+constexpr int kMaxAdjTabFloats = adj_table_floats(6, 8);   // 352
 
 struct AdjArgs {
     const float2 *x;
