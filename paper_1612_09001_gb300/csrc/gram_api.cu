@@ -23,18 +23,22 @@ bool aligned8(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0
 size_t table_stride(dpd_handle h) { return ((size_t)dpd::wl_table_floats(h->B, h->T) + 3) & ~(size_t)3; }
 size_t factor_size(int K) { return (size_t)K * (K + 1) / 2; }   // values of a packed factor
 
+// p <- `need` values in place of what it held; null, with no error pending, on failure.
 template <class T>
-bool grow(T *&p, size_t have, size_t need)
+bool grow(T *&p, size_t need)
 {
-    if (need <= have && p) return true;
     cudaFree(p);
     p = nullptr;
-    return cudaMalloc(&p, std::max<size_t>(need, 1) * sizeof(T)) == cudaSuccess;
+    if (cudaMalloc(&p, std::max<size_t>(need, 1) * sizeof(T)) == cudaSuccess) return true;
+    p = nullptr;
+    cudaGetLastError();
+    return false;
 }
 
 // Make sure the workspace holds nprob problems with cpp Gram CTAs each at this
 // precision and nsamp samples of refinement buffers.  Synchronises the device when it
-// grows.
+// grows.  A capacity counts only once all its arrays are there: after a failure the
+// next call, however small, allocates them anew.
 dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsamp)
 {
     EstimateWorkspace &w = h->est;
@@ -46,23 +50,24 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsam
     if (parts > w.partials_cap) {
         cudaDeviceSynchronize();
         w.partials_cap = 0;
-        if (!grow(w.partials, 0, parts)) return DPD_ERR_ALLOC;
+        if (!grow(w.partials, parts)) return DPD_ERR_ALLOC;
         w.partials_cap = parts;
     }
     if (nprob > w.nprob) {
         cudaDeviceSynchronize();
+        w.nprob = 0;
         const size_t np = (size_t)nprob;
-        ok = ok && grow(reinterpret_cast<dpd::GramProblem *&>(w.probs), 0, np);
-        ok = ok && grow(w.S, 0, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, 0, np * dpd::kLagEntries);
-        ok = ok && grow(w.G, 0, np * K * K) && grow(w.U, 0, np * factor_size(K));
-        ok = ok && grow(w.g, 0, np * K) && grow(w.h64, 0, np * K);
-        ok = ok && grow(w.d, 0, np * K) && grow(w.tt, 0, np) && grow(w.info, 0, np);
-        ok = ok && grow(w.tab, 0, np * table_stride(h));
+        ok = ok && grow(reinterpret_cast<dpd::GramProblem *&>(w.probs), np);
+        ok = ok && grow(w.S, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, np * dpd::kLagEntries);
+        ok = ok && grow(w.G, np * K * K) && grow(w.U, np * factor_size(K));
+        ok = ok && grow(w.g, np * K) && grow(w.h64, np * K);
+        ok = ok && grow(w.d, np * K) && grow(w.tt, np) && grow(w.info, np);
+        ok = ok && grow(w.tab, np * table_stride(h));
         // partial pairs, the completion counter (zero)
-        ok = ok && grow(w.norm_part, 0, (size_t)2 * dpd::kFwdNormSlots + 1) &&
+        ok = ok && grow(w.norm_part, (size_t)2 * dpd::kFwdNormSlots + 1) &&
              cudaMemset(w.norm_part, 0, ((size_t)2 * dpd::kFwdNormSlots + 1) * sizeof(double)) == cudaSuccess;
-        ok = ok && grow(w.ubasis, 0, np * dpd::kUSize) && grow(w.ubasis64, 0, np * dpd::kUSize);
-        ok = ok && grow(w.mom_part, 0, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
+        ok = ok && grow(w.ubasis, np * dpd::kUSize) && grow(w.ubasis64, np * dpd::kUSize);
+        ok = ok && grow(w.mom_part, std::max<size_t>(np, dpd::kMomBlocks) * dpd::kMomK);
         if (!ok) return DPD_ERR_ALLOC;
         w.nprob = nprob;
     }
@@ -79,15 +84,18 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsam
         if (cudaMallocHost(&w.h_G, sizeof(double2) * K * K) != cudaSuccess ||
             cudaMallocHost(&w.h_U, sizeof(float4) * factor_size(K)) != cudaSuccess ||
             cudaMallocHost(&w.h_info, sizeof(int)) != cudaSuccess ||
-            cudaMallocHost(&w.h_norm, 2 * sizeof(double)) != cudaSuccess)
+            cudaMallocHost(&w.h_norm, 2 * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
             return DPD_ERR_ALLOC;
+        }
         w.hK = K;
     }
     if (!w.ev_U && cudaEventCreateWithFlags(&w.ev_U, cudaEventDisableTiming) != cudaSuccess) return DPD_ERR_CUDA;
     if (!w.ev_G && cudaEventCreateWithFlags(&w.ev_G, cudaEventDisableTiming) != cudaSuccess) return DPD_ERR_CUDA;
     if (nsamp > w.nsamp) {
         cudaDeviceSynchronize();
-        ok = grow(w.y, 0, (size_t)nsamp) && grow(w.e, 0, (size_t)nsamp);
+        w.nsamp = 0;
+        ok = grow(w.y, (size_t)nsamp) && grow(w.e, (size_t)nsamp);
         if (!ok) return DPD_ERR_ALLOC;
         w.nsamp = nsamp;
     }
@@ -305,27 +313,22 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     }
     if ((size_t)count > w.bprob_cap) {
         cudaDeviceSynchronize();
-        cudaFree(w.bstreams);
-        cudaFree(w.badj);
-        w.bstreams = w.badj = nullptr;
         w.bprob_cap = 0;
-        if (cudaMalloc(&w.bstreams, sizeof(dpd::BatchStream) * count) != cudaSuccess ||
-            cudaMalloc(&w.badj, sizeof(dpd::AdjArgs) * count) != cudaSuccess)
+        if (!grow(reinterpret_cast<dpd::BatchStream *&>(w.bstreams), (size_t)count) ||
+            !grow(reinterpret_cast<dpd::AdjArgs *&>(w.badj), (size_t)count))
             return DPD_ERR_ALLOC;
         w.bprob_cap = (size_t)count;
     }
     if ((size_t)count * rows > w.bpart_cap) {
         cudaDeviceSynchronize();
         w.bpart_cap = 0;
-        if (!grow(w.bpart, 0, (size_t)count * rows * K)) return DPD_ERR_ALLOC;
+        if (!grow(w.bpart, (size_t)count * rows * K)) return DPD_ERR_ALLOC;
         w.bpart_cap = (size_t)count * rows;
     }
     if (items.size() > w.bitems_cap) {
         cudaDeviceSynchronize();
-        cudaFree(w.bitems);
-        w.bitems = nullptr;
         w.bitems_cap = 0;
-        if (cudaMalloc(&w.bitems, sizeof(dpd::BatchItem) * items.size()) != cudaSuccess) return DPD_ERR_ALLOC;
+        if (!grow(reinterpret_cast<dpd::BatchItem *&>(w.bitems), items.size())) return DPD_ERR_ALLOC;
         w.bitems_cap = items.size();
     }
     for (int p = 0; p < count; ++p) adj[p].partials = w.bpart + (size_t)p * rows * K;
