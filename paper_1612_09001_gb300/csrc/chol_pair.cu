@@ -7,7 +7,8 @@
 // operation on pairs costs 6 to 12 FP32 instructions.  A problem whose smallest
 // pivot is not well above the pair arithmetic's error is left to the FP64 kernel
 // (chol64_kernel), which every factorisation launches behind the pair kernel and
-// which returns at once for all others.
+// which returns at once for all others; its factor stays in FP64, and so do the solves
+// with it.
 #include <type_traits>
 
 #include "dpd_device.cuh"
@@ -387,8 +388,8 @@ __global__ void __launch_bounds__(kCholThreads, 1)
 constexpr int kChol64Threads = 256;
 
 __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *__restrict__ Gall, int K, float4 *Uall,
-                                                                double *__restrict__ dall, int *info, float4 *Uhost,
-                                                                int *info_host)
+                                                                int *wide, double *__restrict__ dall, int *info,
+                                                                float4 *Uhost, int *info_host)
 {
     extern __shared__ double2 A[];   // lower triangle of K x K, packed by rows (tri_row)
     __shared__ double dsh[kCholMaxK];
@@ -397,15 +398,19 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
     grid_dep_wait();
     const int p = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
     // Host copies of the first problem, whichever kernel factored it.
-    auto to_host = [&](int status) {
+    auto to_host = [&](int status, int fp64) {
         if (p != 0 || !Uhost) return;
 #pragma unroll 8
         for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = __ldcg(Uall + e);
-        if (tid == 0) *info_host = status;
+        if (tid == 0) {
+            info_host[0] = status;
+            info_host[1] = fp64;
+        }
     };
     const int before = info[p];
+    if (tid == 0) wide[p] = before == kNeedFp64;
     if (before != kNeedFp64) {
-        to_host(before);
+        to_host(before, 0);
         return;
     }
     const int tx = tid & 15, ty = tid >> 4, nty = nt >> 4;
@@ -481,21 +486,20 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *_
         }
         __syncthreads();
     }
-    float4 *U = Uall + (size_t)p * tri_row(K);
+    double2 *U = reinterpret_cast<double2 *>(Uall + (size_t)p * tri_row(K));
     for (int i = ty; i < K; i += nty)
         for (int k = tx; k <= i; k += 16) {
             const double s = 1.0 / A[tri_row(k) + k].x;
             const double2 v = A[tri_row(i) + k];
-            const float2 re = to_pair(k < i ? v.x * s : s * s), im = to_pair(k < i ? v.y * s : 0.0);
-            U[tri_row(i) + k] = make_float4(re.x, im.x, re.y, im.y);
+            U[tri_row(i) + k] = make_double2(k < i ? v.x * s : s * s, k < i ? v.y * s : 0.0);
         }
     for (int i = tid; i < K; i += nt) dall[(size_t)p * K + i] = dsh[i];
     if (tid == 0) info[p] = bad;
     __syncthreads();   // U and every thread's read of info
-    to_host(bad);
+    to_host(bad, 1);
 }
 
-cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, float4 *Uhost,
+cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, int *wide, double *d, int *info, float4 *Uhost,
                         int *info_host, int *status, cudaStream_t s)
 {
     if (K < 2 || K > kCholMaxK) return cudaErrorInvalidValue;
@@ -511,7 +515,7 @@ cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d
     static SmemAttr smem_rec;
     e = ensure_smem(smem_rec, (const void *)chol64_kernel, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(chol64_kernel, grid, kChol64Threads, smem, s, G, K, U, d, info, Uhost, info_host);
+    return launch_pdl(chol64_kernel, grid, kChol64Threads, smem, s, G, K, U, wide, d, info, Uhost, info_host);
 }
 
 // One CTA per problem: x = D U^{-H} Delta^{-1} U^{-1} D rhs, in FP32 pairs.  The CTA
@@ -598,15 +602,46 @@ __device__ __forceinline__ float4 cpair_add(const float4 &a, const float4 &b)
     const float2 im = pair_add(make_float2(a.y, a.w), make_float2(b.y, b.w));
     return make_float4(re.x, im.x, re.y, im.y);
 }
+// x <- U^{-H} Delta^{-1} U^{-1} x in FP64, one row per thread of the CTA, for the few
+// problems that the FP64 kernel factored (U in shared memory, two doubles a value).
+__device__ __noinline__ void solve_fp64(const double2 *U, double2 *x, int K, int tid)
+{
+    for (int j = 0; j < K; ++j) {
+        const double2 b = x[j];
+        if (tid > j && tid < K) {
+            const double2 a = U[tri_row(tid) + j];
+            double2 &v = x[tid];
+            v.x = fma(-a.x, b.x, fma(a.y, b.y, v.x));
+            v.y = fma(-a.x, b.y, fma(-a.y, b.x, v.y));
+        }
+        __syncthreads();
+    }
+    if (tid < K) {
+        const double s = U[tri_row(tid) + tid].x;
+        x[tid] = make_double2(x[tid].x * s, x[tid].y * s);
+    }
+    __syncthreads();
+    for (int j = K - 1; j >= 0; --j) {
+        const double2 b = x[j];
+        if (tid < j) {
+            const double2 a = U[tri_row(j) + tid];   // conj(a) b
+            double2 &v = x[tid];
+            v.x = fma(-a.x, b.x, fma(-a.y, b.y, v.x));
+            v.y = fma(-a.x, b.y, fma(a.y, b.x, v.y));
+        }
+        __syncthreads();
+    }
+}
 }  // namespace
 
-__global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restrict__ Uall,
+__global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restrict__ Uall, const int *wide,
                                                          const double *__restrict__ dall,
                                                          const int *__restrict__ info, int K, SolveIo io,
                                                          int *status)
 {
     extern __shared__ __align__(128) float4 Us[];   // U, lower triangle packed by rows (tri_row), 1 / pivots on the diagonal
     __shared__ float4 w[kCholMaxK];
+    double2 *x64 = reinterpret_cast<double2 *>(w);
     __shared__ double2 mono[kCholMaxK];      // a vector before and after a change of basis
     __shared__ float4 part[8][kCholMaxK];    // sums of rows by warp
     __shared__ uint64_t bar;
@@ -620,6 +655,7 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     const int warp = tid >> 5, lane = tid & 31;
     const int sub = tid & 7, grp = tid >> 3, ngrp = nt >> 3;   // 8 threads per row in the updates
     if (info[p] != 0) return;   // uniform over the CTA
+    const bool fp64 = wide[p] != 0;
     const float4 *U = Uall + (size_t)p * tri_row(K);
     const double *d = dall + (size_t)p * K;
     const double *W = io.basis ? io.basis + (size_t)p * kUSize : nullptr;
@@ -660,8 +696,13 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
         const double2 v = !io.rows ? io.rhs[(size_t)p * K + tid]
                           : W      ? basis_transform<false>(mono, W, tid, K, io.Bp, io.Bq, io.T)
                                    : mono[tid];
-        const float2 re = to_pair(v.x * d[tid]), im = to_pair(v.y * d[tid]);
-        w[tid] = make_float4(re.x, im.x, re.y, im.y);
+        const double2 b = make_double2(v.x * d[tid], v.y * d[tid]);
+        if (fp64)
+            x64[tid] = b;
+        else {
+            const float2 re = to_pair(b.x), im = to_pair(b.y);
+            w[tid] = make_float4(re.x, im.x, re.y, im.y);
+        }
     }
     if (!mbar_wait(smem_addr(&bar), 0u, status)) {   // the copy lands before the CTA leaves, within the limit
         mbar_wait(smem_addr(&bar), 0u, status);
@@ -669,9 +710,10 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     }
     __syncthreads();
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (fp64) solve_fp64(reinterpret_cast<const double2 *>(Us), x64, K, tid);
 
     // forward: U y = D b
-    for (int b0 = 0; b0 < K; b0 += kSolveNB) {
+    for (int b0 = 0; b0 < K && !fp64; b0 += kSolveNB) {
         const int nb = min(kSolveNB, K - b0);
         if (warp == 0) {
             const bool in = lane < nb;
@@ -702,7 +744,7 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
         }
         __syncthreads();
     }
-    if (tid < K) {   // z = Delta^{-1} y
+    if (tid < K && !fp64) {   // z = Delta^{-1} y
         const float4 q = Us[tri_row(tid) + tid], y = w[tid];
         const float2 s = make_float2(q.x, q.z);
         const float2 re = pair_mul(make_float2(y.x, y.z), s), im = pair_mul(make_float2(y.y, y.w), s);
@@ -710,7 +752,7 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     }
     __syncthreads();
     // backward: U^H v = z
-    for (int b0 = ((K - 1) / kSolveNB) * kSolveNB; b0 >= 0; b0 -= kSolveNB) {
+    for (int b0 = ((K - 1) / kSolveNB) * kSolveNB; b0 >= 0 && !fp64; b0 -= kSolveNB) {
         const int nb = min(kSolveNB, K - b0);
         if (warp == 0) {
             const bool in = lane < nb;
@@ -745,7 +787,8 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     }
     if (tid < K) {
         const float4 v = w[tid];
-        double2 x = make_double2(to_double(v.x, v.z) * d[tid], to_double(v.y, v.w) * d[tid]);
+        double2 x = fp64 ? x64[tid] : make_double2(to_double(v.x, v.z), to_double(v.y, v.w));
+        x = make_double2(x.x * d[tid], x.y * d[tid]);
         double2 *h = io.h + (size_t)p * K + tid;
         if (io.accumulate) x = make_double2(h->x + x.x, h->y + x.y);
         *h = x;
@@ -765,15 +808,15 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     wl_table_entry([hf](int i) { return hf[i]; }, tid, io.Bp, io.Bq, io.T, B, io.tab + (size_t)p * io.tstride, nullptr);
 }
 
-cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, int nprob, int K, const SolveIo &io,
-                              int *status, cudaStream_t s)
+cudaError_t launch_chol_solve(const float4 *U, const int *wide, const double *d, const int *info, int nprob, int K,
+                              const SolveIo &io, int *status, cudaStream_t s)
 {
     if (K < 1 || K > kCholMaxK) return cudaErrorInvalidValue;
     const size_t smem = sizeof(float4) * (size_t)tri_row(K);
     static SmemAttr smem_rec;
     const cudaError_t e = ensure_smem(smem_rec, (const void *)chol_solve_kernel, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(chol_solve_kernel, dim3((unsigned)nprob), 256, smem, s, U, d, info, K, io, status);
+    return launch_pdl(chol_solve_kernel, dim3((unsigned)nprob), 256, smem, s, U, wide, d, info, K, io, status);
 }
 
 }  // namespace dpd

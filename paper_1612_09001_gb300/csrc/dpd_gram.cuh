@@ -119,10 +119,11 @@ cudaError_t launch_basis(const GramProblem *probs, GramProblem one, int nprob, i
 int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
 // Equilibrated factorisation of every G: D G D = U Delta U^H, D = diag(G)^{-1/2}, U
 // unit lower triangular, Delta diagonal.  U per problem: K (K + 1) / 2 values packed
-// by rows, each an FP32 pair {re.hi, im.hi, re.lo, im.lo}, with 1 / Delta on the
-// diagonal; d: K per problem; info[p] = 0 or the failing pivot + 1.  Uhost, info_host:
-// copies of the first problem's factor and status in mapped host memory, or null.
-cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, double *d, int *info, float4 *Uhost,
+// by rows, with 1 / Delta on the diagonal, each an FP32 pair {re.hi, im.hi, re.lo,
+// im.lo} or, with wide[p], two doubles {re, im} in the same 16 bytes; d: K per problem;
+// info[p] = 0 or the failing pivot + 1.  Uhost, info_host: copies of the first problem's
+// factor, and of its status and wide flag, in mapped host memory, or null.
+cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, int *wide, double *d, int *info, float4 *Uhost,
                         int *info_host, int *status, cudaStream_t s);
 // x = G^{-1} rhs using the factorisation (problems that did not factor are skipped).
 // Every pointer: `nprob` consecutive vectors, K apart unless stated.
@@ -138,8 +139,8 @@ struct SolveIo {
     int tstride;
     int Bp, Bq, T;
 };
-cudaError_t launch_chol_solve(const float4 *U, const double *d, const int *info, int nprob, int K, const SolveIo &io,
-                              int *status, cudaStream_t s);
+cudaError_t launch_chol_solve(const float4 *U, const int *wide, const double *d, const int *info, int nprob, int K,
+                              const SolveIo &io, int *status, cudaStream_t s);
 // e = t - y (n samples).
 cudaError_t launch_residual(const float2 *t, const float2 *y, int64_t n, float2 *e, cudaStream_t s);
 // e = t - y together with out[0] = sum |e|^2, out[1] = sum |t|^2 in FP64

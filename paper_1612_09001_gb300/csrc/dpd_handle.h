@@ -19,6 +19,7 @@ struct EstimateWorkspace {
     double *Clag = nullptr;       // [nprob][kLagEntries]: summed lag sums (tensor-core Gram)
     double2 *G = nullptr, *g = nullptr, *h64 = nullptr;
     float4 *U = nullptr;          // [nprob][K (K + 1) / 2] factors (launch_chol)
+    int *wide = nullptr;          // [nprob] whether a factor is in FP64
     double *d = nullptr, *tt = nullptr;
     int *info = nullptr;
     float *tab = nullptr;         // [nprob][table_stride] forward tables of the current coefficients
@@ -32,7 +33,7 @@ struct EstimateWorkspace {
     int hK = 0;                   // K the host buffers were sized for
     double2 *h_G = nullptr;       // Gram matrix G, K x K (condition estimate on the host)
     float4 *h_U = nullptr;        // factor of D G D (launch_chol)
-    int *h_info = nullptr;        // pivot status of the factorisation
+    int *h_info = nullptr;        // pivot status of the factorisation, whether the factor is in FP64
     double *h_norm = nullptr;     // ||t - Psi h||^2, ||t||^2
     cudaEvent_t ev_G = nullptr;   // h_G is written
     // batched refinement (dpd_estimate_batched): work lists of the batched forward and

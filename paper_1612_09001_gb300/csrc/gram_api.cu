@@ -59,7 +59,7 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsam
         const size_t np = (size_t)nprob;
         ok = ok && grow(reinterpret_cast<dpd::GramProblem *&>(w.probs), np);
         ok = ok && grow(w.S, np * dpd::kGramS * dpd::kGramPartCols) && grow(w.Clag, np * dpd::kLagEntries);
-        ok = ok && grow(w.G, np * K * K) && grow(w.U, np * factor_size(K));
+        ok = ok && grow(w.G, np * K * K) && grow(w.U, np * factor_size(K)) && grow(w.wide, np);
         ok = ok && grow(w.g, np * K) && grow(w.h64, np * K);
         ok = ok && grow(w.d, np * K) && grow(w.tt, np) && grow(w.info, np);
         ok = ok && grow(w.tab, np * table_stride(h));
@@ -83,7 +83,7 @@ dpd_status reserve(dpd_handle h, int nprob, int cpp, int precision, int64_t nsam
         w.hK = 0;
         if (cudaMallocHost(&w.h_G, sizeof(double2) * K * K) != cudaSuccess ||
             cudaMallocHost(&w.h_U, sizeof(float4) * factor_size(K)) != cudaSuccess ||
-            cudaMallocHost(&w.h_info, sizeof(int)) != cudaSuccess ||
+            cudaMallocHost(&w.h_info, 2 * sizeof(int)) != cudaSuccess ||
             cudaMallocHost(&w.h_norm, 2 * sizeof(double)) != cudaSuccess) {
             cudaGetLastError();
             return DPD_ERR_ALLOC;
@@ -139,8 +139,8 @@ dpd_status solve(dpd_handle h, int p0, int np, const float2 *rows, int nrows, fl
     io.Bp = h->Bp;
     io.Bq = h->Bq;
     io.T = h->T;
-    return dpd::launch_chol_solve(w.U + p0 * factor_size(h->K), w.d + off, w.info + p0, np, h->K, io, h->d_status, s) ==
-                   cudaSuccess
+    return dpd::launch_chol_solve(w.U + p0 * factor_size(h->K), w.wide + p0, w.d + off, w.info + p0, np, h->K, io,
+                                  h->d_status, s) == cudaSuccess
                ? DPD_OK
                : DPD_ERR_CUDA;
 }
@@ -673,22 +673,23 @@ double largest_dgd(const double2 *G, int K)
 }
 
 // Largest eigenvalue of (D G D)^{-1} with the packed factor of D G D = U Delta U^H
-// (launch_chol): two triangular solves per product, by rows of U and of U^T.  The factor
-// is a little off (about 2^-42 of the diagonal), and so is the eigenvector that Lanczos
+// (launch_chol; `wide`: in FP64): two triangular solves per product, by rows of U and of
+// U^T.  A factor in pairs is a little off (about 2^-42 of the diagonal), and so is the eigenvector that Lanczos
 // finds with it, but the value is then taken as the Rayleigh quotient of that vector with
 // a product refined against G itself, whose error is that of the vector squared.
-double largest_inverse(const float4 *Up, const double2 *G, int K)
+double largest_inverse(const float4 *Up, bool wide, const double2 *G, int K)
 {
     const int N = (K + 1) & ~1;
     Split U(K, N), Ut(K, N);
     std::vector<double> dinv(K);
     for (int i = 0; i < K; ++i) {
         const float4 *row = Up + factor_size(i);   // i (i + 1) / 2
+        const double2 *row64 = reinterpret_cast<const double2 *>(row);
         for (int k = 0; k < i; ++k) {
-            Ut.r(k)[i] = U.r(i)[k] = (double)row[k].x + (double)row[k].z;
-            Ut.i(k)[i] = U.i(i)[k] = (double)row[k].y + (double)row[k].w;
+            Ut.r(k)[i] = U.r(i)[k] = wide ? row64[k].x : (double)row[k].x + (double)row[k].z;
+            Ut.i(k)[i] = U.i(i)[k] = wide ? row64[k].y : (double)row[k].y + (double)row[k].w;
         }
-        dinv[i] = (double)row[i].x + (double)row[i].z;
+        dinv[i] = wide ? row64[i].x : (double)row[i].x + (double)row[i].z;
     }
     auto solve = [&](const double *vr, const double *vi, double *wr, double *wi) {
         std::copy(vr, vr + N, wr);
@@ -753,6 +754,7 @@ void free_estimate_workspace(EstimateWorkspace &w)
     cudaFree(w.G);
     cudaFree(w.g);
     cudaFree(w.U);
+    cudaFree(w.wide);
     cudaFree(w.h64);
     cudaFree(w.d);
     cudaFree(w.tt);
@@ -828,7 +830,7 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if ((st = run_gram(h, 1, cpp, precision, s, &pr, nullptr, nullptr, false, stats ? w.h_G : nullptr)) != DPD_OK)
         return st;
     if (stats && cudaEventRecord(w.ev_G, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if (dpd::launch_chol(w.G, 1, K, w.U, w.d, w.info, w.h_U, w.h_info, h->d_status, s) != cudaSuccess ||
+    if (dpd::launch_chol(w.G, 1, K, w.U, w.wide, w.d, w.info, w.h_U, w.h_info, h->d_status, s) != cudaSuccess ||
         cudaEventRecord(w.ev_U, s) != cudaSuccess)
         return DPD_ERR_CUDA;
     float2 *out = static_cast<float2 *>(h_out);
@@ -851,8 +853,8 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
         }
     }
     const bool synced = cudaEventSynchronize(w.ev_U) == cudaSuccess;
-    const int info = synced ? *w.h_info : 0;
-    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_U, w.h_G, K);
+    const int info = synced ? w.h_info[0] : 0;
+    if (synced && stats && info == 0) linv = cond::largest_inverse(w.h_U, w.h_info[1] != 0, w.h_G, K);
     if (threaded) dgd_run.join();
     if (!synced) return DPD_ERR_CUDA;
     if (stats && !threaded) lmax = cond::largest_dgd(w.h_G, K);
@@ -894,7 +896,8 @@ dpd_status dpd_estimate_batched(dpd_handle h, const void *const *u, const void *
         return DPD_ERR_CUDA;
     if (ortho(h) && (st = compute_basis(h, nullptr, count, nmax, s)) != DPD_OK) return st;
     if ((st = run_gram(h, count, cpp, precision, s)) != DPD_OK) return st;
-    if (dpd::launch_chol(w.G, count, h->K, w.U, w.d, w.info, nullptr, nullptr, h->d_status, s) != cudaSuccess) return DPD_ERR_CUDA;
+    if (dpd::launch_chol(w.G, count, h->K, w.U, w.wide, w.d, w.info, nullptr, nullptr, h->d_status, s) != cudaSuccess)
+        return DPD_ERR_CUDA;
     float2 *out = static_cast<float2 *>(h_out);
     if ((st = solve(h, 0, count, nullptr, 0, out, s)) != DPD_OK) return st;
     // The pivot status comes back here only for the refinement problem by

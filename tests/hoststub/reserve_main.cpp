@@ -38,7 +38,7 @@ namespace {
 static bool whole(const EstimateWorkspace &w)
 {
     for (const void *p : {(const void *)w.probs, (const void *)w.partials, (const void *)w.S, (const void *)w.Clag,
-                          (const void *)w.G, (const void *)w.g, (const void *)w.U, (const void *)w.h64,
+                          (const void *)w.G, (const void *)w.g, (const void *)w.U, (const void *)w.wide, (const void *)w.h64,
                           (const void *)w.d, (const void *)w.tt, (const void *)w.info, (const void *)w.tab,
                           (const void *)w.norm_part, (const void *)w.ubasis, (const void *)w.ubasis64,
                           (const void *)w.mom_part, (const void *)w.y, (const void *)w.e, (const void *)w.h_G,

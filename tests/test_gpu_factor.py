@@ -88,3 +88,49 @@ def test_collinear_columns_go_to_fp64():
     e0[0] = 1.0
     assert np.abs(hb[0].cpu().numpy() - e0).max() <= 1e-3 and np.array_equal(hb[0].cpu().numpy(), hb[2].cpu().numpy())
     f.close()
+
+
+def _nearly_real(n, seed):
+    """Samples whose imaginary part is 2^-15 of their real part: the two branches' columns
+    differ by that much, so the second branch's pivots are about 2^-28 times the first's
+    (the difference is exact: both branches' Gram entries use the same real sums)."""
+    a, b = synth.clipped_gaussian(n, 0.3, key=(144, seed)), synth.clipped_gaussian(n, 0.3, key=(145, seed))
+    return torch.from_numpy((a.real + 1j * b.real * 2.0 ** -15).astype(np.complex64)).cuda()
+
+
+@pytest.mark.parametrize("P,Q,M", [(1, 1, 0), (1, 1, 3), (3, 3, 3), (3, 3, 7), (5, 5, 5)])
+@pytest.mark.parametrize("precision", ["fp32", "tf32x3"])
+def test_fp64_factor_and_solve(P, Q, M, precision):
+    """Smallest pivots between 1e-14 and 2^-25, which the pair kernel leaves to FP64:
+    the coefficients against numpy's FP64 solve of the library's own G (its lower
+    triangle, which the factorisation reads) and g, within K cond(A) 2^-53 and the FP32
+    rounding of h, alone, as a batch of one (the same G) and beside problems that the pair
+    kernel keeps."""
+    n = 30000
+    u = _nearly_real(n, M)
+    f = dpd.DPD(P, Q, M)
+    f.set_coeffs(synth.coeffs(P, Q, M, key=(146, P)))
+    t = f.apply(u)
+    h, _ = f.estimate(u, t, precision=precision, refine_iters=0)
+    h1, info1 = f.estimate_batched([u], [t], precision=precision, refine_iters=0)
+    G, g, _ = f.gram(u, t, precision=precision)
+    G, g = G.cpu().numpy(), g.cpu().numpy()
+    d = 1.0 / np.sqrt(np.real(np.diag(G)))
+    A = np.tril(G) + np.tril(G, -1).conj().T
+    A = A * d[:, None] * d[None, :]
+    pivot, cond = np.abs(np.diag(np.linalg.cholesky(A))).min() ** 2, np.linalg.cond(A)
+    assert 1e-14 < pivot < 2.0 ** -25, pivot
+    ref = d * np.linalg.solve(A, d * g)
+    for got in (h, h1[0]):
+        err = np.linalg.norm(got.cpu().numpy() - ref) / np.linalg.norm(ref)
+        print(f"K {f.K} pivot {pivot:.1e} cond {cond:.1e} error {err:.1e} = cond 2^{np.log2(err / cond):.1f}")
+        assert err <= f.K * cond * 2.0 ** -53 + 2.0 ** -23
+    assert info1 == [0]
+    good = torch.from_numpy(synth.clipped_gaussian(n, 0.3, key=(147, 1))).cuda()
+    tg = f.apply(good)
+    hb, info = f.estimate_batched([good, u, good], [tg, t, tg], precision=precision, refine_iters=0)
+    hg, _ = f.estimate_batched([good] * 3, [tg] * 3, precision=precision, refine_iters=0)
+    assert info == [0, 0, 0] and torch.equal(hb[0], hg[0]) and torch.equal(hb[2], hg[0])
+    f.set_coeffs(hb[1].contiguous())
+    assert float((f.apply(u) - t).norm()) <= 1e-3 * float(t.norm())
+    f.close()
