@@ -674,9 +674,11 @@ double largest_dgd(const double2 *G, int K)
 
 // Largest eigenvalue of (D G D)^{-1} with the packed factor of D G D = U Delta U^H
 // (launch_chol; `wide`: in FP64): two triangular solves per product, by rows of U and of
-// U^T.  A factor in pairs is a little off (about 2^-42 of the diagonal), and so is the eigenvector that Lanczos
-// finds with it, but the value is then taken as the Rayleigh quotient of that vector with
-// a product refined against G itself, whose error is that of the vector squared.
+// U^T.  A factor in pairs is a little off (about 2^-42 of the diagonal), and so is the
+// eigenvector that Lanczos finds with it, but the value is then taken as the Rayleigh
+// quotient of that vector with a product refined against G itself, whose error is that of
+// the vector squared.  Of G the lower triangle, as in the factorisation: the end products
+// of the tensor-core form leave the upper one up to 1e-10 off its conjugate.
 double largest_inverse(const float4 *Up, bool wide, const double2 *G, int K)
 {
     const int N = (K + 1) & ~1;
@@ -711,15 +713,23 @@ double largest_inverse(const float4 *Up, bool wide, const double2 *G, int K)
         xr[i] = d[i] * w.r(0)[i];
         xi[i] = d[i] * w.i(0)[i];
     }
-    for (int i = 0; i < K; ++i) {   // v - D G D w
-        double sr = 0.0, si = 0.0;
-        for (int k = 0; k < K; ++k) {
-            const double2 g = G[(size_t)i * K + k];
+    std::vector<double> yr(K), yi(K);   // G x
+    for (int i = 0; i < K; ++i) {
+        const double2 *row = G + (size_t)i * K;
+        double sr = row[i].x * xr[i], si = row[i].x * xi[i];
+        for (int k = 0; k < i; ++k) {
+            const double2 g = row[k];
             sr += g.x * xr[k] - g.y * xi[k];
             si += g.x * xi[k] + g.y * xr[k];
+            yr[k] += g.x * xr[i] + g.y * xi[i];
+            yi[k] += g.x * xi[i] - g.y * xr[i];
         }
-        res.r(0)[i] = v.r(0)[i] - d[i] * sr;
-        res.i(0)[i] = v.i(0)[i] - d[i] * si;
+        yr[i] = sr;
+        yi[i] = si;
+    }
+    for (int i = 0; i < K; ++i) {   // v - D G D w
+        res.r(0)[i] = v.r(0)[i] - d[i] * yr[i];
+        res.i(0)[i] = v.i(0)[i] - d[i] * yi[i];
     }
     solve(res.r(0), res.i(0), cor.r(0), cor.i(0));
     double num = 0.0, den = 0.0;

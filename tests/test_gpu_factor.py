@@ -134,3 +134,23 @@ def test_fp64_factor_and_solve(P, Q, M, precision):
     f.set_coeffs(hb[1].contiguous())
     assert float((f.apply(u) - t).norm()) <= 1e-3 * float(t.norm())
     f.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32x3", "bf16x3"])
+def test_condition_of_the_factored_matrix(precision):
+    """The condition number of the matrix that was factored (G's lower triangle) where the
+    tensor-core forms leave the upper triangle 1e-10 off its conjugate: at 1e11 the two
+    triangles' values differ by more than their sizes.  FP64 rounding of both sides is K
+    2^-53 of the largest eigenvalue, so K cond 2^-53 relative, four times for the reference's."""
+    u = _nearly_real(30000, 5)
+    f = dpd.DPD(5, 5, 5)
+    f.set_coeffs(synth.coeffs(5, 5, 5, key=(146, 5)))
+    t = f.apply(u)
+    _, st = f.estimate(u, t, precision=precision, refine_iters=0)
+    G = f.gram(u, t, precision=precision)[0].cpu().numpy()
+    f.close()
+    d = 1.0 / np.sqrt(np.real(np.diag(G)))
+    w = np.linalg.eigvalsh((np.tril(G) + np.tril(G, -1).conj().T) * d[:, None] * d[None, :])
+    cond = w[-1] / w[0]
+    print(f"cond {cond:.3e} error {abs(st['cond_est'] / cond - 1):.1e}")
+    assert abs(st["cond_est"] / cond - 1) <= 1e-10 + 4 * len(d) * cond * 2.0 ** -53
