@@ -62,6 +62,9 @@ __device__ __forceinline__ float2 to_pair(double x)
 
 __device__ __forceinline__ double to_double(float h, float l) { return (double)h + (double)l; }
 
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }   // biased
+__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((e + 1023) << 20, 0); }   // |e| <= 1022
+
 // A double whose exponent leaves both parts normal FP32 numbers, split by its bits
 // (no FP64 instruction): hi is its leading 24 bits, lo the other 29 rounded to 24.
 __device__ __forceinline__ bool splittable(double x)
@@ -645,7 +648,9 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     __shared__ double2 mono[kCholMaxK];      // a vector before and after a change of basis
     __shared__ float4 part[8][kCholMaxK];    // sums of rows by warp
     __shared__ uint64_t bar;
+    __shared__ int top;                      // largest exponent in D rhs
     if (threadIdx.x == 0) {
+        top = 0;
         mbar_init(smem_addr(&bar), 1);
         fence_barrier_init();
     }
@@ -688,25 +693,43 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
             float4 v = part[0][tid];
 #pragma unroll
             for (int q = 1; q < 8; ++q) v = cpair_add(v, part[q][tid]);
-            mono[tid] = make_double2(to_double(v.x, v.z), to_double(v.y, v.w));
+            double2 g = make_double2(to_double(v.x, v.z), to_double(v.y, v.w));
+            if (!isfinite(g.x) || !isfinite(g.y)) {   // a sum outside FP32's range (or an infinite row)
+                g = make_double2(0.0, 0.0);
+                for (int r = 0; r < io.nrows; ++r) {
+                    const float2 e = rows[(size_t)r * K + tid];
+                    g = make_double2(g.x + (double)e.x, g.y + (double)e.y);
+                }
+            }
+            mono[tid] = g;
         }
         __syncthreads();
     }
+    double2 b = make_double2(0.0, 0.0);   // element tid of D rhs
     if (tid < K) {
         const double2 v = !io.rows ? io.rhs[(size_t)p * K + tid]
                           : W      ? basis_transform<false>(mono, W, tid, K, io.Bp, io.Bq, io.T)
                                    : mono[tid];
-        const double2 b = make_double2(v.x * d[tid], v.y * d[tid]);
-        if (fp64)
-            x64[tid] = b;
-        else {
-            const float2 re = to_pair(b.x), im = to_pair(b.y);
-            w[tid] = make_float4(re.x, im.x, re.y, im.y);
-        }
+        b = make_double2(v.x * d[tid], v.y * d[tid]);
+        atomicMax(&top, max(exponent(b.x), exponent(b.y)));
     }
     if (!mbar_wait(smem_addr(&bar), 0u, status)) {   // the copy lands before the CTA leaves, within the limit
         mbar_wait(smem_addr(&bar), 0u, status);
         return;
+    }
+    __syncthreads();
+    // In pairs the right-hand side is scaled by the power of two that brings its largest
+    // element to [1, 2), and the result back: exact, and no element that matters leaves
+    // FP32's range on the way (a positive definite matrix with pivots above kPivotMin).
+    const int shift = top >= 1 && top <= 2045 ? top - 1023 : 0;
+    if (tid < K) {
+        if (fp64) {
+            x64[tid] = b;
+        } else {
+            const double s = power_of_two(-shift);
+            const float2 re = to_pair(b.x * s), im = to_pair(b.y * s);
+            w[tid] = make_float4(re.x, im.x, re.y, im.y);
+        }
     }
     __syncthreads();
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -787,8 +810,9 @@ __global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restric
     }
     if (tid < K) {
         const float4 v = w[tid];
+        const double s = fp64 ? 1.0 : power_of_two(shift);
         double2 x = fp64 ? x64[tid] : make_double2(to_double(v.x, v.z), to_double(v.y, v.w));
-        x = make_double2(x.x * d[tid], x.y * d[tid]);
+        x = make_double2(x.x * d[tid] * s, x.y * d[tid] * s);
         double2 *h = io.h + (size_t)p * K + tid;
         if (io.accumulate) x = make_double2(h->x + x.x, h->y + x.y);
         *h = x;

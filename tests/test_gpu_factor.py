@@ -154,3 +154,29 @@ def test_condition_of_the_factored_matrix(precision):
     cond = w[-1] / w[0]
     print(f"cond {cond:.3e} error {abs(st['cond_est'] / cond - 1):.1e}")
     assert abs(st["cond_est"] / cond - 1) <= 1e-10 + 4 * len(d) * cond * 2.0 ** -53
+
+
+@pytest.mark.parametrize("P,Q,M", [(1, 1, 1), (7, 7, 3), (9, 9, 6)])
+@pytest.mark.parametrize("e", [-124, -120, -100, 100, 118, 121])
+def test_targets_far_from_one(P, Q, M, e):
+    """Targets scaled by 2^e, up to where their products with the basis still are FP32
+    numbers: the solve of the library's own G and g within the bound of
+    test_solve_at_panel_edges, in FP32's smallest and largest numbers too."""
+    n = 400000
+    u = torch.from_numpy(synth.clipped_gaussian(n, 0.3, key=(148, P))).cuda()
+    f = dpd.DPD(P, Q, M)
+    f.set_coeffs(synth.coeffs(P, Q, M, key=(149, P)))
+    t = f.apply(u) * 2.0 ** e
+    h, _ = f.estimate(u, t, precision="fp32", refine_iters=0)
+    h1, _ = f.estimate_batched([u], [t], precision="fp32", refine_iters=0)
+    G, g, _ = f.gram(u, t, precision="fp32")
+    f.close()
+    G, g = G.cpu().numpy(), g.cpu().numpy()
+    d = 1.0 / np.sqrt(np.real(np.diag(G)))
+    A = G * d[:, None] * d[None, :]
+    ref, cond = d * np.linalg.solve(A, d * g), np.linalg.cond(A)
+    assert np.all(np.isfinite(ref)) and np.abs(ref).max() < 1e38
+    for got in (h, h1[0]):
+        err = np.linalg.norm(got.cpu().numpy().astype(np.complex128) - ref) / np.linalg.norm(ref)
+        # FP32's smallest step, 2^-149, is a rounding of its own for the coefficients themselves
+        assert err <= cond * 2.0 ** -38 + 2.0 ** -23 + 2.0 ** -149 * len(ref) / np.linalg.norm(ref), (err, cond)
