@@ -29,8 +29,28 @@ from .autograd import DPDFunction
 
 
 class SqErrorLoss(torch.autograd.Function):
-    """L = scale * ||y - gain x||^2 (dpd_sq_error); backward forms the gradient from the
-    same y and x, scaled by dL, in one pass (dpd_sq_error_grad)."""
+    """L = scale * ||y - gain x||^2 with its gradient produced in the same device
+    pass (dpd_sq_error); backward scales the saved gradient by dL, so y and x may
+    change in between and the product can be differentiated with respect to dL."""
+
+    @staticmethod
+    def forward(ctx, y, x, filt, gain, scale):
+        gy = torch.empty_like(y)
+        loss = filt.sq_error(y, x, gain=gain, scale=scale, gy=gy)
+        ctx.save_for_backward(gy)
+        return loss[0]
+
+    @staticmethod
+    def backward(ctx, gl):
+        (gy,) = ctx.saved_tensors
+        return gy * gl, None, None, None, None
+
+
+class _StepLoss(torch.autograd.Function):
+    """SqErrorLoss for a y that nothing else holds and a gradient that goes on into
+    DPDFunction.backward (a raw kernel, which ends any second differentiation): backward
+    forms the gradient from y and x, scaled by dL, in one pass (dpd_sq_error_grad): 6 us
+    of a training step of 2^20 samples less than SqErrorLoss."""
 
     @staticmethod
     def forward(ctx, y, x, filt, gain, scale):
@@ -114,7 +134,9 @@ class DirectLearner:
 
     def loss(self):
         y = self.tx(DPDFunction.apply(self.x, self.h, self.filt))
-        return SqErrorLoss.apply(y, self.x, self.filt, self.gain, self.scale)
+        # A Transmitter keeps no reference to its output; another callable might.
+        loss = _StepLoss if type(self.tx) is Transmitter else SqErrorLoss
+        return loss.apply(y, self.x, self.filt, self.gain, self.scale)
 
     def _adam_step(self):
         """self.opt.step(), as one launch of the library's kernel on the optimiser's own

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 import paper_1612_09001_gb300 as dpd  # noqa: E402
 from paper_1612_09001_gb300 import _lib  # noqa: E402
-from paper_1612_09001_gb300.direct import DirectLearner, Transmitter  # noqa: E402
+from paper_1612_09001_gb300.direct import DirectLearner, SqErrorLoss, Transmitter  # noqa: E402
 
 
 @pytest.mark.parametrize("n", [0, 1, 66, 255, 256, 257, 1000])
@@ -93,3 +93,59 @@ def test_learner_steps_match_the_optimisers_own():
         out.append((lr.h.detach().clone(), float(lr.opt.state[lr.param]["step"])))
     assert out[0][1] == out[1][1] == 23.0
     assert float((out[0][0] - out[1][0]).abs().max()) <= 1e-4
+
+
+def _loss_case(n=1000):
+    x = torch.from_numpy(synth.ofdm2(n, key=(134, 0))).cuda()
+    y0 = torch.from_numpy(synth.ofdm2(n, key=(135, 0))).cuda().requires_grad_()
+    f = dpd.DPD(1, 0, 0)
+    return x, y0, f, (2 * 0.25) * (y0 - (0.9 + 0.1j) * x).detach()
+
+
+def test_loss_gradient_is_that_of_the_y_it_saw():
+    x, y0, f, ref = _loss_case()
+    y = y0 * 1
+    loss = SqErrorLoss.apply(y, x, f, 0.9 + 0.1j, 0.25)
+    with torch.no_grad():
+        y.zero_()
+    loss.backward()
+    assert float((y0.grad - ref).abs().max()) <= 1e-6 * float(ref.abs().max())
+    f.close()
+
+
+def test_loss_gradient_is_differentiable_by_its_factor():
+    x, y0, f, ref = _loss_case()
+    loss = SqErrorLoss.apply(y0, x, f, 0.9 + 0.1j, 0.25)
+    gl = torch.tensor(1.5, device="cuda", requires_grad=True)
+    (gy,) = torch.autograd.grad(loss, y0, gl, create_graph=True)
+    (d,) = torch.autograd.grad(torch.view_as_real(gy).square().sum(), gl)
+    want = 2 * 1.5 * float(torch.view_as_real(ref).double().square().sum())
+    assert abs(float(d) - want) <= 1e-5 * want
+    f.close()
+
+
+def test_loss_gradients_of_several_factors_at_once():
+    x, y0, f, ref = _loss_case()
+    loss = SqErrorLoss.apply(y0, x, f, 0.9 + 0.1j, 0.25)
+    k = torch.tensor([1.0, -2.0, 0.5], device="cuda")
+    (gy,) = torch.autograd.grad(loss, y0, k, is_grads_batched=True)
+    assert float((gy - k[:, None] * ref).abs().max()) <= 2e-6 * float(ref.abs().max())
+    f.close()
+
+
+def test_learner_with_a_transmitter_of_its_own():
+    """A callable that keeps its output and changes it after the loss."""
+    x = torch.from_numpy(synth.ofdm2(4096, key=(136, 0))).cuda()
+    kept = []
+
+    def tx(v):
+        kept.append(v * (1.1 + 0.1j))
+        return kept[-1]
+    lr = DirectLearner(x, tx, 3, 3, 1, lr=1e-3)
+    want = DirectLearner(x, lambda v: v * (1.1 + 0.1j), 3, 3, 1, lr=1e-3)
+    loss = lr.loss()
+    with torch.no_grad():
+        kept[-1].zero_()
+    loss.backward()
+    want.loss().backward()
+    assert torch.equal(lr.param.grad, want.param.grad)
