@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(256)
         const double vi = beta2 * (double)v[i] + (1.0 - beta2) * gd * gd;
         m[i] = (float)mi;
         v[i] = (float)vi;
-        const double root = vi > 0.0 ? vi * inv_sqrt(vi * c2) : sqrt(vi);
+        const double root = vi > 0.0 && vi < 1e300 ? vi * inv_sqrt(vi * c2) : sqrt(vi);   // 0, infinity, NaN
         const double den = root + eps;
         param[i] = (float)((double)param[i] - (den > 0.0 ? rate * mi * inv_newton(den) : rate * mi / den));
     }

@@ -149,3 +149,23 @@ def test_learner_with_a_transmitter_of_its_own():
     loss.backward()
     want.loss().backward()
     assert torch.equal(lr.param.grad, want.param.grad)
+
+
+def test_adam_step_at_the_ends_of_fp32():
+    """An infinite second moment (gradients above 2^64 overflow its FP32 storage) gives
+    steps of zero, as sqrt(inf) does; infinite and NaN gradients give NaN."""
+    inf, nan = float("inf"), float("nan")
+    g = np.array([0.0, 1e25, 1e-30, inf, nan, 3e38], np.float32)
+    m = np.array([1.0, 1e24, 0.0, 0.0, 0.0, 0.0], np.float32)
+    v = np.array([inf, inf, 1e-45, 1.0, 1.0, 0.0], np.float32)
+    p = np.ones(6, np.float32)
+    d = [torch.from_numpy(a.copy()).cuda() for a in (p, g, m, v)]
+    step, lr = torch.tensor(5.0, device="cuda"), torch.tensor(1e-2, device="cuda")
+    _lib.check("dpd_adam_step", dpd.lib().dpd_adam_step(*[a.data_ptr() for a in d], step.data_ptr(), 6, lr.data_ptr(),
+                                                        0.9, 0.999, 1e-8, torch.cuda.current_stream().cuda_stream))
+    with np.errstate(all="ignore"):
+        m64 = 0.9 * m.astype(np.float64) + (1 - 0.9) * g.astype(np.float64)
+        v64 = 0.999 * v.astype(np.float64) + (1 - 0.999) * g.astype(np.float64) ** 2
+        p64 = p - float(lr) / (1 - 0.9 ** 6) * m64 / (np.sqrt(v64 / (1 - 0.999 ** 6)) + 1e-8)
+    got = d[0].cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(p64)) and np.allclose(got, p64, rtol=2.0 ** -23, atol=0, equal_nan=True), got
