@@ -135,7 +135,7 @@ __device__ __forceinline__ double equilibration(double g)   // g^{-1/2}, or 0
 // NG: row groups of 32, and rounds of panels (columns 32 c + 4 warp + q).
 template <int NG>
 __global__ void __launch_bounds__(kCholThreads, 1)
-    chol_pair_kernel(const double2 *__restrict__ Gall, int K, float4 *__restrict__ Uall, double *__restrict__ dall,
+    chol_pair_kernel(const double2 *Gall, int K, float4 *__restrict__ Uall, double *__restrict__ dall,
                      int *__restrict__ info, int *status)
 {
     constexpr float kBias = 6.f;
@@ -390,9 +390,9 @@ __global__ void __launch_bounds__(kCholThreads, 1)
 // many lanes it has).
 constexpr int kChol64Threads = 256;
 
-__global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *__restrict__ Gall, int K, float4 *Uall,
-                                                                int *wide, double *__restrict__ dall, int *info,
-                                                                float4 *Uhost, int *info_host)
+__global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *Gall, int K, float4 *Uall, int *wide,
+                                                                double *__restrict__ dall, int *info, float4 *Uhost,
+                                                                int *info_host)
 {
     extern __shared__ double2 A[];   // lower triangle of K x K, packed by rows (tri_row)
     __shared__ double dsh[kCholMaxK];
@@ -637,10 +637,8 @@ __device__ __noinline__ void solve_fp64(const double2 *U, double2 *x, int K, int
 }
 }  // namespace
 
-__global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *__restrict__ Uall, const int *wide,
-                                                         const double *__restrict__ dall,
-                                                         const int *__restrict__ info, int K, SolveIo io,
-                                                         int *status)
+__global__ void __launch_bounds__(256) chol_solve_kernel(const float4 *Uall, const int *wide, const double *dall,
+                                                         const int *info, int K, SolveIo io, int *status)
 {
     extern __shared__ __align__(128) float4 Us[];   // U, lower triangle packed by rows (tri_row), 1 / pivots on the diagonal
     __shared__ float4 w[kCholMaxK];

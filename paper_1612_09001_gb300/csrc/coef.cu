@@ -7,7 +7,7 @@
 
 namespace dpd {
 
-__global__ void wl_table_kernel(const float2 *__restrict__ h, int Bp, int Bq, int T, int B, float *__restrict__ tab,
+__global__ void wl_table_kernel(const float2 *h, int Bp, int Bq, int T, int B, float *__restrict__ tab,
                                 float *__restrict__ adj)
 {
     grid_dep_wait();
@@ -27,7 +27,7 @@ cudaError_t launch_wl_table(const float2 *h, int Bp, int Bq, int T, float *tab, 
 constexpr int kFinalizeWarps = 8;
 
 __global__ void __launch_bounds__(32 * kFinalizeWarps)
-    adj_finalize_kernel(const float2 *__restrict__ partials, int rows, int K, float2 *__restrict__ gh)
+    adj_finalize_kernel(const float2 *partials, int rows, int K, float2 *__restrict__ gh)
 {
     grid_dep_wait();
     const int i = blockIdx.x * kFinalizeWarps + (threadIdx.x >> 5), t = threadIdx.x & 31;

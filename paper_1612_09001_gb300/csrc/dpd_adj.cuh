@@ -132,7 +132,7 @@ static_assert(kAdjGhHalo % 2 == 0 && kHalo % 2 == 0, "slot parts must stay 16-by
 // NS samples from element `off` of a tile whose slot holds the first `cnt` of
 // the `left` samples that the record has from the tile's start (src) on.
 template <int NS>
-__device__ __forceinline__ void adj_slot_window_tail(const float2 *slot, int cnt, const float2 *__restrict__ src,
+__device__ __forceinline__ void adj_slot_window_tail(const float2 *slot, int cnt, const float2 *src,
                                                      int off, int64_t left, float2 (&out)[NS])
 {
 #pragma unroll
@@ -142,7 +142,7 @@ __device__ __forceinline__ void adj_slot_window_tail(const float2 *slot, int cnt
         if (g < cnt)
             v = slot[g];
         else if (g < left)
-            v = __ldg(src + g);
+            v = src[g];
         out[j] = v;
     }
 }
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(32 * kAdjGhWarps, 1)
 // from args[z].
 template <int B, int TG, int V>
 __global__ void __launch_bounds__(32 * kAdjGhWarps, 1)
-    adj_gh_tma_batched_kernel(const AdjArgs *__restrict__ args, int T, int Bp, int Bq, int K)
+    adj_gh_tma_batched_kernel(const AdjArgs *args, int T, int Bp, int Bq, int K)
 {
     grid_dep_wait();   // before args is read: the work list may have just been uploaded
     const AdjArgs a = args[blockIdx.z];

@@ -137,7 +137,7 @@ __host__ __device__ constexpr int tab_bytes()
 // tile is in the slot (the vectorised fast path).
 template <int T, int V>
 __device__ __forceinline__ bool load_window(const float2 *slot, int64_t s0, int S, int64_t n,
-                                            const float2 *__restrict__ x, int t_in_tile,
+                                            const float2 *x, int t_in_tile,
                                             float (&wr)[V + T - 1], float (&wi)[V + T - 1])
 {
     constexpr int W = V + T - 1;
@@ -204,7 +204,7 @@ __device__ __forceinline__ void tile_copy_range(int64_t s0, int S, int64_t n, in
 // code cost the headline kernel two registers and a CTA per SM).  GB300, 16 blocks
 // of 30,720 samples, P = Q = 7, M = 3: 142.9 us; with a second launch per block
 // that recomputed the first M outputs 197.5 (5.6 us of 10 us per block).
-__device__ __forceinline__ void put_history(float2 *slot, const float2 *__restrict__ x, int64_t n, float2 *hist,
+__device__ __forceinline__ void put_history(float2 *slot, const float2 *x, int64_t n, float2 *hist,
                                             int lane)
 {
     static_assert(kHalo <= 32, "one lane per history sample");

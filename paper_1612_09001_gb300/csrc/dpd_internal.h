@@ -203,7 +203,9 @@ inline cudaError_t occupancy(OccCache &c, const void *kern, int threads, size_t 
 
 // Launch `kern` with programmatic stream serialisation: it may begin while the
 // kernel before it in the stream drains, and must call grid_dep_wait() before it
-// touches memory that earlier work wrote or may still read.
+// touches memory that earlier work wrote or may still read.  Such memory is not read
+// through const __restrict__ pointers or __ldg: these promise data that stay the same
+// for the kernel's whole life, which begins before the wait.
 template <class... P, class... A>
 cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A &...args)
 {

@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const GramProblem 
 // transforms.  A moment matrix that is not positive definite gives the monomials (U = I).
 // FP64's latency (64 cycles) bounds it: 13 us; a kernel for the sums, two copies, two
 // synchronisations and the same factorisation on the host took about 45.
-__global__ void __launch_bounds__(32 * kMomK) basis_kernel(const GramProblem *__restrict__ probs, GramProblem one,
-                                                           const double *__restrict__ part, int blocks, int B,
+__global__ void __launch_bounds__(32 * kMomK) basis_kernel(const GramProblem *probs, GramProblem one,
+                                                           const double *part, int blocks, int B,
                                                            float *__restrict__ ubasis, double *__restrict__ ubasis64)
 {
     __shared__ double mu[kMomK], L[kMaxB][kMaxB], rinv[kMaxB];

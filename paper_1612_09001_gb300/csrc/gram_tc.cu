@@ -491,7 +491,7 @@ size_t gram_lag_smem(int fmt)
 
 // ---- finishing: partial lag sums -> S
 // C[p][e] = sum over the problem's CTAs of the partial pairs, in a fixed order (FP32 pairs, then FP64).
-__global__ void __launch_bounds__(256) gram_lag_reduce_kernel(const float2 *__restrict__ partials, int cpp,
+__global__ void __launch_bounds__(256) gram_lag_reduce_kernel(const float2 *partials, int cpp,
                                                               double *__restrict__ C)
 {
     __shared__ double grp[8][32];
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(256) gram_lag_reduce_kernel(const float2 *__re
 
 // The same for the few CTAs of a problem of a batch: one thread per entry.
 constexpr int kLagFew = 8;
-__global__ void __launch_bounds__(256) gram_lag_reduce_few_kernel(const float2 *__restrict__ partials, int cpp,
+__global__ void __launch_bounds__(256) gram_lag_reduce_few_kernel(const float2 *partials, int cpp,
                                                                   double *__restrict__ C)
 {
     grid_dep_wait();
@@ -567,9 +567,8 @@ __device__ __forceinline__ void lag_source(int d, int B, int T, int &sig, int &t
 // last T - 1 samples of every signal evaluated as the tensor kernel evaluates
 // them; they are a few of the N products of an entry, so they are summed in
 // FP32 and only the difference is formed in FP64.
-__global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *__restrict__ Call,
-                                                                const GramProblem *__restrict__ probs,
-                                                                GramProblem one, const float *__restrict__ ubasis,
+__global__ void __launch_bounds__(256) gram_lag_assemble_kernel(const double *Call, const GramProblem *probs,
+                                                                GramProblem one, const float *ubasis,
                                                                 int K, int Bp, int B, int T, int lower,
                                                                 double2 *__restrict__ G, double2 *__restrict__ g,
                                                                 double *__restrict__ tt, double2 *Ghost)

@@ -67,7 +67,7 @@ cudaError_t launch_stream_head(const float *tab, int B, int T, const float2 *x, 
 constexpr int kLossThreads = 512;
 
 __global__ void __launch_bounds__(kLossThreads)
-    sq_error_kernel(const float2 *__restrict__ y, const float2 *__restrict__ x, int64_t n, float2 g, double scale,
+    sq_error_kernel(const float2 *y, const float2 *x, int64_t n, float2 g, double scale,
                     double *__restrict__ part, float2 *__restrict__ gy, float *__restrict__ loss)
 {
     grid_dep_wait();
@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(kLossThreads)
 
 // The loss's gradient on its own, scaled by dL (one device float): gy = dL 2 scale (y - g x).
 __global__ void __launch_bounds__(kLossThreads)
-    sq_error_grad_kernel(const float2 *__restrict__ y, const float2 *__restrict__ x, int64_t n, float2 g, double scale,
-                         const float *__restrict__ dl, float2 *__restrict__ gy)
+    sq_error_grad_kernel(const float2 *y, const float2 *x, int64_t n, float2 g, double scale,
+                         const float *dl, float2 *__restrict__ gy)
 {
     grid_dep_wait();
     const float s2 = (float)(2.0 * scale), l = dl[0];
@@ -187,8 +187,8 @@ __device__ __forceinline__ double inv_newton(double x)   // 1 / x, x > 0
 }
 
 __global__ void __launch_bounds__(256)
-    adam_kernel(float *__restrict__ param, const float *__restrict__ grad, float *__restrict__ m,
-                float *__restrict__ v, float *__restrict__ step, int64_t n, const float *__restrict__ lr, double beta1,
+    adam_kernel(float *__restrict__ param, const float *grad, float *__restrict__ m,
+                float *__restrict__ v, float *__restrict__ step, int64_t n, const float *lr, double beta1,
                 double beta2, double eps)
 {
     grid_dep_wait();
