@@ -402,10 +402,12 @@ __global__ void __launch_bounds__(kChol64Threads) chol64_kernel(const double2 *G
     const int p = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
     // Host copies of the first problem, whichever kernel factored it.
     auto to_host = [&](int status, int fp64) {
-        if (p != 0 || !Uhost) return;
+        if (p != 0) return;
+        if (Uhost) {
 #pragma unroll 8
-        for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = __ldcg(Uall + e);
-        if (tid == 0) {
+            for (int e = tid; e < tri_row(K); e += nt) Uhost[e] = __ldcg(Uall + e);
+        }
+        if (info_host && tid == 0) {
             info_host[0] = status;
             info_host[1] = fp64;
         }

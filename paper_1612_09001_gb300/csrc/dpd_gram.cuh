@@ -121,8 +121,8 @@ int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n);
 // unit lower triangular, Delta diagonal.  U per problem: K (K + 1) / 2 values packed
 // by rows, with 1 / Delta on the diagonal, each an FP32 pair {re.hi, im.hi, re.lo,
 // im.lo} or, with wide[p], two doubles {re, im} in the same 16 bytes; d: K per problem;
-// info[p] = 0 or the failing pivot + 1.  Uhost, info_host: copies of the first problem's
-// factor, and of its status and wide flag, in mapped host memory, or null.
+// info[p] = 0 or the failing pivot + 1.  Uhost, info_host (each may be null): copies of
+// the first problem's factor, and of its status and wide flag, in mapped host memory.
 cudaError_t launch_chol(const double2 *G, int nprob, int K, float4 *U, int *wide, double *d, int *info, float4 *Uhost,
                         int *info_host, int *status, cudaStream_t s);
 // x = G^{-1} rhs using the factorisation (problems that did not factor are skipped).

@@ -840,7 +840,8 @@ dpd_status dpd_estimate(dpd_handle h, const void *u, const void *t, int64_t n, i
     if ((st = run_gram(h, 1, cpp, precision, s, &pr, nullptr, nullptr, false, stats ? w.h_G : nullptr)) != DPD_OK)
         return st;
     if (stats && cudaEventRecord(w.ev_G, s) != cudaSuccess) return DPD_ERR_CUDA;
-    if (dpd::launch_chol(w.G, 1, K, w.U, w.wide, w.d, w.info, w.h_U, w.h_info, h->d_status, s) != cudaSuccess ||
+    if (dpd::launch_chol(w.G, 1, K, w.U, w.wide, w.d, w.info, stats ? w.h_U : nullptr, w.h_info, h->d_status, s) !=
+            cudaSuccess ||
         cudaEventRecord(w.ev_U, s) != cudaSuccess)
         return DPD_ERR_CUDA;
     float2 *out = static_cast<float2 *>(h_out);

@@ -180,3 +180,24 @@ def test_targets_far_from_one(P, Q, M, e):
         err = np.linalg.norm(got.cpu().numpy().astype(np.complex128) - ref) / np.linalg.norm(ref)
         # FP32's smallest step, 2^-149, is a rounding of its own for the coefficients themselves
         assert err <= cond * 2.0 ** -38 + 2.0 ** -23 + 2.0 ** -149 * len(ref) / np.linalg.norm(ref), (err, cond)
+
+
+@pytest.mark.parametrize("nearly_real", [False, True])
+def test_fit_without_statistics(nearly_real):
+    """stats = NULL: the same coefficients (from either factorisation), and a Gram matrix
+    that is not positive definite is still reported."""
+    n = 20000
+    u = _nearly_real(n, 3) if nearly_real else torch.from_numpy(synth.clipped_gaussian(n, 0.3, key=(150, 0))).cuda()
+    f = dpd.DPD(3, 3, 3)
+    f.set_coeffs(synth.coeffs(3, 3, 3, key=(151, 0)))
+    t = f.apply(u)
+    want, _ = f.estimate(u, t, refine_iters=1)
+    h = torch.empty(f.K, dtype=torch.complex64, device="cuda")
+
+    def call(x):
+        return dpd.lib().dpd_estimate(f.handle, x.data_ptr(), t.data_ptr(), n, dpd.PRECISIONS["tf32x3"], 1, h.data_ptr(),
+                                      None, torch.cuda.current_stream().cuda_stream)
+    assert call(u) == 0 and torch.equal(h, want)
+    assert call(torch.zeros_like(u)) == 6
+    assert call(u) == 0 and torch.equal(h, want)
+    f.close()
