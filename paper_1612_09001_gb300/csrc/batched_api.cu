@@ -30,6 +30,9 @@ namespace {
 
 // An item's sub-blocks in BatchItem::tile: first * 4 + (count - 1).
 constexpr int64_t kMaxBlocks = (int64_t)1 << 29;
+// What an item of one sub-block costs besides its samples, in multiply-adds: it ends before
+// the copies of the item after the next have arrived, where a full item covers them.
+constexpr double kShortItem = 250000.0;
 int batch_tile(int64_t block, int nsub) { return (int)(block * 4 + nsub - 1); }
 
 // Whether the launch runs one CTA per SM (its ring takes more than half of the shared memory).
@@ -105,24 +108,30 @@ dpd_status build_items(dpd_plan p, int V, int warps, int nsub, bool contiguous)
             list.push_back({si, batch_tile(b, (int)std::min<int64_t>(nsub, from + count - b))});
     };
     double total = 0.0;
-    // Cost of a sample: 4 B T multiply-adds, and what a sample takes besides them (about
-    // the time of 28: one model at a time over 5.6 M samples, us per launch, 60
-    // multiply-adds 18.6, 100 26.7, 140 32.9).
-    auto cost = [&](int si) { return 4.0 * p->streams[si].B * p->streams[si].T + 28.0; };
+    auto blocks_of = [&](int si) { return (p->streams[si].n + block - 1) / block; };
+    // Cost of a sub-block of a stream, in multiply-adds.  A sample: 4 B T, and what it takes
+    // besides them (about the time of 28: one model at a time over 5.6 M samples, us per
+    // launch, 60 multiply-adds 18.6, 100 26.7, 140 32.9), a part of a sub-block costing as
+    // much as a whole one; and the share in what the stream's last item takes more.
+    auto cost = [&](int si) {
+        const int64_t blocks = blocks_of(si), missing = (nsub - blocks % nsub) % nsub;
+        return (4.0 * p->streams[si].B * p->streams[si].T + 28.0) * block +
+               kShortItem * (double)missing / (double)((nsub > 1 ? nsub - 1 : 1) * blocks);
+    };
     for (int si : order) {
-        if ((p->streams[si].n + block - 1) / block > kMaxBlocks) return DPD_ERR_UNSUPPORTED;
-        total += cost(si) * (double)p->streams[si].n;
+        if (blocks_of(si) > kMaxBlocks) return DPD_ERR_UNSUPPORTED;
+        if (blocks_of(si) > 0) total += cost(si) * (double)blocks_of(si);
     }
     const int G = p->sm_count;
     if (!contiguous || total <= 0.0) {
-        for (int si : order) put(items, si, 0, (p->streams[si].n + block - 1) / block);
+        for (int si : order) put(items, si, 0, blocks_of(si));
     } else {
         std::vector<std::vector<dpd::BatchItem>> run((size_t)G);
         int k = 0;            // the CTA being filled
         double done = 0.0;    // cost given out
         for (int si : order) {
-            const int64_t n = p->streams[si].n, blocks = (n + block - 1) / block;
-            const double c = cost(si) * block;   // of a sub-block
+            const int64_t blocks = blocks_of(si);
+            const double c = blocks > 0 ? cost(si) : 0.0;
             for (int64_t b = 0; b < blocks;) {
                 const double room = total / G * (k + 1) - done;
                 int64_t take = blocks - b;
@@ -133,7 +142,7 @@ dpd_status build_items(dpd_plan p, int V, int warps, int nsub, bool contiguous)
                 }
                 put(run[(size_t)k], si, b, take);
                 b += take;
-                done += b < blocks ? c * (double)take : c * (double)take - cost(si) * (double)(blocks * block - n);
+                done += c * (double)take;
             }
         }
         size_t rounds = 0;
