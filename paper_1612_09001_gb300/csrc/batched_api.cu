@@ -35,10 +35,16 @@ constexpr int64_t kMaxBlocks = (int64_t)1 << 29;
 constexpr double kShortItem = 250000.0;
 int batch_tile(int64_t block, int nsub) { return (int)(block * 4 + nsub - 1); }
 
-// Whether the launch runs one CTA per SM (its ring takes more than half of the shared memory).
-bool one_per_sm(int V, int warps, int group, int stages, int nsub)
+// Whether the work list is cut into one run of equal cost per CTA (build_items): for launches
+// of one CTA per SM (the ring takes more than half of the shared memory) with 6 samples per
+// thread.  With 8 the window loads' bank conflicts and with 4 the loads themselves bound a
+// sample more than its multiply-adds, so runs of equal cost are not of equal time: 64
+// streams of mixed models, us, dealt out in order / in runs: V = 8, 16 warps, 2 stages 160
+// / 198, V = 8, 8 warps, 4 stages 188 / 236, V = 4, 16 warps, 4 stages 155 / 167, V = 6, 16
+// warps in groups of 4, 2 stages 126 / 119, V = 6, 8 warps, 4 stages 161 / 148.
+bool equal_runs(int V, int warps, int group, int stages, int nsub)
 {
-    return dpd::batch_smem(warps, group > 0 ? group : warps, stages, V, nsub) > dpd::kBatchSmemMax / 2;
+    return V == 6 && dpd::batch_smem(warps, group > 0 ? group : warps, stages, V, nsub) > dpd::kBatchSmemMax / 2;
 }
 
 int nbranch(int order) { return order > 0 ? (order + 1) / 2 : 0; }
@@ -81,7 +87,7 @@ void free_plan(dpd_plan p)
 
 // Work list: streams by decreasing per-sample cost (B * T), in items of up to nsub
 // sub-blocks of warps * 32 * V samples.  CTA b of a launch of G takes items b, b + G, ...
-// With a CTA per SM (`contiguous`) those are one run of the ordered list of equal cost
+// With `contiguous` (equal_runs) those are one run of the ordered list of equal cost
 // for each CTA, so a CTA stays with one model's code (the kernel holds one unrolled
 // body per model, and its instruction fetch was an eighth of the stalls) and the SMs
 // with little arithmetic per sample move their bytes while the others compute: 64
@@ -248,7 +254,7 @@ dpd_status dpd_plan_batched(const dpd_stream_desc *descs, int count, int where, 
         return DPD_ERR_CUDA;
     }
     default_shape(p);
-    dpd_status st = build_items(p, p->V, p->warps, p->nsub, one_per_sm(p->V, p->warps, p->group, p->stages, p->nsub));
+    dpd_status st = build_items(p, p->V, p->warps, p->nsub, equal_runs(p->V, p->warps, p->group, p->stages, p->nsub));
     if (st == DPD_OK && cudaDeviceSynchronize() != cudaSuccess) st = DPD_ERR_CUDA;
     if (st != DPD_OK) {
         free_plan(p);
@@ -267,12 +273,12 @@ dpd_status dpd_plan_set_launch(dpd_plan p, int V, int warps, int stages, int cta
     const int gw = group > 0 ? group : warps;
     if (dpd::batch_smem(warps, gw, stages, V) > dpd::kBatchSmemMax) return DPD_ERR_UNSUPPORTED;
     const int nsub = dpd::batch_nsub(warps, gw, stages, V);
-    const bool single = one_per_sm(V, warps, group, stages, nsub);
+    const bool runs = equal_runs(V, warps, group, stages, nsub);
     if (V != p->V || warps != p->warps || nsub != p->nsub ||
-        single != one_per_sm(p->V, p->warps, p->group, p->stages, p->nsub)) {
+        runs != equal_runs(p->V, p->warps, p->group, p->stages, p->nsub)) {
         // Re-tile first: the new shape is kept only once its work list is on
         // the device; on failure the plan runs with its previous shape.
-        const dpd_status st = build_items(p, V, warps, nsub, single);
+        const dpd_status st = build_items(p, V, warps, nsub, runs);
         if (st != DPD_OK) return st;
     }
     p->V = V;

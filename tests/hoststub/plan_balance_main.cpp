@@ -52,6 +52,11 @@ int main()
             }
             double sum = 0.0;
             for (double c : cost) sum += c;
+            size_t in_order = 0;   // items that follow the one before them in the plan's order
+            for (size_t i = 1; i < g_items.size(); ++i)
+                in_order += g_items[i].stream == g_items[i - 1].stream ? g_items[i].tile > g_items[i - 1].tile
+                                                                       : g_items[i].stream >= 0 && g_items[i - 1].stream >= 0;
+            std::printf("dealt out in order: %d\n", in_order == g_items.size() - 1);
             std::printf("mix %lld + %d x %lld shape %d: largest %.3f of the mean, %d items at most\n", (long long)m.longest, m.count,
                         (long long)m.n, s[0], *std::max_element(cost.begin(), cost.end()) / (sum / G),
                         *std::max_element(number.begin(), number.end()));

@@ -37,5 +37,8 @@ def test_short_streams_spread_over_the_ctas(tmp_path):
     r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stdout + r.stderr)
     print(r.stdout)
+    # shape 8 has 8 samples per thread: its items are dealt out in order
+    dealt = re.findall(r"in order: (\d)\nmix .* shape (\d)", r.stdout)
+    assert len(dealt) == 12 and all((d == "1") == (v == "8") for d, v in dealt), r.stdout
     worst = [float(v) for v in re.findall(r"largest ([0-9.]+) of the mean", r.stdout)]
     assert len(worst) == 12 and max(worst) <= 1.5, r.stdout
