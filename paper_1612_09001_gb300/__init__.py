@@ -40,7 +40,8 @@ def kernel_launches() -> int:
 
 # torch's names that every call needs, bound at the first handle or plan (the
 # module itself imports without torch): _cuda_getCurrentRawStream gives the current
-# stream's address without building a torch.cuda.Stream (0.1 against 2.9 us).
+# stream's address without building a torch.cuda.Stream (0.1 against 2.9 us).  Both
+# names are private to torch; without them the public one serves.
 _empty_like = _raw_stream = _current_device = None
 
 
@@ -48,8 +49,12 @@ def _bind_torch():
     global _empty_like, _raw_stream, _current_device
     if _raw_stream is None:
         import torch
-        _empty_like, _current_device = torch.empty_like, torch._C._cuda_getDevice
-        _raw_stream = torch._C._cuda_getCurrentRawStream
+        _empty_like = torch.empty_like
+        _current_device = getattr(torch._C, "_cuda_getDevice", None)
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if _current_device is None or _raw_stream is None:
+            _current_device = torch.cuda.current_device
+            _raw_stream = lambda device: torch.cuda.current_stream(device).cuda_stream
 
 
 def _stream_ptr(stream):

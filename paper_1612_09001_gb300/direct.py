@@ -22,7 +22,6 @@ import math
 import time
 
 import torch
-from torch.optim.optimizer import _global_optimizer_post_hooks, _global_optimizer_pre_hooks
 
 from . import DPD, _lib, _stream_ptr, lib
 from .autograd import DPDFunction
@@ -147,11 +146,13 @@ class DirectLearner:
         g = opt.param_groups[0]
         st = opt.state.get(p)
         tensors = [p, p.grad, g["lr"]] + ([st["step"], st["exp_avg"], st["exp_avg_sq"]] if st else [])
+        hooks = [getattr(o, name, None) for o, name in (
+            (opt, "_optimizer_step_pre_hooks"), (opt, "_optimizer_step_post_hooks"),
+            (torch.optim.optimizer, "_global_optimizer_pre_hooks"), (torch.optim.optimizer, "_global_optimizer_post_hooks"))]
         plain = (st and type(opt) is torch.optim.Adam and "step" not in vars(opt) and len(opt.param_groups) == 1
                  and len(g["params"]) == 1 and g["params"][0] is p
                  and not (g["weight_decay"] or g["amsgrad"] or g["maximize"] or g["differentiable"])
-                 and not (opt._optimizer_step_pre_hooks or opt._optimizer_step_post_hooks
-                          or _global_optimizer_pre_hooks or _global_optimizer_post_hooks)
+                 and all(h is not None and not h for h in hooks)   # private names: unknown counts as hooked
                  and all(isinstance(b, float) for b in (*g["betas"], g["eps"]))
                  and all(isinstance(t, torch.Tensor) and t.device == p.device and t.dtype == torch.float32
                          and t.is_contiguous() for t in tensors))

@@ -3,11 +3,17 @@ batch of problems into the device addresses and lengths that
 dpd_estimate_batched takes.  The tensor checks (complex64, CUDA, contiguous)
 are replaced by a no-op so that CPU tensors stand in for device ones; the
 address arithmetic is the same."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
 
 import paper_1612_09001_gb300 as dpd
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture
@@ -62,3 +68,22 @@ def test_checks_still_run_without_the_stand_in():
         dpd._batch_pointers(list(X), "u")
     with pytest.raises(TypeError):
         dpd._batch_pointers([torch.zeros(4, dtype=torch.float32)], "u")
+
+
+def test_current_stream_without_torchs_private_names(monkeypatch):
+    """A torch without the private accessors: the public current stream serves."""
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    for name in ("_empty_like", "_raw_stream", "_current_device"):
+        monkeypatch.setattr(dpd, name, None)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: type("S", (), {"cuda_stream": 1000 + device}))
+    assert dpd._stream_ptr(None) == 1003
+    assert dpd._stream_ptr(type("S", (), {"cuda_stream": 7})) == 7
+
+
+def test_direct_learning_imports_without_torchs_private_hook_lists():
+    code = ("import torch.optim.optimizer as o; del o._global_optimizer_pre_hooks, o._global_optimizer_post_hooks; "
+            "import paper_1612_09001_gb300.direct")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 0, r.stderr
