@@ -18,6 +18,7 @@ h = argmin ||Psi(s) h - z|| (dpd_estimate), 1-3 times.
 """
 from __future__ import annotations
 
+import importlib
 import math
 import time
 
@@ -25,6 +26,10 @@ import torch
 
 from . import DPD, _lib, _stream_ptr, lib
 from .autograd import DPDFunction
+
+
+# torch.optim drops its submodule's name in some versions.
+_optimizer = importlib.import_module("torch.optim.optimizer")
 
 
 class SqErrorLoss(torch.autograd.Function):
@@ -148,7 +153,7 @@ class DirectLearner:
         tensors = [p, p.grad, g["lr"]] + ([st["step"], st["exp_avg"], st["exp_avg_sq"]] if st else [])
         hooks = [getattr(o, name, None) for o, name in (
             (opt, "_optimizer_step_pre_hooks"), (opt, "_optimizer_step_post_hooks"),
-            (torch.optim.optimizer, "_global_optimizer_pre_hooks"), (torch.optim.optimizer, "_global_optimizer_post_hooks"))]
+            (_optimizer, "_global_optimizer_pre_hooks"), (_optimizer, "_global_optimizer_post_hooks"))]
         plain = (st and type(opt) is torch.optim.Adam and "step" not in vars(opt) and len(opt.param_groups) == 1
                  and len(g["params"]) == 1 and g["params"][0] is p
                  and not (g["weight_decay"] or g["amsgrad"] or g["maximize"] or g["differentiable"])

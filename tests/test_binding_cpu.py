@@ -83,7 +83,20 @@ def test_current_stream_without_torchs_private_names(monkeypatch):
 
 
 def test_direct_learning_imports_without_torchs_private_hook_lists():
-    code = ("import torch.optim.optimizer as o; del o._global_optimizer_pre_hooks, o._global_optimizer_post_hooks; "
-            "import paper_1612_09001_gb300.direct")
+    code = ("import importlib; o = importlib.import_module('torch.optim.optimizer'); "
+            "del o._global_optimizer_pre_hooks, o._global_optimizer_post_hooks; import paper_1612_09001_gb300.direct")
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT)
     assert r.returncode == 0, r.stderr
+
+
+def test_direct_learning_steps_without_the_optimizer_submodules_name(monkeypatch):
+    """Versions of torch whose torch.optim does not keep the name of its submodule: the step
+    still tells a plain optimiser from a hooked one (here: no state yet, torch's own step)."""
+    from paper_1612_09001_gb300.direct import DirectLearner
+    monkeypatch.delattr(torch.optim, "optimizer", raising=False)
+    lr = DirectLearner.__new__(DirectLearner)
+    lr.param = torch.nn.Parameter(torch.ones(3))
+    lr.param.grad = torch.ones(3)
+    lr.opt = torch.optim.Adam([lr.param], lr=0.1)
+    lr._adam_step()
+    assert torch.allclose(lr.param.detach(), torch.full((3,), 0.9), atol=1e-6)
