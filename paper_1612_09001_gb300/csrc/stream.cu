@@ -122,8 +122,14 @@ __global__ void __launch_bounds__(kLossThreads)
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
-    s = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
+    // Four sums a lane: a chain of all its FP64 additions took 0.7 us more.
+    double q4[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < (kLossBlocks + 31) / 32; ++i) {
+        const int b = lane + 32 * i;
+        q4[i & 3] += b < (int)gridDim.x ? __ldcg(part + b) : 0.0;
+    }
+    s = (q4[0] + q4[1]) + (q4[2] + q4[3]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
