@@ -53,7 +53,9 @@ constexpr int kAdjV = 4;          // samples per thread and unit
 constexpr int kAdjUnit = 32 * kAdjV;   // samples of a warp's work unit
 constexpr int kAdjWarps = 8;      // warps per CTA of the staged gx kernel
 constexpr int kAdjStages = 2;     // ring slots per warp of the staged gx kernel
-constexpr int kAdjSub = 1;        // units per slot of the staged gx kernel
+// Units per slot of the staged gx kernel: with one power of r a unit has too little
+// arithmetic to cover its copies.
+constexpr int adj_sub(int B) { return B == 1 ? 4 : 1; }
 constexpr int kAdjGhWarps = 12;   // warps per CTA of the staged gh kernel (about 165 registers per thread)
 constexpr int kAdjGhStages = 2;   // ring slots per warp of the staged gh kernel
 constexpr int kAdjGhSub = 4;      // units per slot of the staged gh kernel
@@ -63,7 +65,8 @@ constexpr int kAdjGhSub = 4;      // units per slot of the staged gh kernel
 // and 41.2 / 6.7; 2, 4 x 1 53.7 / 8.4 and 42.4 / 6.5; 3, 3 x 1 55.0 / 8.4 and 41.5 /
 // 6.6; 4 (64 registers, spills) 64.4 / 10.2 and 47.5 / 8.0.  The FMA pipe bounds the
 // first (28.5 T FMA/s), traffic the second (4.97 TB/s).  With a ring shared by the CTA's
-// warps and a producer warp: 53.8 / 9.3 and 41.2 / 7.4.
+// warps and a producer warp: 53.8 / 9.3 and 41.2 / 7.4.  P = Q = 1, M = 0 at 2^22 / 2^24:
+// 4 units a slot 8.6 / 62.7, 2 8.9 / 63.1, 1 17.5 / 66.8 (that ring 10.3 / 63.1).
 // gh with its final sum, P = Q = 9, M = 4 and P = Q = 7, M = 3: 41.4 / 14.1 and 32.5 /
 // 11.8; with a ring shared by the CTA's warps, whose slots waited for the slowest
 // warp, 46.0 / 18.6 and 35.3 / 14.8.  At 2^20 the 171 tiles on 152 CTAs take two rounds
@@ -426,7 +429,8 @@ __global__ void __launch_bounds__(256) adj_gx_kernel(AdjArgs a)
     }
 }
 
-using GxRing = AdjRing<kAdjStages, kAdjSub, kHalo>;
+template <int B>
+using GxRing = AdjRing<kAdjStages, adj_sub(B), kHalo>;
 
 // Staged variant: CTAs of kAdjWarps independent warps (see AdjRing).  x and gy
 // 16-byte aligned.
@@ -436,16 +440,17 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 3)
 {
     constexpr int W = V + T - 1;
     constexpr int TABF = adj_table_floats(B, T);
-    constexpr int S = GxRing::S;
+    using Ring = GxRing<B>;
+    constexpr int S = Ring::S;
     static_assert(T - 1 <= kHalo && V == kAdjV, "look-ahead must fit the slot");
     static_assert(kAdjWarps * kAdjStages * 8 <= 512, "barrier area");
     extern __shared__ __align__(128) unsigned char smem[];
     float *tab = reinterpret_cast<float *>(smem + 512);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     grid_dep_wait();
-    GxRing ring;
+    Ring ring;
     const int64_t f0 = ring.init(a, units, warp * gridDim.x + blockIdx.x, kAdjWarps * gridDim.x,
-                                 smem + adj_staged_smem<GxRing>(warp, adj_tab_padded<B, T>()),
+                                 smem + adj_staged_smem<Ring>(warp, adj_tab_padded<B, T>()),
                                  smem_addr(smem) + 8u * kAdjStages * warp, lane);
     if constexpr (!PARAM) {
         for (int i = tid; i < TABF; i += 32 * kAdjWarps) tab[i] = a.adj_tab[i];
@@ -793,7 +798,7 @@ template <int B, int T, int V, bool PARAM>
 cudaError_t launch_adj_gx_tma(const AdjArgs &a, const AdjParamTab<B, T> &ptab, int sm_count, cudaStream_t s)
 {
     // The shared-memory table area is kept in both forms (it is small).
-    const size_t smem = adj_staged_smem<GxRing>(kAdjWarps, adj_tab_padded<B, T>());
+    const size_t smem = adj_staged_smem<GxRing<B>>(kAdjWarps, adj_tab_padded<B, T>());
     auto kern = adj_gx_tma_kernel<B, T, V, PARAM>;
     static SmemAttr smem_rec;
     cudaError_t attr = ensure_smem(smem_rec, (const void *)kern, smem);
