@@ -917,7 +917,7 @@ def measure_gram(dev, reps=5):
     us, ts = torch.stack(us), torch.stack(ts)   # equal lengths: one (problems x rows) tensor each
     useful_b = 8.0 * nb * nr * K * K
     batch_refine = 2
-    out["batch_timing"] = (f"one estimate_batched call over all {nb} problems ((basis,) Gram, FP64 Cholesky, solve, "
+    out["batch_timing"] = (f"one estimate_batched call over all {nb} problems ((basis,) Gram, factorisation, solve, "
                            f"{batch_refine} refinements, info copied to the host): median of {reps} calls after 2 "
                            f"warm-up calls; CUDA events around the call and wall time")
     for prec in ("tf32x3", "bf16x3"):

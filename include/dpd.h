@@ -208,8 +208,8 @@ dpd_status dpd_set_adj_launch(dpd_handle h, int gh_blocks, int tap_group);
  * is only 8-byte aligned, or with plain loads selected, the forward filter with
  * zero history and a second launch of one warp that recomputes y[0 .. min(M, n))
  * and saves the history.  Calls on one handle must therefore be ordered on one
- * stream (or synchronised), and x must stay valid until the last launch has run.  Same buffer rules and errors as
- * dpd_apply; n == 0 changes nothing.  Allocation-free and capturable.
+ * stream (or synchronised), and x must stay valid until the last launch has run.
+ * Same buffer rules and errors as dpd_apply; n == 0 changes nothing.  Allocation-free and capturable.
  */
 dpd_status dpd_apply_stream(dpd_handle h, const void *x, void *y, int64_t n, void *stream);
 
@@ -263,20 +263,22 @@ dpd_status dpd_adam_step(float *param, const float *grad, float *m, float *v, fl
  *               warps: every group has its own ring and barriers and runs on
  *               its own sub-tile (group*32*V samples), independently of the
  *               CTA's other groups
- * Default: mode 3, V 8, 16 warps in groups of 4, 4 stages, as many CTAs as
- * fit, TMA.  Every (P, Q, M) has modes 2 and 3 at V 4, 6 and 8 and mode 0 at
- * V 4; other combinations exist only for the benchmarked orders.  Rings that do
- * not fit one CTA's shared memory give DPD_ERR_UNSUPPORTED; a shape that does
- * not fit the device otherwise, or one not built for the handle's (P, Q, M),
- * makes dpd_apply return DPD_ERR_CUDA.
+ * Default: mode 3, TMA, as many CTAs as fit, and V, warps, stages and groups by
+ * the model, the length of the input and where the coefficients came from, until
+ * this function sets a shape.  dpd_apply_host's copy pipeline filters its chunks
+ * with V 8, 16 warps in groups of 4, 4 stages.  Every (P, Q, M) has modes 2 and 3
+ * at V 4, 6 and 8 and mode 0 at V 4; other combinations exist only for the
+ * benchmarked orders.  Rings that do not fit one CTA's shared memory give
+ * DPD_ERR_UNSUPPORTED; a shape that does not fit the device otherwise, or one not
+ * built for the handle's (P, Q, M), makes dpd_apply return DPD_ERR_CUDA.
  */
 dpd_status dpd_set_fwd_launch(dpd_handle h, int mode, int V, int warps, int stages, int ctas_per_sm,
                               int use_tma, int group);
 
 /* ------------------------------------------------------------ least squares */
 
-/* Precision of the Gram contraction Psi^H Psi (accumulation is FP32, the
- * K x K solve FP64 in every mode):
+/* Precision of the Gram contraction Psi^H Psi (accumulation is FP32; the
+ * K x K solve is the same in every mode, see dpd_estimate):
  *   DPD_PREC_FP32    plain FP32 fused multiply-adds on the CUDA cores
  *   DPD_PREC_TF32X3  tensor cores, operands split a = hi + lo in TF32,
  *                    hi*hi + hi*lo + lo*hi (about FP32 accuracy)
@@ -320,8 +322,10 @@ dpd_status dpd_set_estimate_basis(dpd_handle h, int basis);
  * Least-squares coefficients (Sec. 2.2): h = argmin ||Psi(u) h - t||_2, i.e.
  * (Psi^H Psi) h = Psi^H t.  The Gram matrix is formed in `precision`, the
  * system is equilibrated (D = diag(G)^{-1/2}) and solved by a factorisation
- * U Delta U^H in FP32 (hi, lo) pairs (FP64 where a pivot is below 2^-24 or a
- * scale outside FP32's range), then refined `refine_iters` times (0..100) with
+ * U Delta U^H in FP32 (hi, lo) pairs, solutions within about cond 2^-38
+ * relative; where a pivot is below 2^-24 or an entry of D outside FP32's range,
+ * by an FP64 factorisation and FP64 solves (K cond 2^-53).  It is then
+ * refined `refine_iters` times (0..100) with
  * h += G^{-1} Psi^H (t - Psi h), the residual computed by the FP32 filter
  * and adjoint kernels.  In the indirect learning architecture u is the PA
  * output divided by its gain and t the predistorter output.
@@ -329,7 +333,8 @@ dpd_status dpd_set_estimate_basis(dpd_handle h, int basis);
  *           left unchanged; install the result with dpd_set_coeffs)
  *   stats : host double[2] or NULL: [0] 2-norm condition number of D G D
  *           (Lanczos on D G D and on its inverse through the factor, the latter
- *           refined against G; host, FP64, about 1e-11 relative),
+ *           refined against G; host, FP64: about 1e-11 relative up to a condition of
+ *           5e5, then growing with it, 2e-5 at 2e11),
  *           [1] ||t - Psi h||^2 / ||t||^2 of the returned h (FP32 residual and
  *           squares, sums in FP32 pairs, FP64 at the end)
  * Synchronises `stream` once, at the end: the condition estimate runs on the
@@ -398,7 +403,8 @@ dpd_status dpd_exec_batched(dpd_plan plan, void *stream);
  * rebuilds the work list, synchronously, in a new device buffer), stages 2..8,
  * ctas_per_sm >= 0 (0 = as many as fit), group = warps per group dividing
  * `warps` (every group has its own ring of slots and barriers and filters its
- * own part of each work item) or 0 for one group.  Default 8, 8, 4, 0, 0.
+ * own part of each work item) or 0 for one group.  Default 6, 16, 2, 0, 4, and
+ * 4, 4, 3, 0, 0 for batches of fewer than 8,192 samples per SM.
  * Rings larger than one CTA's shared memory give DPD_ERR_UNSUPPORTED.  On any
  * error the plan keeps its previous shape and work list.  A CUDA graph
  * captured from dpd_exec_batched holds the shape and work list of its

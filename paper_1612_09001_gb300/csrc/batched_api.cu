@@ -28,12 +28,10 @@ struct dpd_plan_s {
 
 namespace {
 
-// An item's sub-blocks in BatchItem::tile: first * 4 + (count - 1).
-constexpr int64_t kMaxBlocks = (int64_t)1 << 29;
+constexpr int64_t kMaxBlocks = (int64_t)1 << 29;   // what dpd::batch_tile packs
 // What an item of one sub-block costs besides its samples, in multiply-adds: it ends before
 // the copies of the item after the next have arrived, where a full item covers them.
 constexpr double kShortItem = 250000.0;
-int batch_tile(int64_t block, int nsub) { return (int)(block * 4 + nsub - 1); }
 
 // Whether the work list is cut into one run of equal cost per CTA (build_items): for launches
 // of one CTA per SM (the ring takes more than half of the shared memory) with 6 samples per
@@ -111,7 +109,7 @@ dpd_status build_items(dpd_plan p, int V, int warps, int nsub, bool contiguous)
     std::vector<dpd::BatchItem> items;
     auto put = [&](std::vector<dpd::BatchItem> &list, int si, int64_t from, int64_t count) {
         for (int64_t b = from; b < from + count; b += nsub)
-            list.push_back({si, batch_tile(b, (int)std::min<int64_t>(nsub, from + count - b))});
+            list.push_back({si, dpd::batch_tile(b, (int)std::min<int64_t>(nsub, from + count - b))});
     };
     double total = 0.0;
     auto blocks_of = [&](int si) { return (p->streams[si].n + block - 1) / block; };

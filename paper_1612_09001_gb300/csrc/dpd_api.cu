@@ -321,7 +321,8 @@ dpd_status dpd_set_coeffs(dpd_handle h, const void *coeffs, int K, int where, vo
 //     B T = 48: 29.3 against 41.5; 2^24, B T = 25 63.4 against 72.2), with fewer warps
 //     where there is little arithmetic (2^24, B T = 9: 43.4 against 47.6)
 //   V = 8, 16 warps in groups of 4: long inputs at B T = 20 .. 25 with coefficients in the
-//     parameter bank, whose multiply-adds fill the pipe (2^24, B T = 25: 54.4 against 57.7)
+//     parameter bank, whose multiply-adds fill the pipe (2^24, against V = 6 in groups of 8:
+//     B T = 20 47.8 / 49.0, 21 51.5 / 52.8, 24 55.8 / 57.0, 25 55.4 / 57.7)
 static dpd::FwdLaunch launch_for(dpd_handle h, int64_t n, bool param_tab)
 {
     dpd::FwdLaunch L = h->fwd;

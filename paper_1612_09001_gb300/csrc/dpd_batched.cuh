@@ -30,7 +30,7 @@ struct BatchStream {
 };
 
 // Work item: sub-blocks [tile / 4, tile / 4 + tile % 4 + 1) of a stream, a sub-block
-// being one run of V samples per consumer thread of the CTA (batch_item packs the
+// being one run of V samples per consumer thread of the CTA (batch_tile packs the
 // pair).  An item of -1, -1 ends the list of the CTA that takes it.
 struct BatchItem {
     int stream;
@@ -82,7 +82,8 @@ __device__ __forceinline__ bool item_ok(const BatchArgs &a, const BatchItem &w, 
     return w.stream >= 0 && w.stream < a.nstreams && st.tab_off >= 0 && st.tab_bytes > 0 &&
            st.tab_bytes <= kBatchTabBytes && (st.tab_bytes & 15) == 0 && (st.tab_off & 3) == 0 &&
            (int64_t)st.tab_off + st.tab_bytes / 4 <= a.tab_floats && w.tile >= 0 &&
-           w.tile % kBatchMaxSub < a.nsub && (int64_t)(w.tile / kBatchMaxSub) * block < st.n && ((reinterpret_cast<uintptr_t>(st.x) & 15u) == 0);
+           w.tile % kBatchMaxSub < a.nsub && (int64_t)(w.tile / kBatchMaxSub) * block < st.n &&
+           ((reinterpret_cast<uintptr_t>(st.x) & 15u) == 0);
 }
 
 template <int B, int T, int V>

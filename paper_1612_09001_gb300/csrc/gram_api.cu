@@ -282,7 +282,10 @@ dpd_status refine_batched(dpd_handle h, const std::vector<dpd::GramProblem> &pro
     const int S = nsub * warps * 32 * V;
     // CTAs of a problem and tap group in the coefficient gradient, one per SM: the rounds
     // that the launch takes, each a share of the samples and a CTA's start and end, about
-    // kCtaSamples samples' time.
+    // kCtaSamples samples' time.  A batched fit with two refinements, us, with 1, 2, 3, 4, 8
+    // rows: 256 x 2^16 at K = 97 1611 1602 1607 1624 1694; 64 x 2^18 at K = 33 1101 993 1048
+    // 999 1015; 16 x 2^20 at K = 51 2113 1529 1319 1232 1079.  The choice here is within 2 %
+    // of the best of 1 .. 11 on these and four more.
     const int groups = (h->T + h->adj.tap_group - 1) / h->adj.tap_group;
     int rows = 1;
     int64_t best = INT64_MAX;

@@ -845,7 +845,9 @@ int gram_ctas_per_problem(int precision, int sm_count, int nprob, int64_t n)
     // kernel: one CTA per SM, so a launch takes as many rounds as its CTAs fill the SMs,
     // each round a share of the stages and the start and end of a CTA, about kCtaStages
     // stages' time.  256 problems of 2^16 samples (TF32: 256 stages) on 152 SMs, us:
-    // 1 CTA each (2 rounds) 617, 4 (7 rounds) 568, 7 (12 rounds) 590.
+    // 1 CTA each (2 rounds) 617, 4 (7 rounds) 568, 7 (12 rounds) 590.  The same for BF16's
+    // longer stages: a batched fit without refinement, us, 64 x 2^18 at K = 33 with 1, 2, 4,
+    // 8, 9 CTAs 813 472 482 486 450 and 444 with the 7 chosen; 16 x 2^20 at K = 51 466 with 9.
     const int rows = precision == kPrecFP32   ? kF32Rows
                      : precision == kPrecBF16x3 ? LagGeom<kFmtBF16>::R
                                                 : LagGeom<kFmtTF32>::R;   // samples per stage
